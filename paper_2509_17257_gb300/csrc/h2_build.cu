@@ -519,8 +519,8 @@ int build_device(h2_matrix* A, const double* pts_host, uint32_t precisions, cuda
     A->up_ptr[L + 1] = (int64_t)up_list.size();
     A->down_ptr[L + 1] = (int64_t)down_list.size();
     if (k <= 64) {
-        // gather, forward transformation (one launch), coupling, downward pass (one launch), leaf phase
-        A->launches_per_product = A->down_ptr[L + 1] > 0 ? 5 : 4;
+        // gather, leaf forward, upward pass (one launch), coupling, downward pass (one launch), leaf phase
+        A->launches_per_product = A->down_ptr[L + 1] > 0 ? 6 : 4;
     } else {
         A->launches_per_product = 4;  // gather, leaf forward, coupling, leaf backward, + one launch per level
         for (int l = 0; l <= L; ++l) {
@@ -593,6 +593,25 @@ int build_device(h2_matrix* A, const double* pts_host, uint32_t precisions, cuda
             nearT_blk[p] = (int32_t)j;
         }
     }
+    // list owners by falling work: admissible blocks of a cluster, nearfield entries of a leaf
+    auto by_work = [](const std::vector<int64_t>& work) {
+        std::vector<int32_t> o(work.size());
+        for (size_t i = 0; i < o.size(); ++i) o[i] = (int32_t)i;
+        std::stable_sort(o.begin(), o.end(), [&](int32_t a, int32_t b) { return work[a] > work[b]; });
+        return o;
+    };
+    std::vector<int64_t> work_r(nc), work_c(nc), work_lr(NL, 0), work_lc(NL, 0);
+    for (int64_t c = 0; c < nc; ++c) {
+        work_r[c] = adm_rowptr[c + 1] - adm_rowptr[c];
+        work_c[c] = admT_rowptr[c + 1] - admT_rowptr[c];
+    }
+    for (int64_t j = 0; j < A->n_near; ++j) {
+        const int64_t e = T.size[near_row[j]] * T.size[near_col[j]];
+        work_lr[leaf_pos[near_row[j]]] += e;
+        work_lc[leaf_pos[near_col[j]]] += e;
+    }
+    const std::vector<int32_t> adm_order = by_work(work_r), admT_order = by_work(work_c);
+    const std::vector<int32_t> near_order = by_work(work_lr), nearT_order = by_work(work_lc);
     std::vector<double> pts_p((size_t)n * 3);
     for (int64_t i = 0; i < n; ++i)
         for (int d = 0; d < 3; ++d) pts_p[3 * i + d] = pts_host[3 * T.perm[i] + d];
@@ -633,6 +652,10 @@ int build_device(h2_matrix* A, const double* pts_host, uint32_t precisions, cuda
     UP(A->d_nearT_ptr, nearT_ptr);
     UP(A->d_nearT_row, nearT_row);
     UP(A->d_nearT_blk, nearT_blk);
+    UP(A->d_adm_order, adm_order);
+    UP(A->d_admT_order, admT_order);
+    UP(A->d_near_order, near_order);
+    UP(A->d_nearT_order, nearT_order);
     UP(A->d_pts, pts_p);
     double* d_box = nullptr;
     UP(d_box, T.box);

@@ -380,6 +380,9 @@ struct h2_matrix {
     int32_t* d_nearT_ptr = nullptr;  // [n_leaves+1] by column leaf position
     int32_t* d_nearT_row = nullptr;  // [n_near] row cluster t
     int32_t* d_nearT_blk = nullptr;  // [n_near] block index j
+    // clusters (leaf positions) by falling work of their lists: the order the FP64 kernels issue their CTAs in
+    int32_t *d_adm_order = nullptr, *d_admT_order = nullptr;    // [nc]
+    int32_t *d_near_order = nullptr, *d_nearT_order = nullptr;  // [n_leaves]
     double* d_pts = nullptr;         // [n][3] points in cluster order
     double* d_nodes = nullptr;       // [nc][3][q] Chebyshev nodes per cluster
 
@@ -559,6 +562,17 @@ int flow_capture(h2_batch* b, const std::vector<int>& sys, const TcGemmParams& p
 size_t product_scratch_bytes(const h2_matrix* A, int64_t m, int32_t dtype);
 int matmul_in_scratch(h2_matrix* A, double alpha, const double* X, int64_t ldx, double* Y, int64_t ldy,
                       int64_t m, int32_t dtype, cudaStream_t st, void* scratch);
+
+// The FP64 phases (h2_mm64.cu): k <= 64 for the two transfer passes, kron the
+// factors of E for q = 4 or null; m columns, row stride m, except Y's.
+int launch_up64(h2_matrix* A, const double* V, const double* E, const double* kron, const double* Xp, double* xhat,
+                int m, const SyncBufs& sb, cudaStream_t st);
+int launch_down64(h2_matrix* A, const double* E, const double* kron, double* yhat, int m, const SyncBufs& sb,
+                  cudaStream_t st);
+int launch_coupling64(h2_matrix* A, const double* S, const double* xhat, double* yhat, int m, bool trans,
+                      cudaStream_t st);
+int launch_leaf64(h2_matrix* A, const double* V, const double* G, const double* yhat, const double* Xp, double* Y,
+                  int64_t ldy, double alpha, int m, bool trans, bool overwrite, cudaStream_t st);
 
 // tcgen05 BF16 kernels (h2_tc.cu)
 int tc_smem_bytes();

@@ -1,5 +1,6 @@
-// H² matrix × dense block, SIMT kernels for FP64 and FP32 (Sec. 3 Alg.
-// "H2_mvm" with the k×m coefficient blocks of Sec. 4).
+// H² matrix × dense block, the product's chains and their SIMT kernels (Sec. 3
+// Alg. "H2_mvm" with the k×m coefficient blocks of Sec. 4); the FP64 phases are
+// in h2_mm64.cu, the tensor-core phases in h2_tc.cu.
 //
 // The product Y += α·A·X runs as a stream-ordered chain:
 //   gather      Xp = X[perm]                       (cluster order, compute type)
@@ -15,6 +16,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "h2_async.cuh"
@@ -1418,10 +1420,15 @@ int forward_pass(h2_matrix* A, const T* V, const T* E, const T* Xp, T* xhat, int
     const int k = A->k;
     const unsigned NL = (unsigned)A->leaves.size();
     if (gzk == 1) {
-        k_up_fused<T, RM, CN><<<dim3(NL, gy), kThreads, 0, st>>>(A->d_leaves, A->d_cl_off, A->d_cl_size,
-                                                                A->d_parent, A->d_son0, A->d_son1, V, E, Xp, xhat,
-                                                                sb.cnt, k, m, kron);
-        H2_LAUNCH_CHECK();
+        if constexpr (std::is_same_v<T, double>) {
+            const int rc = launch_up64(A, V, E, kron, Xp, xhat, m, sb, st);
+            if (rc) return rc;
+        } else {
+            k_up_fused<T, RM, CN><<<dim3(NL, gy), kThreads, 0, st>>>(A->d_leaves, A->d_cl_off, A->d_cl_size,
+                                                                    A->d_parent, A->d_son0, A->d_son1, V, E, Xp, xhat,
+                                                                    sb.cnt, k, m, kron);
+            H2_LAUNCH_CHECK();
+        }
         marks.mark();
         marks.mark();
         return 0;
@@ -1449,6 +1456,7 @@ int backward_pass(h2_matrix* A, const T* E, T* yhat, int m, unsigned gy, unsigne
     const int n_items = (int)A->down_ptr[A->depth + 1];
     if (n_items == 0) return 0;
     if (gzk == 1) {
+        if constexpr (std::is_same_v<T, double>) return launch_down64(A, E, kron, yhat, m, sb, st);
         // ready flags and claim tickets start at zero for every product (graph-replay safe)
         H2_CUDA_TRY(cudaMemsetAsync(sb.flag, 0, (size_t)A->nc * gy * sizeof(int), st));
         H2_CUDA_TRY(cudaMemsetAsync(sb.claim, 0, gy * sizeof(unsigned), st));
@@ -1507,6 +1515,8 @@ int run_chain(h2_matrix* A, const MatData& D, double alpha, const double* X, int
             set_error("complex product: column tiles must hold whole complex columns");
             return H2_E_UNSUPPORTED;
         }
+    } else if constexpr (std::is_same_v<T, double>) {
+        if ((rc = launch_coupling64(A, S, xhat, yhat, m, transposed, st))) return rc;
     } else if (transposed)
         k_coupling<T, RM, CN, true><<<dim3((unsigned)A->nc, gy, gzk), kThreads, 0, st>>>(
             A->d_admT_rowptr, A->d_admT_row, A->d_admT_blk, S, xhat, yhat, k, m);
@@ -1528,6 +1538,8 @@ int run_chain(h2_matrix* A, const MatData& D, double alpha, const double* X, int
             set_error("complex product: column tiles must hold whole complex columns");
             return H2_E_UNSUPPORTED;
         }
+    } else if constexpr (std::is_same_v<T, double>) {
+        if ((rc = launch_leaf64(A, V, G, yhat, Xp, Y, ldy, alpha, m, transposed, overwrite, st))) return rc;
     } else if (transposed)
         k_leaf_bwd_near<T, RM, CN, true><<<dim3(NL, gy, gzl), kThreads, 0, st>>>(
             A->d_leaves, A->d_cl_off, A->d_cl_size, A->d_perm, V, yhat, A->d_nearT_ptr, A->d_nearT_row,
@@ -2130,11 +2142,10 @@ int forward_transform_f64(h2_matrix* A, const double* X, int64_t ldx, int64_t m,
     H2_LAUNCH_CHECK();
     PhaseMarks none(nullptr, st);
     const double* V = (const double*)A->f64.V;
+    const double* kron = (A->k == 64 && A->use_kron) ? (const double*)A->f64.kron : nullptr;
     const double* E = (const double*)A->f64.E;
     const unsigned gzk = (unsigned)((A->k + 63) / 64);
-    if (m <= 16) return forward_pass<double, 4, 1>(A, V, E, Xp, xhat, (int)m, (unsigned)((m + 15) / 16), gzk, st, sb, none);
-    if (m <= 32) return forward_pass<double, 4, 2>(A, V, E, Xp, xhat, (int)m, (unsigned)((m + 31) / 32), gzk, st, sb, none);
-    return forward_pass<double, 4, 4>(A, V, E, Xp, xhat, (int)m, (unsigned)((m + 63) / 64), gzk, st, sb, none);
+    return forward_pass<double, 4, 4>(A, V, E, Xp, xhat, (int)m, (unsigned)((m + 63) / 64), gzk, st, sb, none, kron);
 }
 
 size_t product_scratch_bytes(const h2_matrix* A, int64_t m, int32_t dtype) {

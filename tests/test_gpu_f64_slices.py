@@ -1,0 +1,42 @@
+"""The FP64 phases (h2_mm64.cu) at the edges of their cuts: output pairs (odd k and odd leaf
+sizes), chunks of 128 pairs, column tiles of 32, slices of 1, 2 and 4 columns, 64-column tiles."""
+import numpy as np
+import pytest
+
+from _helpers import rel_fro, require_cuda
+from oracle import h2_oracle as O
+from workloads import ellipsoid_points, gaussian_rhs
+
+pytestmark = pytest.mark.gpu
+
+# a sum of p products of FP64 numbers rounds to p·2^-53 of its absolute terms; p is at most
+# the points of the near lists and k per level, below 2000 here, and the terms do not cancel
+# by more than the oracle's own rounding shows
+TOL = 2000 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("q,leaf", [(1, 24), (2, 7), (3, 64), (4, 33), (5, 64)])
+@pytest.mark.parametrize("m", [1, 2, 3, 16, 17, 32, 33, 64, 65, 130])
+def test_f64_product_at_the_cuts(q, leaf, m):
+    torch = require_cuda()
+    import paper_2509_17257_gb300 as P
+
+    n = 1501
+    pts = ellipsoid_points(n, (0.6, 1.1, 1.9), 3)
+    H = O.H2Matrix(pts, q=q, leaf_size=leaf, eta=2.0, sigma=1e-2)
+    A = P.H2Matrix(pts, q=q, leaf_size=leaf, eta=2.0, sigma=1e-2, precisions=())
+    X, Y0 = gaussian_rhs(n, m, 5), gaussian_rhs(n, m, 6)
+    want = O.h2mm(H, 0.5, X, Y0)
+    for ld in (m, m + 3):
+        Xd = torch.zeros(n, ld, dtype=torch.float64, device="cuda")[:, :m]
+        Yd = torch.zeros(n, ld, dtype=torch.float64, device="cuda")[:, :m]
+        for product in (A.matmul, A.matmul_transposed):  # the kernel is symmetric
+            Xd.copy_(torch.from_numpy(X))
+            Yd.copy_(torch.from_numpy(Y0))
+            product(Xd, Yd, alpha=0.5, dtype="f64")
+            first = Yd.cpu().numpy()
+            assert rel_fro(first, want) <= TOL
+            Yd.copy_(torch.from_numpy(Y0))
+            product(Xd, Yd, alpha=0.5, dtype="f64")
+            assert np.array_equal(first, Yd.cpu().numpy())
+    A.close()
