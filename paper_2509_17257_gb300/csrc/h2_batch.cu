@@ -154,8 +154,8 @@ int flow_capture(h2_batch* b, const std::vector<int>& sys, const TcGemmParams& p
         if ((e = cudaEventRecord(b->join[i], b->streams[i])) != cudaSuccess) break;
         e = cudaStreamWaitEvent(b->origin, b->join[i], 0);
     }
-    if (!rc && e == cudaSuccess) rc = launch_tc_gemm(3, 1, p1, std::min(p1.n_items, kTcGrid), b->origin);
-    if (!rc && e == cudaSuccess) rc = launch_tc_gemm(3, 1, p2, std::min(p2.n_items, kTcGrid), b->origin);
+    if (!rc && e == cudaSuccess) rc = launch_tc_gemm(3, 1, p1, b->origin);
+    if (!rc && e == cudaSuccess) rc = launch_tc_gemm(3, 1, p2, b->origin);
     if (!rc && e == cudaSuccess) e = cudaEventRecord(b->fork, b->origin);
     for (int j = 0; j < ns && !rc && e == cudaSuccess; ++j) {
         const int i = sys[j];

@@ -151,10 +151,9 @@ struct TcGemmParams {
     // mode 3 with several systems: per-system arguments (items carry their system in
     // bits 18.. of np); the launch-wide R is the largest system's
     const TcSys* sys;
-    // matrix-free coupling (mode 2): Chebyshev nodes [cluster][KP] (x, y, z, 0) and
-    // the kernel's 1/length; S_b[ν, μ] = exp(-|ξ_{t,ν} - ξ_{s,μ}| / length) for ν, μ < k
+    // matrix-free coupling (mode 2): Chebyshev nodes [cluster][KP] (x, y, z, 0), scaled
+    // by log2(e) / length: S_b[ν, μ] = 2^(-|node_{t,ν} - node_{s,μ}|) for ν, μ < k
     const float4* nodes;
-    float inv_len;
     int KP;
     // modes 0 and 1 of the complex product: terms marked kTermImag apply i·act
     int cplx;
@@ -166,7 +165,7 @@ struct TcData {
     int KP = 0, NP = 0;
     uint8_t* mat = nullptr;    // BF16 core-matrix tiles: S (list order), V (leaf order), G (near order)
     uint8_t* mat32 = nullptr;  // the same tiles in FP32 (offsets ×2), for the 3xTF32 product
-    float4* nodes4 = nullptr;  // [n_clusters][KP] Chebyshev tensor nodes (x, y, z, 0), zero past k (matrix-free coupling)
+    float4* nodes4 = nullptr;  // [n_clusters][KP] Chebyshev tensor nodes (x, y, z, 0) × log2(e) / length, zero past k (matrix-free coupling)
     int64_t bytes = 0;
     bool has_bf16 = false, has_tf32 = false;
     // coupling: outputs are clusters with at least one admissible block
@@ -581,7 +580,7 @@ int tc_prepare();
 // transfer-pass bookkeeping, kernel attributes), so that the product itself
 // allocates nothing (e.g. while it is captured into a CUDA graph).
 int product_prepare(h2_matrix* A, int64_t m, int32_t dtype, cudaStream_t st);
-int launch_tc_gemm(int mode, int kind, TcGemmParams p, int grid, cudaStream_t st, int stages = 0);
+int launch_tc_gemm(int mode, int kind, TcGemmParams p, cudaStream_t st, int stages = 0);
 // Rebuild the subtree schedules of the CUDA-core transfer passes for other cut targets.
 int set_transfer_targets(h2_matrix* A, int up_target, int down_target, cudaStream_t st);
 // Work list of the coupling launch with the clusters above the upward cut (TcData::h_*).

@@ -1595,7 +1595,6 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
     const float* V = (const float*)A->f32.V;
     const float* E = (const float*)A->f32.E;
 
-    const int grid_cap = kTcGrid;
     SyncBufs sbc = sb;
     for (int c0 = 0; c0 < m; c0 += 64) {
         const int mc = std::min(64, m - c0);
@@ -1707,18 +1706,18 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
                 f2.items = D.f2_items;
                 f2.terms = D.f2_terms;
                 marks.kernel_begin();
-                if ((rc = launch_tc_gemm(3, 1, f1, std::min(f1.n_items, grid_cap), st, stg))) return rc;
+                if ((rc = launch_tc_gemm(3, 1, f1, st, stg))) return rc;
                 marks.kernel_end();
                 marks.mark();
                 marks.mark();
                 marks.mark();
-                if ((rc = launch_tc_gemm(3, 1, f2, std::min(f2.n_items, grid_cap), st, stg))) return rc;
+                if ((rc = launch_tc_gemm(3, 1, f2, st, stg))) return rc;
                 marks.mark();
             } else {
                 f1.n_items = D.up_nitems;
                 f1.items = D.up_items;
                 f1.terms = D.up_terms;
-                if ((rc = launch_tc_gemm(3, 1, f1, std::min(f1.n_items, grid_cap), st, stg))) return rc;
+                if ((rc = launch_tc_gemm(3, 1, f1, st, stg))) return rc;
                 marks.mark();
                 marks.mark();
                 TcGemmParams cp{};
@@ -1735,18 +1734,17 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
                 cp.ldc = mc;
                 cp.err = A->err_dev;
                 cp.nodes = D.nodes4;
-                cp.inv_len = (float)(1.0 / A->length);
                 cp.KP = KP;
                 cp.out_act = ycp;  // split tiles for the downward pass's identity terms
                 marks.kernel_begin();
-                if (cp.n_items > 0 && (rc = launch_tc_gemm(mf ? 2 : 0, 1, cp, std::min(cp.n_items, grid_cap), st, stg)))
+                if (cp.n_items > 0 && (rc = launch_tc_gemm(mf ? 2 : 0, 1, cp, st, stg)))
                     return rc;
                 marks.kernel_end();
                 marks.mark();
                 f2.n_items = D.dn_nitems;
                 f2.items = D.dn_items;
                 f2.terms = D.dn_terms;
-                if ((rc = launch_tc_gemm(3, 1, f2, std::min(f2.n_items, grid_cap), st, stg))) return rc;
+                if ((rc = launch_tc_gemm(3, 1, f2, st, stg))) return rc;
                 marks.mark();
                 TcGemmParams lp{};
                 lp.n_items = trans ? D.lt_nitems : D.l_nitems;
@@ -1763,7 +1761,7 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
                 lp.err = A->err_dev;
                 lp.zp = Xp;
                 lp.ldc = mc;
-                if ((rc = launch_tc_gemm(1, 1, lp, std::min(lp.n_items, grid_cap), st, stg))) return rc;
+                if ((rc = launch_tc_gemm(1, 1, lp, st, stg))) return rc;
             }
             const int64_t total = n * mc;
             const unsigned g = (unsigned)std::min<int64_t>((total + 255) / 256, 152 * 32);
@@ -1820,7 +1818,6 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
         cp.ldc = mc;
         cp.err = A->err_dev;
         cp.nodes = D.nodes4;
-        cp.inv_len = (float)(1.0 / A->length);
         cp.KP = KP;
         cp.cplx = cx ? 1 : 0;
         if (hybrid) {
@@ -1834,7 +1831,7 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
         }
         marks.kernel_begin();
         if (cp.n_items > 0 &&
-            (rc = launch_tc_gemm(hybrid ? 4 : (mf ? 2 : 0), kind, cp, std::min(cp.n_items, grid_cap), st, stg)))
+            (rc = launch_tc_gemm(hybrid ? 4 : (mf ? 2 : 0), kind, cp, st, stg)))
             return rc;
         marks.kernel_end();
         marks.mark();
@@ -1888,7 +1885,7 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
         lp.zp = Xp;  // the gathered FP32 X is no longer read after the forward pass and its packing
         lp.ldc = mc;
         lp.cplx = cx ? 1 : 0;
-        if ((rc = launch_tc_gemm(1, kind, lp, std::min(lp.n_items, grid_cap), st, stg))) return rc;
+        if ((rc = launch_tc_gemm(1, kind, lp, st, stg))) return rc;
         {
             const int64_t total = n * mc;
             const unsigned g = (unsigned)std::min<int64_t>((total + 255) / 256, 152 * 32);
@@ -2142,8 +2139,8 @@ int forward_transform_f64(h2_matrix* A, const double* X, int64_t ldx, int64_t m,
     H2_LAUNCH_CHECK();
     PhaseMarks none(nullptr, st);
     const double* V = (const double*)A->f64.V;
-    const double* kron = (A->k == 64 && A->use_kron) ? (const double*)A->f64.kron : nullptr;
     const double* E = (const double*)A->f64.E;
+    const double* kron = (A->k == 64 && A->use_kron) ? (const double*)A->f64.kron : nullptr;
     const unsigned gzk = (unsigned)((A->k + 63) / 64);
     return forward_pass<double, 4, 4>(A, V, E, Xp, xhat, (int)m, (unsigned)((m + 63) / 64), gzk, st, sb, none, kron);
 }

@@ -26,7 +26,8 @@
 // tcgen05 MMA takes time in proportion to N and the same time for M = 64 as for
 // M = 128, so B_lo rides along in M at no cost.
 //
-// Kernel roles (one persistent CTA per SM; 7 warps for KIND 0, 11 for KIND 1):
+// Kernel roles (one persistent CTA per SM, or two with at most 32 columns; 7 warps
+// for KIND 0, 11 for KIND 1):
 //   warp 0          bulk-copy producer (cp.async.bulk + mbarrier complete_tx)
 //   warp 1          TMEM owner and MMA issuer (tcgen05.mma kind::f16 or
 //                   kind::tf32, FP32 accumulate): KIND 0 all terms, KIND 1 the
@@ -54,10 +55,12 @@ namespace h2 {
 
 namespace {
 
-constexpr int kMaxStages = 16;
+constexpr int kMaxStages = 16, kMaxStagesNarrow = 6;
 constexpr int kSmemBudget = 225 * 1024;  // dynamic shared memory per CTA (one CTA per SM)
+// NARROW instances (R <= 64 activation rows): two CTAs per SM.  Of an SM's 228 KiB
+// each CTA's 1 KiB reserve and about 0.7 KiB of static shared memory come off.
+constexpr int kSmemBudgetNarrow = 228 * 1024 / 2 - 1024 - 768;
 constexpr int kSplitWarps = 4;  // KIND 1: warps 6..9 write [B; B_lo] into TMEM, one lane quadrant each
-constexpr int kASlots = 4;      // KIND 1: TMEM slots of the MMA's A operand (64 columns each, after the accumulators)
 // warps: 0 producer, 1 and kIssuer2 MMA issuers (even and odd terms), 2..5
 // epilogue, KIND 1: 6..9 splitter
 template <int KIND>
@@ -66,7 +69,12 @@ template <int KIND>
 __host__ __device__ constexpr int tc_threads() { return 32 * (tc_issuer2<KIND>() + 1); }
 constexpr int kAccCols = 64;                // output columns of one term (the matrix tile's rows)
 constexpr int kAccBufs = 4;                 // accumulator buffers: MMAs of a term overlap the epilogue of the 3 before
-constexpr int kXchBytes = 2 * 64 * 64 * 4;  // TF32 epilogue: remainder sums handed over, two items deep
+// TF32 epilogue: remainder sums handed over, two items deep (64 rows of 64 columns, NARROW 32)
+constexpr int xch_bytes(bool narrow) { return 2 * 64 * (narrow ? 32 : 64) * 4; }
+constexpr int kNodeBytes = 64 * 16;        // MODE 2: the source cluster's nodes, in the stage after its activation tile
+// MODE 2: evaluated tiles, two terms deep, rows of 68 floats (16-byte accesses of
+// eight consecutive rows touch all 32 banks once)
+constexpr int kEvalLd = 68, kEvalBytes = 2 * 64 * kEvalLd * 4;
 
 // Shared-memory matrix descriptor, no swizzle, K-major: LBO = byte distance of
 // core matrices adjacent along K, SBO = byte distance of adjacent 8-row groups.
@@ -172,20 +180,16 @@ __device__ __forceinline__ void tmem_ld32_async(uint32_t taddr, uint32_t (&r)[32
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// 64 consecutive TMEM columns of this warp's 32 lanes from registers; the
+// 32 consecutive TMEM columns of this warp's 32 lanes from registers; the
 // caller waits with tmem_wait_st before signalling the MMA.
-__device__ __forceinline__ void tmem_st64(uint32_t taddr, const uint32_t (&v)[64]) {
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&v)[32]) {
     asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x64.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"
-        "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,"
-        "%43,%44,%45,%46,%47,%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,%59,%60,%61,%62,%63,%64};" ::"r"(taddr),
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"
+        "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(taddr),
         "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
         "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(v[16]), "r"(v[17]), "r"(v[18]),
         "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]),
-        "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31]), "r"(v[32]), "r"(v[33]), "r"(v[34]), "r"(v[35]), "r"(v[36]),
-        "r"(v[37]), "r"(v[38]), "r"(v[39]), "r"(v[40]), "r"(v[41]), "r"(v[42]), "r"(v[43]), "r"(v[44]), "r"(v[45]),
-        "r"(v[46]), "r"(v[47]), "r"(v[48]), "r"(v[49]), "r"(v[50]), "r"(v[51]), "r"(v[52]), "r"(v[53]), "r"(v[54]),
-        "r"(v[55]), "r"(v[56]), "r"(v[57]), "r"(v[58]), "r"(v[59]), "r"(v[60]), "r"(v[61]), "r"(v[62]), "r"(v[63])
+        "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
         : "memory");
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
@@ -296,8 +300,16 @@ __global__ void k_pack_act(const float* __restrict__ src, int64_t ld, int ids, c
 // one system, whose role-0 items write rows of ŷ like MODE 0: the coupling
 // launch that also computes the clusters above the upward pass's cut (their
 // transfer items wait for their sons and release their own tiles).
-template <int MODE, int KIND>
-__global__ void __launch_bounds__(tc_threads<KIND>(), 1) k_tc_gemm(const TcGemmParams p) {
+// NARROW (R <= 64, at most 32 right-hand-side columns): two CTAs per SM, each with
+// half of the SM's stages, accumulators and A slots.  A CTA's hand-offs (about
+// 1300 cycles a term, of which copies and MMAs fill a part) are a serial chain, so
+// two CTAs run two of them at once; 80 registers a thread (KIND 1) suffice because
+// the epilogue sums 32 columns and moves TMEM 32 columns at a time.  One CTA → two
+// (µs, n = 65536, q = 4, m = 32): hybrid coupling 167 → 140, leaf 86 → 73; BF16 130
+// → 91 and 67 → 42; n = 262144, m = 16: 593 → 457 and 294 → 235.  More than 32
+// columns need stages of 48 KiB and 128 accumulator columns: one CTA.
+template <int MODE, int KIND, bool NARROW>
+__global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(const TcGemmParams p) {
     constexpr bool MF = MODE == 2;
     constexpr bool FLOW = MODE == 3;
     constexpr bool LIST = MODE == 3 || MODE == 4;  // items carry roles, terms may wait for ready flags
@@ -309,28 +321,36 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), 1) k_tc_gemm(const TcGemmP
     constexpr int F_FIRST = 1, F_LAST = 2, F_END = 4;
     // TMEM: KIND 0 has kAccBufs accumulators of 64 columns.  KIND 1 has
     // accumulators of R columns (64 or 128: 4 or 2 of them, 256 columns) and
-    // after them kASlots slots of 64 columns for the MMA's A operand [B; B_lo].
-    constexpr int TMEM_COLS = KIND == 1 ? 512 : kAccBufs * kAccCols;
-    constexpr int A_BASE = 256;
-    extern __shared__ __align__(1024) uint8_t smem_raw[];
-    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ __align__(8) uint64_t full_bar[kMaxStages], split_bar[kMaxStages], empty_bar[kMaxStages];
+    // after them kASlots (4) slots of 64 columns for the MMA's A operand [B; B_lo].
+    // NARROW halves both (KIND 1): accumulators of 32 or 64 columns in 128, two A slots.
+    constexpr int TMEM_COLS = KIND == 1 ? (NARROW ? 256 : 512) : kAccBufs * kAccCols;
+    constexpr int A_BASE = NARROW ? 128 : 256;
+    constexpr int kASlots = NARROW ? 2 : 4;
+    constexpr int kSums = KIND == 1 && NARROW ? 32 : kAccCols;  // right-hand-side columns (KIND 1), tile rows (KIND 0)
+    constexpr int kSt = NARROW ? kMaxStagesNarrow : kMaxStages;
+    extern __shared__ __align__(128) uint8_t smem_raw[];
+    // 128 bytes: a core matrix, which is what bulk copies and descriptors without a swizzle need
+    // (an offset, not a rounded pointer: through an integer the compiler loses the address
+    // space, and every access to the stages becomes a generic load)
+    uint8_t* smem = smem_raw + (-smem_u32(smem_raw) & 127u);
+    __shared__ __align__(8) uint64_t full_bar[kSt], split_bar[kSt], empty_bar[kSt];
     __shared__ __align__(8) uint64_t accf_bar[kAccBufs], acce_bar[kAccBufs], drain_bar[2], aempty_bar[kASlots];
     __shared__ int s_total;  // terms of this CTA
     __shared__ uint32_t tmem_slot;
-    __shared__ int stage_kp[kMaxStages], stage_np[kMaxStages], stage_fl[kMaxStages], stage_R[kMaxStages];
-    __shared__ int stage_t[kMaxStages], stage_s[kMaxStages];  // MODE 2: target and source cluster
+    __shared__ int stage_kp[kSt], stage_np[kSt], stage_fl[kSt], stage_R[kSt];
+    __shared__ int stage_t[MF ? kSt : 1];  // MODE 2: target cluster
     __shared__ int abort_shared;
     volatile int& abort_flag = abort_shared;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int R = p.R;
     const int M = R <= 64 ? 64 : 128;
     const int nst = p.nstages;
-    const int a_bytes = p.a_stage_bytes, b_bytes = 64 * 64 * ES;
+    const int a_bytes = p.a_stage_bytes, b_bytes = MF ? kNodeBytes : 64 * 64 * ES;
     const int stage_bytes = a_bytes + b_bytes;
     const int G = gridDim.x;
-    const int acc_cols = KIND == 1 ? (R <= 64 ? 64 : 128) : kAccCols;  // TMEM columns of one accumulator
-    const int nacc = KIND == 1 ? 256 / acc_cols : kAccBufs;             // accumulator buffers
+    // TMEM columns of one accumulator, and accumulator buffers
+    const int acc_cols = KIND == 1 ? (NARROW ? (R <= 32 ? 32 : 64) : (R <= 64 ? 64 : 128)) : kAccCols;
+    const int nacc = KIND == 1 ? A_BASE / acc_cols : kAccBufs;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < nst; ++s) {
@@ -446,11 +466,12 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), 1) k_tc_gemm(const TcGemmP
                             stage_R[stage] = Ri;
                             stage_fl[stage] = (base + j == 0 ? F_FIRST : 0) | (base + j == nterms - 1 ? F_LAST : 0);
                             if (MF) {
-                                // the source cluster: the activation rows of cluster s start at s·KP
+                                // the source cluster's nodes: cluster s's rows and nodes start at s·KP
+                                const uint32_t nb = (uint32_t)(p.KP * 16);
                                 stage_t[stage] = cur.id;
-                                stage_s[stage] = (int)(aj / ((int64_t)R * ES) / p.KP);
-                                mbar_expect_tx(&full_bar[stage], ab);
+                                mbar_expect_tx(&full_bar[stage], ab + nb);
                                 bulk_g2s(sA, (asj ? p.act1 : p.act0) + aj, ab, &full_bar[stage]);
+                                bulk_g2s(sB, p.nodes + akj, nb, &full_bar[stage]);
                             } else {
                                 mbar_expect_tx(&full_bar[stage], ab + bb);
                                 const uint8_t* asrc = (asj & 3) == 0 ? PSYS(cur, act0)
@@ -625,7 +646,8 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), 1) k_tc_gemm(const TcGemmP
         const int q = warp & 3;
         const int n = 32 * (q & 1) + lane;
         const bool lo_part = q >= 2;
-        float* xch = reinterpret_cast<float*>(smem + nst * stage_bytes);  // [2][64 i][64 n]
+        // [2][kSums i][64 n]
+        float* xch = reinterpret_cast<float*>(smem + nst * stage_bytes + (MF ? kEvalBytes : 0));
         int it = 0, par = 0;
         // rows of Z: the leaf phase, and the leaf items of a transfer-pass launch
         auto leaf_rows = [&](const TcItem& t) { return MODE == 1 || (LIST && item_role(t) == kRoleLeaf); };
@@ -650,14 +672,14 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), 1) k_tc_gemm(const TcGemmP
             const int id = cur.id, np = item_np(cur), nterms = cur.e1 - cur.e0;
             const int Ri = SYSF(cur, R), mci = SYSF(cur, mc), ki = SYSF(cur, k), KPi = SYSF(cur, KP),
                       ldci = SYSF(cur, ldc);
-            const bool wide = Ri > 64;
+            const bool wide = !NARROW && Ri > 64;
             const bool vec4 = (mci & 3) == 0 && (ldci & 3) == 0;
             const int role = LIST ? item_role(cur) : 0;
             // role 0 (MODE 4's coupling items): rows of ŷ, as in MODE 0
             const bool split_out = COUP_SPLIT || (LIST && role != kRoleLeaf && role != 0);
-            float sum[kAccCols];
+            float sum[kSums];
 #pragma unroll
-            for (int j = 0; j < kAccCols; ++j) sum[j] = 0.f;
+            for (int j = 0; j < kSums; ++j) sum[j] = 0.f;
             bool failed = false;
             uint32_t imask = 0;  // complex product: bit t of the batch of 32 terms applies i·act
             for (int term = 0; term < nterms; ++term, ++it) {
@@ -673,18 +695,28 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), 1) k_tc_gemm(const TcGemmP
                 }
                 tc_fence_after();
                 const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * acc_cols);
-                if constexpr (FLOW) {
+                if constexpr (FLOW || NARROW) {
                     // 32 columns per read (16 right-hand-side columns; R > 64 takes four):
-                    // one register buffer, which the multi-system bookkeeping needs room for
+                    // one register buffer, which the multi-system bookkeeping and the two
+                    // CTAs per SM need room for
                     uint32_t r0[32];
 #pragma unroll
-                    for (int h = 0; h < 4; ++h) {
-                        if (h >= 2 && !wide) break;
+                    for (int h = 0; h < kSums / 16; ++h) {
+                        if (NARROW ? 32 * h >= acc_cols : (h >= 2 && !wide)) break;
                         tmem_ld32_async(ta + 32 * h, r0);
                         tmem_wait_ld();
+                        if (FLOW || !imag) {
 #pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            sum[16 * h + j] += __uint_as_float(r0[2 * j]) + __uint_as_float(r0[2 * j + 1]);
+                            for (int j = 0; j < 16; ++j)
+                                sum[16 * h + j] += __uint_as_float(r0[2 * j]) + __uint_as_float(r0[2 * j + 1]);
+                        } else {
+                            // i·act: column 2j takes -(column 2j + 1), column 2j + 1 takes column 2j
+#pragma unroll
+                            for (int j = 0; j < 16; j += 2) {
+                                sum[16 * h + j] -= __uint_as_float(r0[2 * j + 2]) + __uint_as_float(r0[2 * j + 3]);
+                                sum[16 * h + j + 1] += __uint_as_float(r0[2 * j]) + __uint_as_float(r0[2 * j + 1]);
+                            }
+                        }
                     }
                 } else {
                     // 64 columns per read (two loads in flight, one wait); R > 64 takes two
@@ -721,10 +753,10 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), 1) k_tc_gemm(const TcGemmP
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&acce_bar[acc]);
             }
-            float* xb = xch + par * (64 * 64);
+            float* xb = xch + par * (64 * kSums);
             if (lo_part && !failed) {
 #pragma unroll
-                for (int i = 0; i < kAccCols; ++i)
+                for (int i = 0; i < kSums; ++i)
                     if (i < mci) xb[i * 64 + n] = sum[i];
             }
             // every epilogue warp reaches this barrier once per item, failed or not,
@@ -736,26 +768,27 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), 1) k_tc_gemm(const TcGemmP
             }
             if (!lo_part && split_out) {
 #pragma unroll
-                for (int i = 0; i < kAccCols; ++i)
+                for (int i = 0; i < kSums; ++i)
                     if (i < mci) sum[i] += xb[i * 64 + n];
                 // The result goes, split as the activations are (rows 2i: x; 2i + 1: x -
                 // tf32(x); zero past the columns and past column k), into the cluster's
                 // tile: staged in this item's exchange buffer (free once both tile warps
-                // have read it) and stored by one bulk copy per 64 rows.
+                // have read it) and stored by one bulk copy per SB rows.
+                constexpr int SB = kSums;  // rows of KP <= 64 columns that the exchange buffer holds
                 asm volatile("bar.sync 4, 64;" ::: "memory");
                 uint8_t* gtile = (role == kRoleCoupling ? SYSF(cur, out_act2) : SYSF(cur, out_act)) + (int64_t)id * KPi * Ri * 4;
                 const bool nv = n < ki;
 #pragma unroll
-                for (int hh = 0; hh < 2; ++hh) {
-                    const int h0 = 64 * hh;
+                for (int hh = 0; hh < 2 * kSums / SB; ++hh) {
+                    const int h0 = SB * hh;
                     if (h0 >= Ri) break;
-                    const int rows = min(64, Ri - h0);
+                    const int rows = min(SB, Ri - h0);
                     if (h0 > 0) asm volatile("bar.sync 4, 64;" ::: "memory");  // the last store read the buffer
                     if (n < KPi) {
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) {
+                        for (int i = 0; i < SB / 2; ++i) {
                             if (2 * i >= rows) break;
-                            const int ii = 32 * hh + i;
+                            const int ii = SB / 2 * hh + i;
                             const float v = (nv && ii < mci) ? sum[ii] : 0.f;
                             const float lo = v - __uint_as_float(__float_as_uint(v) & 0xFFFFE000u);
                             *(float*)((uint8_t*)xb + cm_off(2 * i, n, KPi, 4)) = v;
@@ -781,7 +814,7 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), 1) k_tc_gemm(const TcGemmP
                 }
             } else if (!lo_part) {
 #pragma unroll
-                for (int i = 0; i < kAccCols; ++i)
+                for (int i = 0; i < kSums; ++i)
                     if (i < mci) sum[i] += xb[i * 64 + n];
                 float* out = nullptr;
                 if (!leaf_rows(cur)) {
@@ -794,12 +827,12 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), 1) k_tc_gemm(const TcGemmP
                 if (out) {
                     if (vec4) {
 #pragma unroll
-                        for (int i = 0; i < kAccCols; i += 4)
+                        for (int i = 0; i < kSums; i += 4)
                             if (i < mci)
                                 *reinterpret_cast<float4*>(out + i) = make_float4(sum[i], sum[i + 1], sum[i + 2], sum[i + 3]);
                     } else {
 #pragma unroll
-                        for (int i = 0; i < kAccCols; ++i)
+                        for (int i = 0; i < kSums; ++i)
                             if (i < mci) out[i] = sum[i];
                     }
                 }
@@ -954,6 +987,8 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), 1) k_tc_gemm(const TcGemmP
         int stage = 0, sit = 0;
         uint32_t phase = 0;
         bool pre = false;  // the next iteration's stage and A-slot phases were seen complete
+        float4 xt = make_float4(0.f, 0.f, 0.f, 0.f);  // MODE 2: this row's target node, of cluster xt_of
+        int xt_of = -1;
         while (true) {
             bool ok = pre || __any_sync(0xffffffffu, mbar_wait(&full_bar[stage], phase));
             const int fl = ok ? stage_fl[stage] : 0;
@@ -964,36 +999,47 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), 1) k_tc_gemm(const TcGemmP
             pre = false;
             if (ok && !end) tc_fence_after();
             const int kp = ok ? stage_kp[stage] : 0;
-            float* xbuf = (float*)(smem + stage * stage_bytes + a_bytes);  // MODE 2: [64 μ][64 rows]
+            // MODE 2: row n of the evaluated tile, two terms deep (a warp is past the
+            // barrier of term t + 1 only when its partner has read term t's tile)
+            float* xrow = (float*)(smem + nst * stage_bytes + (sit & 1) * (kEvalBytes / 2)) + n * kEvalLd;
             if (MF) {
                 // row n of S_b: g(ξ_{t,n}, ξ_{s,μ}) = exp(-|ξ_{t,n} - ξ_{s,μ}| / length) for
                 // n, μ < k, zero in the padding.  The tile warp (q < 2) and the remainder
                 // warp (q + 2) of the same rows each evaluate half of the columns and
-                // swap halves through the stage's (unused) matrix region.  The exponential
-                // is 2^(-r·log2(e)/length) with r = d²·rsqrt(d²) (hardware approximations,
-                // relative error below 1e-6).
+                // swap halves through shared memory.  The source nodes come with the stage
+                // and are read by the whole warp at once (one broadcast per node); the
+                // row's own node stays in a register over the item.  The nodes are scaled,
+                // so a value is a hardware square root and a hardware 2^x (relative error
+                // below 1e-6): 8 instructions and 16 cycles of the SFU per warp.  n = 65536,
+                // q = 4, m = 32: 786 µs with node loads from global memory, shuffles and one
+                // CTA per SM, 670 with the nodes in the stage, 402 with two CTAs, about 190
+                // with scaled nodes, a square root and 16-byte exchanges.
                 if (ok && !end) {
                     const bool rv = n < p.k;
-                    const float4 xt = p.nodes[(int64_t)stage_t[stage] * p.KP + (rv ? n : 0)];
-                    const int mu0 = lo_part ? 32 : 0;
-                    // the warp's 32 source nodes: one coalesced load (lane l holds node
-                    // mu0 + l), handed to every lane by shuffles
-                    const float4 ys = mu0 + lane < p.KP ? p.nodes[(int64_t)stage_s[stage] * p.KP + mu0 + lane]
-                                                        : make_float4(0.f, 0.f, 0.f, 0.f);
-                    const float sc = -p.inv_len * 1.4426950408889634f;
-#pragma unroll 8
-                    for (int j = 0; j < 32; ++j) {
-                        const int mu = mu0 + j;
-                        const float y0 = __shfl_sync(0xffffffffu, ys.x, j), y1 = __shfl_sync(0xffffffffu, ys.y, j),
-                                    y2 = __shfl_sync(0xffffffffu, ys.z, j);
-                        float g = 0.f;
-                        if (rv && mu < p.k) {
-                            const float d0 = xt.x - y0, d1 = xt.y - y1, d2 = xt.z - y2;
+                    if (stage_t[stage] != xt_of) {
+                        xt_of = stage_t[stage];
+                        xt = p.nodes[(int64_t)xt_of * p.KP + (rv ? n : 0)];
+                    }
+                    const int half = p.KP >> 1, mu0 = lo_part ? half : 0;
+                    const float4* ys = (const float4*)(smem + stage * stage_bytes + a_bytes);
+                    for (int j0 = mu0; j0 < mu0 + half; j0 += 8) {
+                        float g[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            const float4 y = ys[j0 + j];
+                            const float d0 = xt.x - y.x, d1 = xt.y - y.y, d2 = xt.z - y.z;
                             const float r2 = fmaf(d2, d2, fmaf(d1, d1, d0 * d0));
-                            const float e = r2 * rsqrtf(r2) * sc;
-                            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(g) : "f"(e));
+                            float r;
+                            asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(r2));
+                            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(g[j]) : "f"(-r));
                         }
-                        xbuf[mu * 64 + n] = g;
+                        if (p.k < p.KP) {
+#pragma unroll
+                            for (int j = 0; j < 8; ++j)
+                                if (!rv || j0 + j >= p.k) g[j] = 0.f;
+                        }
+                        *(float4*)(xrow + j0) = make_float4(g[0], g[1], g[2], g[3]);
+                        *(float4*)(xrow + j0 + 4) = make_float4(g[4], g[5], g[6], g[7]);
                     }
                 }
                 // the pair (quadrants q and q ^ 2, named barrier 2 or 3) meets once per
@@ -1013,29 +1059,26 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), 1) k_tc_gemm(const TcGemmP
                 const uint32_t nphase = stage + 1 == nst ? phase ^ 1u : phase;
                 const bool pf = mbar_test(&full_bar[nstage], nphase);
                 const bool pa = mbar_test(&aempty_bar[(sit + 1) % kASlots], (((sit + 1) / kASlots) & 1) ^ 1);
-                uint32_t v[64];
-                if (MF) {
+                const uint8_t* row =
+                    smem + stage * stage_bytes + a_bytes + (n >> 3) * (kp >> 2) * 128 + (n & 7) * 16;
+                const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(A_BASE + 64 * as);
 #pragma unroll
-                    for (int mu = 0; mu < 64; ++mu) {
-                        float g = mu < kp ? xbuf[mu * 64 + n] : 0.f;
-                        if (lo_part) g -= __uint_as_float(__float_as_uint(g) & 0xFFFFE000u);
-                        v[mu] = __float_as_uint(g);
-                    }
-                } else {
-                    const uint8_t* row =
-                        smem + stage * stage_bytes + a_bytes + (n >> 3) * (kp >> 2) * 128 + (n & 7) * 16;
+                for (int h = 0; h < 2; ++h) {
+                    if (32 * h >= kp) break;
+                    uint32_t v[32];
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) {
+                    for (int c = 0; c < 8; ++c) {
                         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (4 * c < kp) x = *(const float4*)(row + c * 128);
+                        if (32 * h + 4 * c < kp)
+                            x = *(const float4*)(MF ? (const uint8_t*)(xrow + 32 * h + 4 * c) : row + (8 * h + c) * 128);
                         if (lo_part) x = tf32_lo(x);
                         v[4 * c] = __float_as_uint(x.x);
                         v[4 * c + 1] = __float_as_uint(x.y);
                         v[4 * c + 2] = __float_as_uint(x.z);
                         v[4 * c + 3] = __float_as_uint(x.w);
                     }
+                    tmem_st32(ta + 32 * h, v);
                 }
-                tmem_st64(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(A_BASE + 64 * as), v);
                 tmem_wait_st();
                 tc_fence_before();
                 ++sit;
@@ -1071,21 +1114,71 @@ __global__ void k_zero_tiles(const int32_t* __restrict__ ids, int count, uint8_t
     }
 }
 
-// Stage geometry for R activation rows and element size es: A holds R rows,
-// B 64 rows, both with up to 64 contraction columns.  The TF32 kernel keeps
-// its epilogue exchange tile (kXchBytes) after the stages (its B_lo lives in
-// TMEM).
-void tc_stage_geometry(int R, int es, int* a_bytes, int* stage_bytes, int* nstages) {
-    const int rows = R <= 64 ? 64 : 128;  // the BF16 MMA reads M = 64 or 128 activation rows
-    *a_bytes = rows * 64 * es;
-    *stage_bytes = *a_bytes + 64 * 64 * es;
-    *nstages = std::min(kMaxStages, (kSmemBudget - 1024 - (es == 4 ? kXchBytes : 0)) / *stage_bytes);
+// Stage geometry for R activation rows and element size es: A holds R rows (the
+// BF16 MMA reads M = 64 or 128 of them), B 64 rows, both with up to 64
+// contraction columns; MODE 2 has the source nodes in place of B.  After the
+// stages come MODE 2's evaluated tiles and the TF32 kernel's epilogue exchange
+// (its B_lo lives in TMEM).  NARROW instances split an SM's shared memory between
+// two CTAs.
+struct TcGeometry {
+    int a_bytes, stage_bytes, nstages, after;
+};
+TcGeometry tc_geometry(int R, int mode, int kind, bool narrow) {
+    TcGeometry g;
+    const int es = kind == 0 ? 2 : 4;
+    const int rows = kind == 1 && narrow ? R : (R <= 64 ? 64 : 128);
+    g.a_bytes = rows * 64 * es;
+    g.stage_bytes = g.a_bytes + (mode == 2 ? kNodeBytes : 64 * 64 * es);
+    g.after = (mode == 2 ? kEvalBytes : 0) + (kind == 1 ? xch_bytes(narrow) : 0);
+    const int budget = (narrow ? kSmemBudgetNarrow : kSmemBudget) - 128 - g.after;
+    g.nstages = std::min(narrow ? kMaxStagesNarrow : kMaxStages, budget / g.stage_bytes);
+    return g;
+}
+
+// CTAs of a NARROW instance that are resident on one SM with `smem` bytes of
+// dynamic shared memory: two if shared memory, registers (four partitions of the
+// register file, a warp's in units of 256) and TMEM (256 of 512 columns each)
+// allow it.  The runtime's occupancy query answers one for every kernel with a
+// tcgen05.alloc; on the device two start at once (304 CTAs of 352 threads, 256
+// columns and 114816 bytes on 152 SMs: none started late).
+struct NarrowFit {
+    int regs = 0, static_smem = 0, sm_smem = 0, reserved = 0;
+    int per_sm(int threads, int smem) const {
+        const int warps = threads / 32, per_warp = (regs * 32 + 255) / 256 * 256;
+        const bool fits = 2 * (smem + static_smem + reserved) <= sm_smem && (2 * warps + 3) / 4 * per_warp <= 65536 / 4;
+        return fits ? 2 : 1;
+    }
+};
+template <int MODE, int KIND>
+NarrowFit& narrow_fit() {
+    static NarrowFit f;
+    return f;
 }
 
 template <int MODE, int KIND>
-int launch_one(const TcGemmParams& p, int grid, int smem, cudaStream_t st) {
-    k_tc_gemm<MODE, KIND><<<grid, tc_threads<KIND>(), smem, st>>>(p);
+int launch_one(const TcGemmParams& p, bool narrow, int smem, cudaStream_t st) {
+    // Every CTA has to be resident: those of modes 3 and 4 wait on each other's
+    // ready flags (bounded).
+    const int per_sm = narrow ? narrow_fit<MODE, KIND>().per_sm(tc_threads<KIND>(), smem) : 1;
+    const int grid = std::min(p.n_items, per_sm * kTcGrid);
+    if (narrow) k_tc_gemm<MODE, KIND, true><<<grid, tc_threads<KIND>(), smem, st>>>(p);
+    else k_tc_gemm<MODE, KIND, false><<<grid, tc_threads<KIND>(), smem, st>>>(p);
     H2_LAUNCH_CHECK();
+    return 0;
+}
+template <int MODE, int KIND>
+int prepare_one(int dev) {
+    H2_CUDA_TRY(cudaFuncSetAttribute(k_tc_gemm<MODE, KIND, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
+    H2_CUDA_TRY(cudaFuncSetAttribute(k_tc_gemm<MODE, KIND, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudgetNarrow));
+    H2_CUDA_TRY(cudaFuncSetAttribute(k_tc_gemm<MODE, KIND, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+    cudaFuncAttributes at;
+    H2_CUDA_TRY(cudaFuncGetAttributes(&at, k_tc_gemm<MODE, KIND, true>));
+    NarrowFit f;
+    f.regs = at.numRegs;
+    f.static_smem = (int)at.sharedSizeBytes;
+    H2_CUDA_TRY(cudaDeviceGetAttribute(&f.sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
+    H2_CUDA_TRY(cudaDeviceGetAttribute(&f.reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev));
+    narrow_fit<MODE, KIND>() = f;
     return 0;
 }
 
@@ -1099,49 +1192,43 @@ int tc_prepare() {
     int dev = 0;
     H2_CUDA_TRY(cudaGetDevice(&dev));
     if (dev == g_tc_attr_device) return 0;
-    H2_CUDA_TRY(cudaFuncSetAttribute(k_tc_gemm<0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
-    H2_CUDA_TRY(cudaFuncSetAttribute(k_tc_gemm<1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
-    H2_CUDA_TRY(cudaFuncSetAttribute(k_tc_gemm<0, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
-    H2_CUDA_TRY(cudaFuncSetAttribute(k_tc_gemm<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
-    H2_CUDA_TRY(cudaFuncSetAttribute(k_tc_gemm<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
-    H2_CUDA_TRY(cudaFuncSetAttribute(k_tc_gemm<3, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
-    H2_CUDA_TRY(cudaFuncSetAttribute(k_tc_gemm<4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
-    H2_CUDA_TRY(cudaFuncSetAttribute(k_tc_gemm<4, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
+    int rc = 0;
+    if ((rc = prepare_one<0, 0>(dev)) || (rc = prepare_one<1, 0>(dev)) || (rc = prepare_one<4, 0>(dev)) ||
+        (rc = prepare_one<0, 1>(dev)) || (rc = prepare_one<1, 1>(dev)) || (rc = prepare_one<2, 1>(dev)) ||
+        (rc = prepare_one<3, 1>(dev)) || (rc = prepare_one<4, 1>(dev)))
+        return rc;
     g_tc_attr_device = dev;
     return 0;
 }
 
-int launch_tc_gemm(int mode, int kind, TcGemmParams p, int grid, cudaStream_t st, int stages) {
-    int a_bytes, stage_bytes, nstages;
-    tc_stage_geometry(p.R, kind == 0 ? 2 : 4, &a_bytes, &stage_bytes, &nstages);
+int launch_tc_gemm(int mode, int kind, TcGemmParams p, cudaStream_t st, int stages) {
+    const bool narrow = p.R <= 64;
+    TcGeometry g = tc_geometry(p.R, mode, kind, narrow);
     // a tuned stage count (h2_autotune) below the number that fits
-    if (stages >= 2 && stages < nstages) nstages = stages;
+    if (stages >= 2 && stages < g.nstages) g.nstages = stages;
     // A parity wait is exact only while its waiter cannot get two uses of a stage
     // ahead (the protocol model in tests/test_pipeline_protocol.py checks this).
     // The FP32 issuers wait on the in-order splitter, which keeps them in step;
     // the BF16 kernel has one issuer, which waits on every stage in order.
-    if (nstages < 2) { set_error("tensor-core stage does not fit in shared memory"); return H2_E_UNSUPPORTED; }
-    p.a_stage_bytes = a_bytes;
-    p.nstages = nstages;
+    if (g.nstages < 2) { set_error("tensor-core stage does not fit in shared memory"); return H2_E_UNSUPPORTED; }
+    p.a_stage_bytes = g.a_bytes;
+    p.nstages = g.nstages;
     int rc = tc_prepare();
     if (rc) return rc;
-    const int smem = nstages * stage_bytes + (kind == 1 ? kXchBytes : 0) + 1024;
-    if (mode == 2) {
-        if (kind != 1) { set_error("matrix-free coupling runs on the TF32 path only"); return H2_E_UNSUPPORTED; }
-        return launch_one<2, 1>(p, grid, smem, st);
+    const int smem = g.nstages * g.stage_bytes + g.after + 128;
+    if (kind == 0) {
+        if (mode == 0) return launch_one<0, 0>(p, narrow, smem, st);
+        if (mode == 1) return launch_one<1, 0>(p, narrow, smem, st);
+        if (mode == 4) return launch_one<4, 0>(p, narrow, smem, st);
+        set_error(mode == 2 ? "matrix-free coupling runs on the TF32 path only"
+                            : "the tensor-core transfer passes run on the TF32 path only");
+        return H2_E_UNSUPPORTED;
     }
-    if (mode == 3) {
-        if (kind != 1) { set_error("the tensor-core transfer passes run on the TF32 path only"); return H2_E_UNSUPPORTED; }
-        // its CTAs wait on each other's ready flags: one CTA per SM, at most one per SM
-        // of the device, so that every CTA is resident (the waits are bounded in any case)
-        return launch_one<3, 1>(p, grid, smem, st);
-    }
-    // waits on flags too: one CTA per SM, every CTA resident
-    if (mode == 4) return kind == 1 ? launch_one<4, 1>(p, grid, smem, st) : launch_one<4, 0>(p, grid, smem, st);
-    if (mode == 0 && kind == 0) return launch_one<0, 0>(p, grid, smem, st);
-    if (mode == 1 && kind == 0) return launch_one<1, 0>(p, grid, smem, st);
-    if (mode == 0 && kind == 1) return launch_one<0, 1>(p, grid, smem, st);
-    return launch_one<1, 1>(p, grid, smem, st);
+    if (mode == 2) return launch_one<2, 1>(p, narrow, smem, st);
+    if (mode == 3) return launch_one<3, 1>(p, narrow, smem, st);
+    if (mode == 4) return launch_one<4, 1>(p, narrow, smem, st);
+    if (mode == 0) return launch_one<0, 1>(p, narrow, smem, st);
+    return launch_one<1, 1>(p, narrow, smem, st);
 }
 
 int launch_pack_tiles(const TcPackTile* tiles, int64_t count, const double* src, uint8_t* dst, int es,
