@@ -117,12 +117,11 @@ typedef struct h2_info_t {
     double flops_per_col; /* algorithmic flops of one product per column of X */
     int32_t launches;     /* kernel launches of one product on the CUDA cores (FP64)     */
     int32_t launches_tc;  /* kernel launches of one tensor-core product (FP32, BF16) of at
-                             most 64 columns, a multiple of 4 of them; with k % 4 == 0 and
-                             k <= 64 the transfer passes pack the tensor-core operands
-                             themselves, otherwise three packing launches are counted  */
+                             most 64 columns: with q = 2, 3, 4 the transfer passes are lists
+                             of pairs, otherwise three packing launches are counted        */
     int32_t kernel;       /* h2_kernel of the build                                     */
     int32_t hybrid;       /* 1: the FP32 and BF16 tensor-core products take, by default,
-                             the hybrid upward pass (the CUDA-core subtree pass stops at its
+                             the hybrid upward pass (the lists of pairs stop at the first
                              cut, the clusters above it are transfer items of the coupling
                              launch)                                                      */
     int64_t n_above_cut;  /* clusters above that cut (transfer items of that launch)      */
@@ -134,7 +133,7 @@ typedef struct h2_info_t {
  *     H2_FORCE_SIMT=1        FP32 products on the CUDA cores only
  *     H2_TC_TRANSFER=0|1     FP32 transfer passes on the CUDA cores / the tensor cores
  *     H2_TC_HYBRID=0|1       the hybrid upward pass off / on
- *     H2_KRON=0              q = 4 transfer passes on the dense transfer matrices
+ *     H2_KRON=0              transfer passes on the dense transfer matrices
  *     H2_HYBRID_ROUND_TERMS  coupling terms per CTA between two heights of the hybrid
  *                            pass's transfer items (1..64, default 16)
  *   read by h2_batch_create for that batch:
@@ -400,13 +399,12 @@ int h2_batch_block_cg(h2_batch* batch, const double* const* B, const int64_t* ld
  *      "forward/backward" as work lists in dependency order: one launch per
  *      phase, path 2, or sharing the coupling's and the leaf phase's launches,
  *      path 3; FP32 only), CUDA cores only (path 4; FP32 only), and tensor
- *      cores with the CUDA-core subtree passes stopping at the upward cut,
+ *      cores with the CUDA-core transfer passes stopping at the upward cut,
  *      whose clusters above the cut become transfer items of the coupling
  *      launch (path 5; FP32 and BF16);
  *   2. on the best path, the pipeline stage count of the tensor-core kernels
  *      (4 and 5 against as many as fit);
- *   3. on paths 1 and 5, the cut targets of the CUDA-core subtree passes (the task
- *      counts that the upward and the downward schedules aim at: half and
+ *   3. on paths 1 and 5, the cut targets of the CUDA-core transfer passes (half and
  *      twice the default, upward first).
  * The fastest variant is kept for later products of this precision whose
  * column chunks fall in the same class (at most 8, 16, 32 or 64 columns per
@@ -457,9 +455,9 @@ int h2_tree_build(const h2_build_params* params, const double* pts, int64_t n, h
 /* Pointers stay valid until h2_tree_free. */
 int h2_tree_view_get(const h2_tree* T, h2_tree_view* view);
 int h2_tree_free(h2_tree* T);
-/* The schedules of the FP32/BF16 transfer passes for this tree (each CTA owns
- * the subtrees of cut clusters; the same builder serves h2_build), for
- * inspection and tests.  which = 0: downward pass, steps (c, rd, wr, flags)
+/* Subtree schedules of the two transfer passes for this tree (tasks that each own
+ * the subtree of a cut cluster, in an order that needs no other task), for
+ * inspection and for callers that walk the tree themselves.  which = 0: downward pass, steps (c, rd, wr, flags)
  * with flags 1 = load the root's ŷ into entry wr, 2 = store ŷ_c (a leaf);
  * which = 1: upward pass, steps (c, rd0, rd1, wr), a leaf having rd0 = -1 and
  * rd1 = its position among the leaves.  Entries index a per-task stack of

@@ -315,16 +315,19 @@ int h2_info(const h2_matrix* A, h2_info_t* info) {
         info->flops_per_col = 2.0 * (2.0 * 2.0 * (double)A->n * k + 2.0 * 2.0 * (double)(A->nc - 1) * k * k) +
                               8.0 * ((double)A->n_adm * k * k + (double)A->nnz_near) + 4.0 * (double)A->n;
     info->launches = A->launches_per_product;
-    // tensor-core chain: gather, upward pass, coupling, downward pass, leaf phase, scatter into Y, + zeroing of
-    // clusters without couplings (done by the gather with the hybrid upward pass); where the subtree-owning
-    // transfer passes do not apply (k % 4 != 0 or k > 64) also the packing of X, x̂ and ŷ
-    const bool own_passes = A->f32.Et && A->k % 8 == 0 && A->k <= 64;
-    const bool hybrid_default = own_passes && (A->tc.hybrid || A->tc.hybrid_bf16) && A->tc.h_default;
-    info->launches_tc = A->tc.built ? (own_passes ? 5 : 8) + (A->down_ptr.back() > 0 ? 1 : 0) +
-                                          (A->tc.c_nzero > 0 && !hybrid_default ? 1 : 0)
-                                    : 0;
+    // tensor-core chain with the transfer passes as lists of pairs: leaves, a launch per stage of
+    // both passes, coupling, leaf phase, scatter into Y.  Without: gather, upward pass, coupling,
+    // downward pass, leaf phase, scatter, three packing launches, + zeroing of clusters without couplings
+    const bool pairs = A->pairs_built && A->use_kron;
+    const bool hybrid = pairs && (A->tc.hybrid || A->tc.hybrid_bf16) && A->tc.h_default;
+    info->launches_tc = 0;
+    if (A->tc.built && pairs)
+        info->launches_tc = 4 + (int32_t)(A->down_pairs.stages.size() +
+                                          (hybrid ? (size_t)A->up_pairs.below_cut : A->up_pairs.stages.size()));
+    else if (A->tc.built)
+        info->launches_tc = 8 + (A->down_ptr.back() > 0 ? 1 : 0) + (A->tc.c_nzero > 0 ? 1 : 0);
     info->kernel = A->kernel;
-    info->hybrid = (A->tc.hybrid || A->tc.hybrid_bf16) && A->tc.h_default ? 1 : 0;
+    info->hybrid = hybrid ? 1 : 0;
     info->n_above_cut = A->tc.h_nabove;
     return 0;
 }

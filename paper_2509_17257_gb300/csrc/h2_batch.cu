@@ -415,8 +415,8 @@ int h2_autotune_ex(h2_matrix* A, int64_t m, int32_t dtype, void* stream, h2_tune
     // 2. the stage count of the tensor-core kernels on the best path
     if (!rc && best_t.path != kPathSimt)
         for (int sc : {4, 5}) trial(Tune{best_t.path, (int8_t)sc}, best_up, best_down);
-    // 3. the cut of the CUDA-core subtree passes, upward then downward
-    const bool subtree = A->f32.Et && A->k % 8 == 0 && A->k <= 64 && mc % 4 == 0 && A->T.leaf_size <= 64;
+    // 3. the cuts of the CUDA-core transfer passes, upward then downward
+    const bool subtree = A->pairs_built && A->use_kron;
     if (!rc && (best_t.path == kPathTcOwn || best_t.path == kPathTcHybrid) && subtree) {
         const int up0 = best_up;
         for (int u : {kUpTasks / 2, kUpTasks * 2}) trial(best_t, u, best_down);

@@ -232,18 +232,6 @@ int upload(h2_matrix* A, T** dst, const std::vector<T>& src, cudaStream_t st) {
     return 0;
 }
 
-// Et[c][μ][ν] = E[c][ν][μ] in FP32, rows of kEtLd floats (k×kEtLd per cluster, zero
-// past column k): one bulk copy lands a cluster's block with the row stride the
-// downward pass's warp-MMA fragment loads want (≡ 8 mod 32, no bank conflicts).
-__global__ void k_transpose_f32(const double* __restrict__ E, float* __restrict__ Et, int64_t nc, int k) {
-    const int64_t per = (int64_t)k * kEtLd;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nc * per; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t c = e / per;
-        const int q = (int)((e % per) / kEtLd), r = (int)(e % kEtLd);
-        Et[e] = r < k ? (float)E[c * k * k + (int64_t)r * k + q] : 0.f;
-    }
-}
-
 // Lays out a work list sorted by decreasing cost for a kernel whose CTA b
 // takes positions b, b + G, b + 2G, ...: round r of G items goes to the CTAs
 // in order for even r and in reverse for odd r (the last, partial round in
@@ -630,17 +618,6 @@ int build_device(h2_matrix* A, const double* pts_host, uint32_t precisions, cuda
     UP(A->d_leaves, A->leaves);
     UP(A->d_up_list, up_list);
     UP(A->d_down_list, down_list);
-    {
-        std::vector<int32_t> task_ptr;
-        std::vector<DownStep> dsteps;
-        down_schedule(T, A->down_target, task_ptr, dsteps, A->dn_ntasks, A->dn_entries);
-        UP(A->d_dn_task_ptr, task_ptr);
-        UP(A->d_dn_steps, dsteps);
-        std::vector<UpStep> usteps;
-        up_schedule(T, A->up_target, task_ptr, usteps, A->up_ntasks, A->up_entries, &A->up_cut);
-        UP(A->d_up_task_ptr, task_ptr);
-        UP(A->d_up_steps, usteps);
-    }
     UP(A->d_adm_rowptr, adm_rowptr);
     UP(A->d_adm_col, adm_col);
     UP(A->d_adm_row, adm_row);
@@ -746,13 +723,7 @@ int build_device(h2_matrix* A, const double* pts_host, uint32_t precisions, cuda
             if ((rc = cast_copy(A, (const double*)A->f64.V, &A->f32.V, (int64_t)n * k, st))) return rc;
             if ((rc = cast_copy(A, (const double*)A->f64.E, &A->f32.E, nc * k * k, st))) return rc;
         }
-        if (k % 8 == 0 && k <= 64) {
-            // transposed transfer matrices for the subtree-owning downward pass
-            if ((rc = device_alloc(A, &A->f32.Et, (size_t)nc * k * kEtLd * sizeof(float)))) return rc;
-            k_transpose_f32<<<1216, 256, 0, st>>>((const double*)A->f64.E, (float*)A->f32.Et, nc, k);
-            H2_LAUNCH_CHECK();
-        }
-
+        if ((rc = build_pairs(A, st))) return rc;
         if ((rc = build_tc(A, want_bf16, want_tf32, st))) return rc;
     }
     H2_CUDA_TRY(cudaStreamSynchronize(st));
@@ -947,8 +918,8 @@ int flow_lists(h2_matrix* A, const FlowTiles& ft, const std::vector<int64_t>& s_
     return 0;
 }
 
-// The coupling launch of the hybrid upward pass (k_tc_gemm<4, KIND>).  The CUDA-core
-// subtree pass (k_up_own without its climb) computes every cluster at or below
+// The coupling launch of the hybrid upward pass (k_tc_gemm<4, KIND>).  The lists
+// of pairs compute every cluster at or below
 // the cut level up_cut (and the leaves above it); the clusters above the cut,
 // x̂_t = E_s0ᵀ x̂_s0 + E_s1ᵀ x̂_s1 (Alg. "forward/backward"), become transfer items
 // of the coupling launch, each writing its split tile and ready flag.  A term
@@ -1414,47 +1385,17 @@ int build_tc_transposed(h2_matrix* A, cudaStream_t st) {
     return 0;
 }
 
-// New cut targets for the subtree schedules of the CUDA-core transfer passes
-// (h2_autotune): the schedules are rebuilt and replace the old ones, which are
-// freed once the stream has finished with them.
+// New cut targets for the transfer passes (h2_autotune): their lists are rebuilt
+// and replace the old ones once the stream has finished with them.
 int set_transfer_targets(h2_matrix* A, int up_target, int down_target, cudaStream_t st) {
     if (up_target == A->up_target && down_target == A->down_target) return 0;
-    std::vector<int32_t> dptr, uptr;
-    std::vector<DownStep> dsteps;
-    std::vector<UpStep> usteps;
-    int32_t dn_ntasks = 0, dn_entries = 0, up_ntasks = 0, up_entries = 0;
-    down_schedule(A->T, down_target, dptr, dsteps, dn_ntasks, dn_entries);
-    int32_t up_cut = 0;
-    up_schedule(A->T, up_target, uptr, usteps, up_ntasks, up_entries, &up_cut);
-    if (up_entries > kUpMaxEntries || dn_entries > 8) {
-        set_error("transfer-pass schedule needs more stack entries than the kernels hold");
-        return H2_E_UNSUPPORTED;
-    }
-    int32_t *d_dptr = nullptr, *d_uptr = nullptr;
-    DownStep* d_ds = nullptr;
-    UpStep* d_us = nullptr;
-    int rc = 0;
-    if ((rc = upload(A, &d_dptr, dptr, st)) || (rc = upload(A, &d_ds, dsteps, st)) || (rc = upload(A, &d_uptr, uptr, st)) ||
-        (rc = upload(A, &d_us, usteps, st)))
-        return rc;
-    H2_CUDA_TRY(cudaStreamSynchronize(st));
-    release_allocation(A, A->d_dn_task_ptr);
-    release_allocation(A, A->d_dn_steps);
-    release_allocation(A, A->d_up_task_ptr);
-    release_allocation(A, A->d_up_steps);
-    A->d_dn_task_ptr = d_dptr;
-    A->d_dn_steps = d_ds;
-    A->dn_ntasks = dn_ntasks;
-    A->dn_entries = dn_entries;
-    A->d_up_task_ptr = d_uptr;
-    A->d_up_steps = d_us;
-    A->up_ntasks = up_ntasks;
-    A->up_entries = up_entries;
     A->up_target = up_target;
     A->down_target = down_target;
-    const bool cut_moved = up_cut != A->up_cut;
-    A->up_cut = up_cut;
-    if (cut_moved && A->tc.built) return hybrid_lists(A, st);
+    if (!A->pairs_built) return 0;
+    const int32_t was = A->up_cut;
+    int rc = build_pairs(A, st);
+    if (rc) return rc;
+    if (was != A->up_cut && A->tc.built) return hybrid_lists(A, st);
     return 0;
 }
 

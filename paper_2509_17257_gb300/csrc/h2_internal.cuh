@@ -43,7 +43,6 @@ void set_error(const std::string& msg);
 struct MatData {
     void* V = nullptr;
     void* E = nullptr;
-    void* Et = nullptr;  // FP32 only, k % 8 == 0, k <= 64: E_{t'}ᵀ per cluster, rows of kEtLd floats
     void* kron = nullptr;  // q = 4: the 4×4 factors F_x, F_y, F_z of E_{t'} = F_z ⊗ F_y ⊗ F_x [n_c][48]
     void* S = nullptr;
     void* Near = nullptr;
@@ -241,40 +240,32 @@ struct TcData {
     std::vector<int64_t> ebh_off_host, ebl_off_host;  // Eᵀ_c high and low tiles in mat (bytes)
 };
 
-// Inter-CTA bookkeeping of the one-launch transfer passes: arrival counters of
-// the upward pass (self-resetting), ready flags of the downward pass and its
-// claim tickets (both cleared before every downward pass, so a captured CUDA
-// graph can replay the product).
-// One step of the subtree-owning downward pass (k_down_own, h2_mm.cu): cluster c
-// gets ŷ_c = ŷ_c + E_c ŷ_parent with ŷ_parent read from shared-memory stack
-// entry rd and the result kept in entry wr; kDownLoad marks the first step of a
-// task (entry wr ← the root's ŷ, no product), kDownStore a leaf whose ŷ goes
-// back to global memory.
+// One step of the downward subtree schedule (down_schedule): cluster c gets ŷ_c =
+// ŷ_c + E_c ŷ_parent with ŷ_parent in stack entry rd and the result in entry wr;
+// kDownLoad marks the first step of a task (entry wr ← the root's ŷ, no product),
+// kDownStore a leaf.
 struct DownStep {
     int32_t c, rd, wr, flags;
 };
 constexpr int kDownLoad = 1, kDownStore = 2;
-constexpr int kEtLd = 72;  // row stride of the FP32 Eᵀ blocks (≡ 8 mod 32)
 constexpr int kTcGrid = 152;  // CTAs of the tensor-core kernels (one per SM); their work lists are laid out for it
 constexpr int kDownMaxSteps = 192;  // steps of one task at most (the schedule keeps to it)
 
-// One step of the subtree-owning upward pass (k_up_own, h2_mm.cu): a leaf c
-// (rd0 < 0, rd1 = its position among the leaves) gets x̂_c = V_cᵀ X|_ĉ; an
-// inner cluster gets x̂_c = E_s0ᵀ x̂_s0 + E_s1ᵀ x̂_s1 with the sons' x̂ in
-// shared-memory stack entries rd0 and rd1.  x̂_c goes to global memory and to
-// entry wr.
+// One step of the upward subtree schedule (up_schedule): a leaf c (rd0 < 0, rd1 =
+// its position among the leaves) or an inner cluster whose sons are in stack
+// entries rd0 and rd1; x̂_c goes to entry wr.
 struct UpStep {
     int32_t c, rd0, rd1, wr;
 };
 constexpr int kUpMaxSteps = 64;    // steps of one task at most
-// Task counts the cut levels aim at: the downward pass takes the shallowest level
-// with at least kDownTasks subtrees; the upward pass, whose longest subtree bounds
-// its task phase, about 1.7 tasks per CTA slot (two per SM)
+// Default targets of the passes' cuts (h2_autotune moves them): the lists of pairs
+// cut at the shallowest level with a sixth of the leaf count times target / default
+// clusters, the subtree schedules at the shallowest with that many tasks
 constexpr int kDownTasks = 256, kUpTasks = 400;
-constexpr int kUpMaxEntries = 5;   // stack entries at most (three of them serve the climb above the cut)
+constexpr int kUpMaxEntries = 5;   // stack entries at most
 
 struct Tree;
-// Transfer-pass schedules (h2_build.cu), host only
+// Subtree schedules of a tree (h2_build.cu, h2_tree_schedule), host only
 void down_schedule(const Tree& T, int target, std::vector<int32_t>& task_ptr, std::vector<DownStep>& steps,
                    int32_t& ntasks, int32_t& entries);
 void up_schedule(const Tree& T, int target, std::vector<int32_t>& task_ptr, std::vector<UpStep>& steps,
@@ -284,12 +275,12 @@ void up_schedule(const Tree& T, int target, std::vector<int32_t>& task_ptr, std:
 // Product variants the autotuner chooses among (h2_autotune).
 enum ProductPath : int8_t {
     kPathDefault = 0,  // built-in rule: tensor cores where built; their transfer passes where the
-                       // CUDA-core subtree passes do not apply (k % 8 != 0 or columns % 4 != 0)
+                       // lists of pairs do not apply (q = 1 or 5, H2_KRON=0, trees of very long paths)
     kPathTcOwn = 1,    // tensor cores, CUDA-core transfer passes
     kPathTcFlow = 2,   // tensor cores, tensor-core transfer passes, one launch per phase
     kPathTcFused = 3,  // tensor cores, transfer passes sharing launches with coupling and leaf phases
     kPathSimt = 4,     // CUDA cores only (FP32)
-    kPathTcHybrid = 5  // tensor cores, CUDA-core subtree passes below the cut, the clusters above
+    kPathTcHybrid = 5  // tensor cores, CUDA-core transfer passes below the cut, the clusters above
                        // the upward cut as transfer items of the coupling launch
 };
 struct Tune {
@@ -298,6 +289,30 @@ struct Tune {
 };
 inline int column_class(int mc) { return mc <= 8 ? 0 : (mc <= 16 ? 1 : (mc <= 32 ? 2 : 3)); }
 
+// The transfer passes of the tensor-core products (h2_transfer.cu): items of one
+// launch are the clusters it computes, with the pairs [p0, p1) of (descendant,
+// ancestor) clusters whose contributions they sum; the sources of the first few
+// stand in the item.
+constexpr int kInlineSrc = 4;
+struct PairItem {
+    int32_t c, p0, p1, flags;
+    int32_t src[kInlineSrc];
+};
+struct PairPass {
+    struct Stage {
+        int32_t i0, i1, longest;  // items [i0, i1), pairs of the longest list
+    };
+    std::vector<Stage> stages;  // one launch each, in order
+    int below_cut = 0;          // upward: the stages at or below the first cut
+    PairItem* items = nullptr;
+    int2* pair = nullptr;
+    float* fac = nullptr;       // [pairs][3][q][q]
+};
+
+// Inter-CTA bookkeeping of the one-launch transfer passes: arrival counters of
+// the upward pass (self-resetting), ready flags of the downward pass and its
+// claim tickets (both cleared before every downward pass, so a captured CUDA
+// graph can replay the product).
 struct SyncBufs {
     unsigned* cnt = nullptr;
     int* flag = nullptr;
@@ -305,7 +320,6 @@ struct SyncBufs {
     int epoch = 0;
     int* err = nullptr;
     int* fflag = nullptr;  // [2 × n_clusters] ready flags of the tensor-core upward and downward passes
-    unsigned* claim2 = nullptr;  // the tensor-core chain's downward-pass task counter (claim is the upward one)
 };
 
 struct Workspace {
@@ -357,14 +371,9 @@ struct h2_matrix {
     int32_t* d_son0 = nullptr;       // [nc]
     int32_t* d_son1 = nullptr;       // [nc]
     int32_t* d_down_list = nullptr;  // non-root clusters by level
-    // subtree-owning downward pass: task t runs steps dn_steps[dn_task_ptr[t]..dn_task_ptr[t+1])
-    int32_t* d_dn_task_ptr = nullptr;
-    h2::DownStep* d_dn_steps = nullptr;
-    int32_t dn_ntasks = 0, dn_entries = 0;
-    // subtree-owning upward pass: task t runs up_steps[up_task_ptr[t]..up_task_ptr[t+1]), then climbs
-    int32_t* d_up_task_ptr = nullptr;
-    h2::UpStep* d_up_steps = nullptr;
-    int32_t up_ntasks = 0, up_entries = 0;
+    h2::PairPass up_pairs, down_pairs;  // transfer passes of the tensor-core products (q = 2..4)
+    int4* d_leaf_rec = nullptr;         // [n_leaves] (cluster, first position, points, first X tile column)
+    bool pairs_built = false;
     int32_t* d_adm_rowptr = nullptr; // [nc+1] by row cluster
     int32_t* d_adm_col = nullptr;    // [n_adm]
     int32_t* d_adm_row = nullptr;    // [n_adm]
@@ -405,7 +414,7 @@ struct h2_matrix {
     // (columns per 64-column chunk: <= 8, <= 16, <= 32, <= 64)
     h2::Tune tune[2][4];
     int32_t up_target = h2::kUpTasks, down_target = h2::kDownTasks;  // transfer-pass cut targets
-    int32_t up_cut = 0;  // level of the upward pass's task roots (leaves above it are tasks too)
+    int32_t up_cut = 0;  // first cut of the upward pass: the hybrid launch takes the clusters above it
     // H2_TC_HYBRID at build: 1 / 0 force the hybrid upward pass on / off (unset: tuning or default)
     int use_hybrid = -1;
     // H2_KRON at build: 0 keeps the q = 4 transfer passes on the dense transfer matrices
@@ -581,7 +590,7 @@ int tc_prepare();
 // allocates nothing (e.g. while it is captured into a CUDA graph).
 int product_prepare(h2_matrix* A, int64_t m, int32_t dtype, cudaStream_t st);
 int launch_tc_gemm(int mode, int kind, TcGemmParams p, cudaStream_t st, int stages = 0);
-// Rebuild the subtree schedules of the CUDA-core transfer passes for other cut targets.
+// Rebuild the CUDA-core transfer passes' lists of pairs for other cut targets.
 int set_transfer_targets(h2_matrix* A, int up_target, int down_target, cudaStream_t st);
 // Work list of the coupling launch with the clusters above the upward cut (TcData::h_*).
 int hybrid_lists(h2_matrix* A, cudaStream_t st);
@@ -593,6 +602,14 @@ int launch_pack_act(const float* src, int64_t ld, int ids, const int32_t* idmap,
 int launch_zero_clusters(const int32_t* ids, int count, float* yhat, int k, int ldc, int mc, cudaStream_t st);
 int launch_zero_tiles(const int32_t* ids, int count, uint8_t* buf, int64_t tile_bytes, cudaStream_t st);
 int build_tc(h2_matrix* A, bool bf16, bool tf32, cudaStream_t st);
+// The transfer passes as lists of pairs (h2_transfer.cu), q = 2, 3, 4.
+int build_pairs(h2_matrix* A, cudaStream_t st);
+int launch_pairs(h2_matrix* A, const PairPass& ps, int s0, int s1, bool up, const float* in, float* out, uint8_t* act,
+                 int m, int R, int es, cudaStream_t st);
+int launch_forward(h2_matrix* A, const double* X, int64_t ldx, int mreal, int m, float* xhat, uint8_t* xcm,
+                   uint8_t* Xcm, int R, int es, bool below, int* zflag, int nflag, const int32_t* zid, int nzid,
+                   float* yhat, cudaStream_t st);
+int launch_backward(h2_matrix* A, float* yhat, uint8_t* ycm, int m, int R, int es, cudaStream_t st);
 // Tiles and work lists of the tensor-core product with Aᵀ (once per matrix; allocates).
 int build_tc_transposed(h2_matrix* A, cudaStream_t st);
 

@@ -19,7 +19,6 @@
 #include <type_traits>
 #include <vector>
 
-#include "h2_async.cuh"
 #include "h2_internal.cuh"
 
 namespace h2 {
@@ -231,25 +230,8 @@ __device__ __forceinline__ int row_lanes(int m) {
 
 // ---- gather: Xp[i, :] = X[perm[i], :] in the compute type ----
 template <typename T>
-// With z1/z2/z3 it also zeroes the counters and flags the passes after it use,
-// and with zid the k×zmc blocks of ŷ (rows of zld) of the clusters zid[0..nzc)
-// (in place of separate memsets and launches on the stream).
 __global__ void k_gather(const double* __restrict__ X, int64_t ldx, const int32_t* __restrict__ perm, int64_t n,
-                         int m, T* __restrict__ Xp, unsigned* __restrict__ z1 = nullptr, int n1 = 0,
-                         unsigned* __restrict__ z2 = nullptr, int n2 = 0, int* __restrict__ z3 = nullptr, int n3 = 0,
-                         const int32_t* __restrict__ zid = nullptr, int nzc = 0, float* __restrict__ zy = nullptr,
-                         int zk = 0, int zld = 0, int zmc = 0) {
-    {
-        const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
-        for (int64_t i = t; i < n1; i += nt) z1[i] = 0u;
-        for (int64_t i = t; i < n2; i += nt) z2[i] = 0u;
-        for (int64_t i = t; i < n3; i += nt) z3[i] = 0;
-        const int64_t blk = (int64_t)zk * zmc;
-        for (int64_t e = t; e < nzc * blk; e += nt) {
-            const int64_t c = e / blk, r = e % blk;
-            zy[((int64_t)zid[c] * zk + r / zmc) * zld + r % zmc] = 0.f;
-        }
-    }
+                         int m, T* __restrict__ Xp) {
     const int P = row_lanes(m), R = 32 / P;
     const int lane = threadIdx.x & 31, sub = lane / P, cl = lane % P;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -277,6 +259,12 @@ __global__ void k_scatter_y(const float* __restrict__ Z, int ldz, const int32_t*
             if (overwrite) y[c] = v; else y[c] += v;
         }
     }
+}
+
+void launch_scatter_y(const float* Z, int ldz, const int32_t* perm, int64_t n, int m, const double* X, int64_t ldx,
+                      double* Y, int64_t ldy, double alpha, double sigma, bool overwrite, cudaStream_t st) {
+    const unsigned g = (unsigned)std::min<int64_t>((n * m + 255) / 256, 152 * 32);
+    k_scatter_y<<<g, 256, 0, st>>>(Z, ldz, perm, n, m, X, ldx, Y, ldy, alpha, sigma, overwrite ? 1 : 0);
 }
 
 // ---- the same over C: interleaved (real, imaginary) columns, m2 = 2·m_c, and
@@ -622,755 +610,6 @@ __global__ void __launch_bounds__(kThreads) k_leaf_bwd_near_c(
     }
 }
 
-// ---------------------------------------------------------------------------
-// FP32 transfer passes for k % 4 == 0, k <= 64, m % 4 == 0, leaves of at most
-// 64 points.  The tree is cut at one level; each task (a cut cluster) is owned
-// by one CTA, which evaluates its subtree with every intermediate x̂ or ŷ kept
-// in shared memory.  Static operands (V_t, X|_t̂, the transfer matrices, the
-// coupling results) arrive by bulk copies one step ahead.  Only the clusters
-// above the cut in the upward pass are shared between CTAs (last arriver of
-// two brothers computes the father).
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void cp16_cg(void* s, const void* g) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(s)), "l"(g) : "memory");
-}
-__device__ __forceinline__ void cp_commit_wait() {
-    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-}
-
-// acc[4][4] += a[0:K][rows 4ty..4ty+3] contracted with b[0:K][cols 4tx..4tx+3],
-// row strides lda and ldb floats (multiples of 4).  The operand rows of eight
-// contraction steps are loaded before their 128 FMAs, walking two pointers
-// (a 64×64×32 contraction on four warps: about 2450 cycles, against about 3900
-// for a per-step indexed loop with runtime strides).  Rows and columns past the
-// valid ones read neighbouring data and give outputs nobody stores.
-__device__ __forceinline__ void contract44(float (&acc)[4][4], const float* a, int lda, const float* b, int ldb, int K,
-                                           int tx, int ty) {
-    const float* pa = a + 4 * ty;
-    const float* pb = b + 4 * tx;
-    auto step = [&](const float4 x, const float4 y) {
-        const float xv[4] = {x.x, x.y, x.z, x.w}, yv[4] = {y.x, y.y, y.z, y.w};
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(xv[r], yv[c], acc[r][c]);
-    };
-    int kk = 0;
-    for (; kk + 8 <= K; kk += 8) {
-        float4 x[8], y[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            x[u] = *(const float4*)(pa + u * lda);
-            y[u] = *(const float4*)(pb + u * ldb);
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) step(x[u], y[u]);
-        pa += 8 * lda;
-        pb += 8 * ldb;
-    }
-    for (; kk < K; ++kk) {
-        step(*(const float4*)pa, *(const float4*)pb);
-        pa += lda;
-        pb += ldb;
-    }
-}
-
-// Split activation tiles written by the transfer passes for the tensor-core
-// phases (the layout k_pack_act writes): act holds one R×KP tile per cluster
-// (x̂ in the upward pass, leaf ŷ in the downward pass), leafX one R×kp tile per
-// leaf (kp = xkoff[l+1] - xkoff[l]) of the leaf's X rows.
-struct PackOut {
-    uint8_t* act;
-    uint8_t* leafX;
-    const int64_t* xkoff;
-    int KP, R, es;
-};
-
-// The thread's 4×4 block of a k×m result (rows 4ty.., columns 4tx..) into a
-// cluster's tile, zeros in the padding rows (columns i >= m) and columns
-// (κ >= k).
-__device__ __forceinline__ void pack_rows(const PackOut& pk, uint8_t* tile, const float (&acc)[4][4], int tx, int ty,
-                                          int k, int m) {
-    if (4 * ty >= pk.KP) return;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const int i = 4 * tx + c;
-        if (2 * i >= pk.R) continue;
-        float v[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) v[r] = (i < m && 4 * ty + r < k) ? acc[r][c] : 0.f;
-        put_act4(tile, pk.KP, pk.es, i, 4 * ty, v);
-    }
-}
-
-// A leaf's X rows (nt points × m columns in shared memory, row stride m) into
-// its tile of kp contraction columns (the points), zero padded.
-__device__ __forceinline__ void pack_points(const PackOut& pk, uint8_t* tile, int kp, const float* x, int nt, int m) {
-    const int half = pk.R >> 1;
-    for (int it = threadIdx.x; it < (kp >> 2) * half; it += blockDim.x) {
-        const int q0 = 4 * (it / half), i = it % half;
-        float v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = (i < m && q0 + u < nt) ? x[(q0 + u) * m + i] : 0.f;
-        put_act4(tile, kp, pk.es, i, q0, v);
-    }
-}
-
-// acc (rows 4ty.., columns 4tx.. of a 64-row block) += E_cᵀ x for q = 4, E_c =
-// F_z ⊗ F_y ⊗ F_x with the factors at f (global memory, F_a[μ][ν] row-major) and x
-// in shared memory (row stride ldx): the x mode product in the thread (its rows
-// are one x-fiber), the y and z mode products through `scratch` (64 rows of ld
-// floats, ld >= 4·(tx + 1), of shared memory free for the call).  Columns past
-// the block's read neighbouring data and give outputs nobody stores.  Every
-// thread of the CTA calls it.
-__device__ __forceinline__ void kron_own_t(float (&acc)[4][4], const float* x, int ldx, float* scratch, int ld,
-                                           const float* __restrict__ f, int tx, int ty) {
-    float F[48];
-#pragma unroll
-    for (int i = 0; i < 48; ++i) F[i] = __ldg(f + i);
-    // transposed factors: Fᵀ_a[μ][ν] = F_a[ν][μ]
-    auto Ft = [&](int a, int mu, int nu) { return F[16 * a + 4 * nu + mu]; };
-    const int my = ty & 3, mz = ty >> 2;
-    float t[4][4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        float v[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) v[r] = x[(4 * ty + r) * ldx + 4 * tx + j];
-#pragma unroll
-        for (int mx = 0; mx < 4; ++mx) {
-            float a = 0.f;
-#pragma unroll
-            for (int r = 0; r < 4; ++r) a = fmaf(Ft(0, mx, r), v[r], a);
-            t[mx][j] = a;
-        }
-    }
-    __syncthreads();  // earlier users of the scratch are done
-#pragma unroll
-    for (int mx = 0; mx < 4; ++mx)
-        *(float4*)(scratch + (4 * ty + mx) * ld + 4 * tx) = make_float4(t[mx][0], t[mx][1], t[mx][2], t[mx][3]);
-    __syncthreads();
-#pragma unroll
-    for (int mx = 0; mx < 4; ++mx) {
-        float a[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const float4 w = *(const float4*)(scratch + (mx + 4 * v + 16 * mz) * ld + 4 * tx);
-            const float c = Ft(1, my, v);
-            a[0] = fmaf(c, w.x, a[0]); a[1] = fmaf(c, w.y, a[1]); a[2] = fmaf(c, w.z, a[2]); a[3] = fmaf(c, w.w, a[3]);
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) t[mx][j] = a[j];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int mx = 0; mx < 4; ++mx)
-        *(float4*)(scratch + (4 * ty + mx) * ld + 4 * tx) = make_float4(t[mx][0], t[mx][1], t[mx][2], t[mx][3]);
-    __syncthreads();
-#pragma unroll
-    for (int mx = 0; mx < 4; ++mx)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const float4 w = *(const float4*)(scratch + (mx + 4 * my + 16 * v) * ld + 4 * tx);
-            const float c = Ft(2, mz, v);
-            acc[mx][0] = fmaf(c, w.x, acc[mx][0]);
-            acc[mx][1] = fmaf(c, w.y, acc[mx][1]);
-            acc[mx][2] = fmaf(c, w.z, acc[mx][2]);
-            acc[mx][3] = fmaf(c, w.w, acc[mx][3]);
-        }
-}
-
-// Upward pass with subtree ownership (schedule: up_schedule, h2_build.cu), the
-// forward transformation of Alg. "fast_addeval" (Sec. 3): x̂_t = V_tᵀ X|_t̂ at
-// the leaves and x̂_t = E_s0ᵀ x̂_s0 + E_s1ᵀ x̂_s1 above.  A CTA claims a task and
-// evaluates its subtree in post-order; the static operands of step s + 1 (V_c
-// and X|_ĉ, or E_s0 and E_s1) arrive by bulk copies while step s computes, the
-// sons' x̂ come from the shared-memory stack.  Above the cut the last of two
-// brothers to finish computes their father (an atomic counter per cluster,
-// reset by the last arriver), adding the two brothers' contributions E_sᵀ x̂_s,
-// which each brother computes and publishes before the atomic.  One IEEE
-// addition of two contributions does not depend on their order, so the result
-// does not depend on which brother arrives last.  With climb = 0 a CTA stops
-// at its task's root: the clusters above the cut are then items of the
-// coupling launch (k_tc_gemm<4, 1>).  64·CN threads, thread (tx, ty) owns rows
-// 4ty.. and columns 4tx.. of the k×m result.
-template <int CN>
-__global__ void __launch_bounds__(64 * CN) k_up_own(const int32_t* __restrict__ task_ptr, int ntasks,
-                                                    const UpStep* __restrict__ steps,
-                                                    const int32_t* __restrict__ cl_off,
-                                                    const int32_t* __restrict__ cl_size,
-                                                    const int32_t* __restrict__ parent,
-                                                    const int32_t* __restrict__ son0,
-                                                    const int32_t* __restrict__ son1, const float* __restrict__ V,
-                                                    const float* __restrict__ E, const float* __restrict__ Xp,
-                                                    float* xhat, float* part, unsigned* __restrict__ cnt,
-                                                    unsigned* __restrict__ claim, int* __restrict__ err, int nent, int k,
-                                                    int m, PackOut pk, int climb, const float* __restrict__ kron) {
-    constexpr int NT = 16 * CN;
-    extern __shared__ __align__(16) float fsm[];
-    float* sbuf = fsm;                 // [2 slots][2][64·64]  V_c and X|_ĉ, or E_s0 and E_s1
-    float* stk = sbuf + 4 * 64 * 64;   // [entries][64·NT]     x̂ waiting for the father
-    __shared__ int s_task, s_go;
-    __shared__ UpStep s_steps[kUpMaxSteps];
-    __shared__ int s_off[kUpMaxSteps], s_nt[kUpMaxSteps];
-    __shared__ __align__(8) uint64_t bar[2];
-    const int tx = threadIdx.x % (4 * CN), ty = threadIdx.x / (4 * CN);
-    const bool colv = 4 * tx < m;
-    const int64_t kk = (int64_t)k * k, km = (int64_t)k * m;
-    if (threadIdx.x == 0) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    uint32_t phase = 0;
-    bool failed = false;
-    auto slot = [&](int b, int h) { return sbuf + (2 * b + h) * 64 * 64; };
-    auto ent = [&](int e) { return stk + e * 64 * NT; };
-    // acc → stack entry e, x̂_c in global memory and its split tile for the coupling phase
-    // (the tensor-core phases read only the split tiles, so x̂ is not stored in FP32)
-    auto put = [&](const float (&acc)[4][4], int e, int c) {
-        pack_rows(pk, pk.act + (int64_t)c * pk.KP * pk.R * pk.es, acc, tx, ty, k, m);
-        if (!colv) return;
-        float* out = ent(e);
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-            *(float4*)(out + (4 * ty + r) * m + 4 * tx) = make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
-    };
-    auto wait_slot = [&](int b) {
-        const bool ok = mbar_wait(&bar[b], (phase >> b) & 1u);
-        phase ^= 1u << b;
-        return ok;
-    };
-    while (!failed) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_task = (int)atomicAdd(claim, 1u);
-        __syncthreads();
-        const int task = s_task;
-        if (task >= ntasks) break;
-        const int s0 = task_ptr[task], s1 = min(task_ptr[task + 1], s0 + kUpMaxSteps);
-        for (int i = threadIdx.x; i < s1 - s0; i += blockDim.x) {
-            const UpStep u = steps[s0 + i];
-            s_steps[i] = u;
-            s_off[i] = cl_off[u.c];
-            s_nt[i] = cl_size[u.c];
-        }
-        __syncthreads();
-        auto issue = [&](int s, int b) {
-            if (threadIdx.x != 0) return;
-            const UpStep u = s_steps[s - s0];
-            if (u.rd0 < 0) {
-                const int off = s_off[s - s0], nt = s_nt[s - s0];
-                const uint32_t vb = (uint32_t)nt * k * 4, xb = (uint32_t)nt * m * 4;
-                mbar_expect_tx(&bar[b], vb + xb);
-                bulk_g2s(slot(b, 0), V + (int64_t)off * k, vb, &bar[b]);
-                bulk_g2s(slot(b, 1), Xp + (int64_t)off * m, xb, &bar[b]);
-            } else if (kron) {
-                mbar_arrive(&bar[b]);  // Kronecker factors: nothing to copy, the phase completes now
-            } else {
-                mbar_expect_tx(&bar[b], (uint32_t)(2 * kk * 4));
-                bulk_g2s(slot(b, 0), E + (int64_t)son0[u.c] * kk, (uint32_t)(kk * 4), &bar[b]);
-                bulk_g2s(slot(b, 1), E + (int64_t)son1[u.c] * kk, (uint32_t)(kk * 4), &bar[b]);
-            }
-        };
-        issue(s0, 0);
-        int cur = -1;
-        for (int s = s0; s < s1; ++s) {
-            const int b = (s - s0) & 1;
-            if (s + 1 < s1) issue(s + 1, b ^ 1);
-            const bool ok = wait_slot(b);
-            if (__syncthreads_or(!ok)) {
-                if (threadIdx.x == 0) {
-                    atomicExch(err, 10);
-                    mbar_wait(&bar[b], ((phase >> b) & 1u) ^ 1u);
-                    if (s + 1 < s1) mbar_wait(&bar[b ^ 1], (phase >> (b ^ 1)) & 1u);
-                }
-                failed = true;
-                break;
-            }
-            const UpStep u = s_steps[s - s0];
-            float acc[4][4] = {};
-            if (u.rd0 < 0) {
-                const int nt = s_nt[s - s0];
-                contract44(acc, slot(b, 0), k, slot(b, 1), m, nt, tx, ty);
-                // X|_ĉ (in shared memory) as the leaf's split tile for the nearfield phase
-                const int64_t x0 = pk.xkoff[u.rd1];
-                pack_points(pk, pk.leafX + x0 * pk.R * pk.es, (int)(pk.xkoff[u.rd1 + 1] - x0), slot(b, 1), nt, m);
-            } else if (kron) {
-                // q = 4: E_sᵀ as Kronecker products, slot b (no E copied) as scratch
-                kron_own_t(acc, ent(u.rd0), m, slot(b, 0), NT, kron + (int64_t)son0[u.c] * 48, tx, ty);
-                kron_own_t(acc, ent(u.rd1), m, slot(b, 0), NT, kron + (int64_t)son1[u.c] * 48, tx, ty);
-                __syncthreads();  // x̂ of the father goes into its first son's entry
-            } else {
-                contract44(acc, slot(b, 0), k, ent(u.rd0), m, k, tx, ty);
-                contract44(acc, slot(b, 1), k, ent(u.rd1), m, k, tx, ty);
-                __syncthreads();  // x̂ of the father goes into its first son's entry
-            }
-            put(acc, u.wr, u.c);
-            cur = u.wr;
-            __syncthreads();
-        }
-        if (failed || cur < 0) break;
-        if (!climb) continue;
-        // ---- climb above the cut ----
-        // Every CTA publishes its cluster's contribution P_c = E_cᵀ x̂_c to the father
-        // (in `part`, the ŷ buffer, unused until the coupling phase) before the
-        // atomic, so the last of two brothers only adds P_s0 + P_s1: one
-        // contraction per level on the critical path.
-        int c = s_steps[s1 - 1 - s0].c;
-        // E_c of the next contribution is copied one level ahead (slot 0 is free
-        // after the task's last step)
-        auto fetch_e = [&](int cl) {
-            if (threadIdx.x == 0) {
-                if (kron) {
-                    mbar_arrive(&bar[0]);  // nothing to copy
-                } else {
-                    mbar_expect_tx(&bar[0], (uint32_t)(kk * 4));
-                    bulk_g2s(slot(0, 0), E + (int64_t)cl * kk, (uint32_t)(kk * 4), &bar[0]);
-                }
-            }
-        };
-        if (parent[c] >= 0) fetch_e(c);
-        while (true) {
-            const int par = parent[c];
-            if (par < 0) break;
-            const bool ok = wait_slot(0);
-            if (__syncthreads_or(!ok)) {
-                if (threadIdx.x == 0) atomicExch(err, 10);
-                failed = true;
-                break;
-            }
-            float pc[4][4] = {};
-            if (kron) kron_own_t(pc, ent(cur), m, slot(0, 1), NT, kron + (int64_t)c * 48, tx, ty);
-            else contract44(pc, slot(0, 0), k, ent(cur), m, k, tx, ty);
-            if (colv) {
-                float* g = part + (int64_t)c * km;
-#pragma unroll
-                for (int r = 0; r < 4; ++r)
-                    if (4 * ty + r < k) *(float4*)(g + (4 * ty + r) * m + 4 * tx) = make_float4(pc[r][0], pc[r][1], pc[r][2], pc[r][3]);
-            }
-            __syncthreads();  // every store of P_c is done
-            if (threadIdx.x == 0) {
-                __threadfence();
-                const unsigned old = atomicAdd(&cnt[par], 1u);
-                s_go = old == 1u;
-                if (old == 1u) {
-                    cnt[par] = 0u;
-                    __threadfence();
-                }
-            }
-            __syncthreads();
-            if (!s_go) break;
-            if (parent[par] >= 0) fetch_e(par);  // every thread has finished reading slot 0
-            // the brother's contribution (written by another CTA) through the generic proxy
-            const int bro = son0[par] == c ? son1[par] : son0[par];
-            const int eb = (cur + 1) % 3, er = (cur + 2) % 3;
-            const float* gsrc = part + (int64_t)bro * km;
-            for (int e = threadIdx.x; e < (int)(km / 4); e += blockDim.x) cp16_cg(ent(eb) + 4 * e, gsrc + 4 * e);
-            cp_commit_wait();
-            __syncthreads();
-            const float* pb = ent(eb);
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const float4 v = *(const float4*)(pb + (4 * ty + r) * m + 4 * tx);
-                pc[r][0] += v.x;
-                pc[r][1] += v.y;
-                pc[r][2] += v.z;
-                pc[r][3] += v.w;
-            }
-            put(pc, er, par);
-            cur = er;
-            c = par;
-        }
-    }
-}
-
-// ---- 3xTF32 warp MMAs (mma.sync m16n8k8) for the transfer passes ----
-// A 16×8 TF32 A fragment and 8×8 B fragment per thread (g = lane / 4,
-// t = lane % 4): a0 = A[g][t], a1 = A[g+8][t], a2 = A[g][t+4], a3 = A[g+8][t+4];
-// b0 = B[t][g], b1 = B[t+4][g]; D: d0 = D[g][2t], d1 = D[g][2t+1], d2 = D[g+8][2t],
-// d3 = D[g+8][2t+1].  An FP32 operand x is split into hi = tf32(x) (rounded)
-// and lo = x - hi; D += A_lo·B_hi + A_hi·B_lo + A_hi·B_hi keeps FP32 accuracy.
-__device__ __forceinline__ void tf32_split(float x, uint32_t& hi, uint32_t& lo) {
-    uint32_t h;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(h) : "f"(x));
-    hi = h;
-    lo = __float_as_uint(x - __uint_as_float(h));
-}
-__device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-// d[nt] (N-tile nt: columns 8nt..8nt+7) += A·B over K = kdim (a multiple of 8)
-// for the warp's 16 rows m0..m0+15, with A[i][j] = a[j·lda + i] (a transposed
-// K-major block) and B[j][n] = b[j·ldb + n]; lda, ldb ≡ 8 (mod 32) keep the
-// fragment loads free of bank conflicts.
-template <int NTILES>
-__device__ __forceinline__ void mma_contract(float (&d)[NTILES][4], const float* a, int lda, const float* b, int ldb,
-                                             int kdim, int m0) {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    for (int k0 = 0; k0 < kdim; k0 += 8) {
-        const float* ar = a + (k0 + t) * lda + m0 + g;
-        uint32_t ah[4], al[4];
-        tf32_split(ar[0], ah[0], al[0]);
-        tf32_split(ar[8], ah[1], al[1]);
-        tf32_split(ar[4 * lda], ah[2], al[2]);
-        tf32_split(ar[4 * lda + 8], ah[3], al[3]);
-        const float* br = b + (k0 + t) * ldb + g;
-#pragma unroll
-        for (int nt = 0; nt < NTILES; ++nt) {
-            uint32_t bh0, bl0, bh1, bl1;
-            tf32_split(br[8 * nt], bh0, bl0);
-            tf32_split(br[4 * ldb + 8 * nt], bh1, bl1);
-            mma_tf32(d[nt], al, bh0, bh1);
-            mma_tf32(d[nt], ah, bl0, bl1);
-            mma_tf32(d[nt], ah, bh0, bh1);
-        }
-    }
-}
-
-// Downward pass with subtree ownership (schedule: down_schedule, h2_build.cu).
-// A CTA claims tasks in the stored order; a task is a list of steps, each
-// ŷ_c += E_c ŷ_father (Sec. 3, the downward transformation of
-// Alg. "fast_addeval"), with ŷ_father in a shared-memory stack entry written by
-// an earlier step of the same task, so no step waits for another CTA.
-// Four warps, warp w computing rows 16w..16w+15 of the k×m result with 3xTF32
-// warp MMAs (mma_contract).  Eᵀ_c of step s + 1 (stored with rows of kEtLd
-// floats) arrives by one bulk copy while step s computes; the coupling result
-// ŷ_c of step s + 1 is loaded into the fragment registers meanwhile.  Stack
-// rows have stride NT + 8; the root's ŷ of a task's first step is copied into
-// its entry row by row (warp 0's lanes).
-template <int CN>
-__global__ void __launch_bounds__(128) k_down_own(const int32_t* __restrict__ task_ptr, int ntasks,
-                                                  const DownStep* __restrict__ steps,
-                                                  const float* __restrict__ Et, float* yhat,
-                                                  unsigned* __restrict__ claim, int* __restrict__ err, int k, int m,
-                                                  PackOut pk) {
-    constexpr int NT = 16 * CN, NTILES = 2 * CN, LDA = kEtLd, LDY = NT + 8;
-    extern __shared__ __align__(16) float fsm[];
-    float* ebuf = fsm;                 // [2][64 rows j][LDA]   Eᵀ_c
-    float* stk = ebuf + 2 * 64 * LDA;  // [entries][64][LDY]    final ŷ along the current path
-    __shared__ int s_task;
-    __shared__ DownStep s_steps[kDownMaxSteps];  // the task's steps: no global load between two steps
-    __shared__ __align__(8) uint64_t bar[2];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int m0 = 16 * warp;
-    const int64_t ke = (int64_t)k * LDA, km = (int64_t)k * m;
-    if (threadIdx.x == 0) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    uint32_t phase = 0;  // bit b: parity of the next completion of bar[b]
-    bool failed = false;
-    // the thread's fragment positions of a k×m block: rows m0+g, m0+g+8; columns 8nt+2t, +1
-    auto load_frag = [&](float (&v)[NTILES][4], const float* src) {
-#pragma unroll
-        for (int nt = 0; nt < NTILES; ++nt) {
-            const int c = 8 * nt + 2 * t;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int r = m0 + g + 8 * h;
-                float2 x = make_float2(0.f, 0.f);
-                if (r < k && c < m) x = __ldcg((const float2*)(src + (int64_t)r * m + c));
-                v[nt][2 * h] = x.x;
-                v[nt][2 * h + 1] = x.y;
-            }
-        }
-    };
-    while (!failed) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_task = (int)atomicAdd(claim, 1u);
-        __syncthreads();
-        const int task = s_task;
-        if (task >= ntasks) break;
-        const int s0 = task_ptr[task], s1 = min(task_ptr[task + 1], s0 + kDownMaxSteps);
-        for (int i = threadIdx.x; i < s1 - s0; i += blockDim.x) s_steps[i] = steps[s0 + i];
-        __syncthreads();
-        // warp 0 arms the buffer's barrier and starts the step's copies: one of
-        // Eᵀ_c, or the root's rows into the stack entry (lane l: rows l, l + 32)
-        auto issue = [&](int s, int b) {
-            if (warp != 0) return;
-            const DownStep d = s_steps[s - s0];
-            if (d.flags & kDownLoad) {
-                const uint32_t rowb = (uint32_t)m * 4;
-                if (lane == 0) mbar_expect_tx(&bar[b], rowb * (uint32_t)k);
-                __syncwarp();
-                for (int r = lane; r < k; r += 32)
-                    bulk_g2s(stk + (d.wr * 64 + r) * LDY, yhat + (int64_t)d.c * km + (int64_t)r * m, rowb, &bar[b]);
-            } else if (lane == 0) {
-                mbar_expect_tx(&bar[b], (uint32_t)(ke * 4));
-                bulk_g2s(ebuf + b * 64 * LDA, Et + (int64_t)d.c * ke, (uint32_t)(ke * 4), &bar[b]);
-            }
-        };
-        float ccur[NTILES][4], cnext[NTILES][4];
-        issue(s0, 0);
-        for (int s = s0; s < s1; ++s) {
-            const int b = (s - s0) & 1;
-            if (s + 1 < s1) {
-                issue(s + 1, b ^ 1);
-                const DownStep dn = s_steps[s + 1 - s0];
-                if (!(dn.flags & kDownLoad)) load_frag(cnext, yhat + (int64_t)dn.c * km);
-            }
-            const bool ok = mbar_wait(&bar[b], (phase >> b) & 1u);
-            phase ^= 1u << b;
-            if (__syncthreads_or(!ok)) {
-                // a copy did not land in time: report, let the copies in flight
-                // finish (bounded), stop
-                if (threadIdx.x == 0) {
-                    atomicExch(err, 9);
-                    mbar_wait(&bar[b], ((phase >> b) & 1u) ^ 1u);
-                    if (s + 1 < s1) mbar_wait(&bar[b ^ 1], (phase >> (b ^ 1)) & 1u);
-                }
-                failed = true;
-                break;
-            }
-            const DownStep d = s_steps[s - s0];
-            if (!(d.flags & kDownLoad)) {
-                mma_contract<NTILES>(ccur, ebuf + b * 64 * LDA, LDA, stk + d.rd * 64 * LDY, LDY, k, m0);
-                float* out = stk + d.wr * 64 * LDY;
-#pragma unroll
-                for (int nt = 0; nt < NTILES; ++nt)
-#pragma unroll
-                    for (int h = 0; h < 2; ++h)
-                        *(float2*)(out + (m0 + g + 8 * h) * LDY + 8 * nt + 2 * t) =
-                            make_float2(ccur[nt][2 * h], ccur[nt][2 * h + 1]);
-                if (d.flags & kDownStore) {
-                    // a leaf: ŷ_c into its split tile (what the leaf phase reads), read back
-                    // from the stack entry in 4×4 blocks
-                    __syncthreads();
-                    uint8_t* tile = pk.act + (int64_t)d.c * pk.KP * pk.R * pk.es;
-                    for (int blk = threadIdx.x; blk < 16 * (NT / 4); blk += blockDim.x) {
-                        const int ty = blk / (NT / 4), tx = blk % (NT / 4);
-                        float acc[4][4];
-#pragma unroll
-                        for (int r = 0; r < 4; ++r) {
-                            const float4 v = *(const float4*)(out + (4 * ty + r) * LDY + 4 * tx);
-                            acc[r][0] = v.x; acc[r][1] = v.y; acc[r][2] = v.z; acc[r][3] = v.w;
-                        }
-                        pack_rows(pk, tile, acc, tx, ty, k, m);
-                    }
-                }
-            }
-            if (s + 1 < s1) {
-#pragma unroll
-                for (int nt = 0; nt < NTILES; ++nt)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) ccur[nt][e] = cnext[nt][e];
-            }
-            __syncthreads();
-        }
-    }
-}
-
-// ---- transfer matrices as Kronecker products (q = 4) ----
-// With tensor Chebyshev interpolation E_c[μ, ν] = L_{ν_x}(ξ_{μ_x}) L_{ν_y}(ξ_{μ_y})
-// L_{ν_z}(ξ_{μ_z}) (1-D Lagrange polynomials of the father's nodes at the son's
-// nodes, per axis), so E_c = F_z ⊗ F_y ⊗ F_x with 4×4 factors (ν = ν_x + 4ν_y +
-// 16ν_z): E_c y costs three 4×4 mode products (48 multiply-adds per column and
-// slab) instead of a 64×64 product, and E_c is 48 numbers.  kron[c] holds F_x,
-// F_y, F_z row-major (F_a[μ][ν]).
-//
-// The thread layout of kron_step: lane quad (4 consecutive lanes) g = 0..3 holds
-// the z-slab ν_z = g of one column; the x and y mode products stay in the
-// thread, the z mode product sums the quad's four slabs through shuffles.
-//   f:   F_x and F_y (32 values); fz: the thread's row g of F_z (TR: its column g)
-//   in:  x[ν_y][ν_x] = block rows 16g + 4ν_y + ν_x, one column
-//   out: y[μ_y][μ_x] = rows 16g + 4μ_y + μ_x of (F_z ⊗ F_y ⊗ F_x) x (TR: of the
-//        transposed product, (F_z ⊗ F_y ⊗ F_x)ᵀ = F_zᵀ ⊗ F_yᵀ ⊗ F_xᵀ)
-template <bool TR>
-__device__ __forceinline__ void kron_step(const float (&f)[32], const float (&fz)[4], const float (&x)[16],
-                                          float (&y)[16]) {
-    auto F = [&](int a, int mu, int nu) { return TR ? f[16 * a + 4 * nu + mu] : f[16 * a + 4 * mu + nu]; };
-    float t[16];
-#pragma unroll
-    for (int vy = 0; vy < 4; ++vy)
-#pragma unroll
-        for (int mx = 0; mx < 4; ++mx) {
-            float a = 0.f;
-#pragma unroll
-            for (int vx = 0; vx < 4; ++vx) a = fmaf(F(0, mx, vx), x[4 * vy + vx], a);
-            t[4 * vy + mx] = a;
-        }
-    float u[16];
-#pragma unroll
-    for (int my = 0; my < 4; ++my)
-#pragma unroll
-        for (int mx = 0; mx < 4; ++mx) {
-            float a = 0.f;
-#pragma unroll
-            for (int vy = 0; vy < 4; ++vy) a = fmaf(F(1, my, vy), t[4 * vy + mx], a);
-            u[4 * my + mx] = a;
-        }
-    const int base = (threadIdx.x & 31) & ~3;
-#pragma unroll
-    for (int e = 0; e < 16; ++e) {
-        float a = 0.f;
-#pragma unroll
-        for (int vz = 0; vz < 4; ++vz) a = fmaf(fz[vz], __shfl_sync(0xffffffffu, u[e], base | vz), a);
-        y[e] = a;
-    }
-}
-
-// Downward pass with subtree ownership for q = 4 (the schedule of k_down_own):
-// each step ŷ_c = ŷ_c + E_c ŷ_father as the Kronecker product above, on the
-// CUDA cores.  The father's ŷ comes from a shared-memory stack entry written by
-// an earlier step of the same task; the factors of the next step and its
-// coupling result load into registers while the current step computes.  The
-// first step of a task copies the root's ŷ into its entry (bulk copies); a
-// leaf's ŷ goes to global memory and into its split tile, as in k_down_own.
-// 128 threads: quad (column c, slab g), c = threadIdx.x / 4 + 32j for j < NT/32.
-template <int CN>
-__global__ void __launch_bounds__(128) k_down_kron(const int32_t* __restrict__ task_ptr, int ntasks,
-                                                   const DownStep* __restrict__ steps,
-                                                   const float* __restrict__ kron, float* yhat,
-                                                   unsigned* __restrict__ claim, int* __restrict__ err, int m,
-                                                   PackOut pk) {
-    constexpr int NT = 16 * CN, LDY = NT + 8, NJ = NT >= 32 ? NT / 32 : 1;
-    constexpr int k = 64;
-    extern __shared__ __align__(16) float fsm[];
-    float* stk = fsm;  // [entries][64][LDY]   final ŷ along the current path
-    __shared__ int s_task;
-    __shared__ DownStep s_steps[kDownMaxSteps];
-    __shared__ __align__(8) uint64_t bar;
-    const int g = threadIdx.x & 3, cq = threadIdx.x >> 2;
-    const int64_t km = (int64_t)k * m;
-    if (threadIdx.x == 0) {
-        mbar_init(&bar, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-    uint32_t phase = 0;
-    bool failed = false;
-    // factors (F_x, F_y and row g of F_z) and coupling rows of one step (this
-    // thread's slab, columns c_j)
-    auto load_step = [&](int c, float (&f)[32], float (&fz)[4], float (&cp)[NJ][16]) {
-        if (c < 0) return;
-#pragma unroll
-        for (int i = 0; i < 32; ++i) f[i] = __ldg(kron + (int64_t)c * 48 + i);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) fz[i] = __ldg(kron + (int64_t)c * 48 + 32 + 4 * g + i);
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) {
-            const int col = cq + 32 * j;
-#pragma unroll
-            for (int e = 0; e < 16; ++e)
-                cp[j][e] = (col < m) ? __ldcg(yhat + (int64_t)c * km + (int64_t)(16 * g + e) * m + col) : 0.f;
-        }
-    };
-    while (!failed) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_task = (int)atomicAdd(claim, 1u);
-        __syncthreads();
-        const int task = s_task;
-        if (task >= ntasks) break;
-        const int s0 = task_ptr[task], s1 = min(task_ptr[task + 1], s0 + kDownMaxSteps);
-        for (int i = threadIdx.x; i < s1 - s0; i += blockDim.x) s_steps[i] = steps[s0 + i];
-        __syncthreads();
-        float fcur[32], fnext[32], zcur[4], znext[4], ccur[NJ][16], cnext[NJ][16];
-        {
-            int f0 = -1;
-            for (int t = s0; t < s1; ++t)
-                if (!(s_steps[t - s0].flags & kDownLoad)) { f0 = t; break; }
-            if (f0 >= 0) load_step(s_steps[f0 - s0].c, fcur, zcur, ccur);
-        }
-        for (int s = s0; s < s1; ++s) {
-            const DownStep d = s_steps[s - s0];
-            if (d.flags & kDownLoad) {
-                // the root's ŷ (its coupling result) into entry wr, one bulk copy per row
-                const uint32_t rowb = (uint32_t)m * 4;
-                if (threadIdx.x < 32) {
-                    if (threadIdx.x == 0) mbar_expect_tx(&bar, rowb * (uint32_t)k);
-                    __syncwarp();
-                    for (int r = threadIdx.x; r < k; r += 32)
-                        bulk_g2s(stk + (d.wr * 64 + r) * LDY, yhat + (int64_t)d.c * km + (int64_t)r * m, rowb, &bar);
-                }
-                const bool ok = mbar_wait(&bar, phase);
-                phase ^= 1u;
-                if (__syncthreads_or(!ok)) {
-                    if (threadIdx.x == 0) {
-                        atomicExch(err, 9);
-                        mbar_wait(&bar, phase);  // the copies land before the CTA leaves (bounded)
-                    }
-                    failed = true;
-                    break;
-                }
-                continue;
-            }
-            // the next step's factors and coupling rows load while this one computes
-            int nx = -1;
-            for (int t = s + 1; t < s1; ++t)
-                if (!(s_steps[t - s0].flags & kDownLoad)) { nx = t; break; }
-            load_step(nx >= 0 ? s_steps[nx - s0].c : -1, fnext, znext, cnext);
-            const float* in = stk + d.rd * 64 * LDY;
-            float* out = stk + d.wr * 64 * LDY;
-#pragma unroll
-            for (int j = 0; j < NJ; ++j) {
-                const int col = cq + 32 * j;
-                if (cq < NT) {  // whole quads: the shuffles stay within active lanes
-                    float x[16], y[16];
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) x[e] = in[(16 * g + e) * LDY + col];
-                    kron_step<false>(fcur, zcur, x, y);
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) out[(16 * g + e) * LDY + col] = y[e] + ccur[j][e];
-                }
-            }
-            __syncthreads();  // entry wr complete
-            if (d.flags & kDownStore) {
-                // a leaf: ŷ_c into its split tile (what the leaf phase reads), read back in 4×4 blocks
-                uint8_t* tile = pk.act + (int64_t)d.c * pk.KP * pk.R * pk.es;
-                for (int blk = threadIdx.x; blk < 16 * (NT / 4); blk += blockDim.x) {
-                    const int ty = blk / (NT / 4), tx = blk % (NT / 4);
-                    float acc[4][4];
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        const float4 v = *(const float4*)(out + (4 * ty + r) * LDY + 4 * tx);
-                        acc[r][0] = v.x; acc[r][1] = v.y; acc[r][2] = v.z; acc[r][3] = v.w;
-                    }
-                    pack_rows(pk, tile, acc, tx, ty, k, m);
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < 32; ++i) fcur[i] = fnext[i];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) zcur[i] = znext[i];
-#pragma unroll
-            for (int j = 0; j < NJ; ++j)
-#pragma unroll
-                for (int e = 0; e < 16; ++e) ccur[j][e] = cnext[j][e];
-        }
-    }
-}
-
-// k_up_own: two slots of two 64×64 blocks plus the stack
-int up_own_smem_bytes(int cn, int entries) { return (4 * 64 * 64 + entries * 64 * 16 * cn) * (int)sizeof(float); }
-// k_down_own: two Eᵀ buffers (rows of 72) plus the stack (rows of 16·cn + 8, at most 8 entries)
-int down_own_smem_bytes(int cn, int entries) { return (2 * 64 * 72 + entries * 64 * (16 * cn + 8)) * (int)sizeof(float); }
-// k_down_kron: the stack only (rows of 16·cn + 8)
-int down_kron_smem_bytes(int cn, int entries) { return entries * 64 * (16 * cn + 8) * (int)sizeof(float); }
-
-int g_fast_attr_device = -1;
-
-int fast_prepare() {
-    int dev = 0;
-    H2_CUDA_TRY(cudaGetDevice(&dev));
-    if (dev == g_fast_attr_device) return 0;
-    H2_CUDA_TRY(cudaFuncSetAttribute(k_up_own<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, up_own_smem_bytes(1, kUpMaxEntries)));
-    H2_CUDA_TRY(cudaFuncSetAttribute(k_up_own<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, up_own_smem_bytes(2, kUpMaxEntries)));
-    H2_CUDA_TRY(cudaFuncSetAttribute(k_up_own<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, up_own_smem_bytes(4, kUpMaxEntries)));
-    H2_CUDA_TRY(cudaFuncSetAttribute(k_down_own<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, down_own_smem_bytes(1, 8)));
-    H2_CUDA_TRY(cudaFuncSetAttribute(k_down_own<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, down_own_smem_bytes(2, 8)));
-    H2_CUDA_TRY(cudaFuncSetAttribute(k_down_own<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, down_own_smem_bytes(4, 8)));
-    H2_CUDA_TRY(cudaFuncSetAttribute(k_down_kron<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, down_kron_smem_bytes(1, 8)));
-    H2_CUDA_TRY(cudaFuncSetAttribute(k_down_kron<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, down_kron_smem_bytes(2, 8)));
-    H2_CUDA_TRY(cudaFuncSetAttribute(k_down_kron<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, down_kron_smem_bytes(4, 8)));
-    g_fast_attr_device = dev;
-    return 0;
-}
-
 struct PhaseMarks {
     h2_matrix* A;
     cudaStream_t st;
@@ -1554,6 +793,7 @@ int run_chain(h2_matrix* A, const MatData& D, double alpha, const double* X, int
 }
 
 size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
+int pad4(int x) { return (x + 3) & ~3; }
 
 
 
@@ -1599,29 +839,32 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
     for (int c0 = 0; c0 < m; c0 += 64) {
         const int mc = std::min(64, m - c0);
         const int R = round16(2 * mc);
-        const size_t bXp = align_up((size_t)n * mc * 4), bC = align_up((size_t)nc * k * mc * 4);
         const size_t bXcm = align_up((size_t)R * D.xk_total * es), bAct = align_up((size_t)nc * R * KP * es);
         // The variant of this column chunk: the autotuner's choice, else the built-in
-        // rule (the tensor-core transfer passes where the CUDA-core subtree passes do
-        // not apply).  The tensor-core transfer passes are FP32 only, and not used
+        // rule (the tensor-core transfer passes where the lists of pairs do not
+        // apply).  The tensor-core transfer passes are FP32 only, and not used
         // inside a stream capture, whose concurrent branches could keep some of their
         // CTAs from being resident.
         const Tune tn = A->tune[kind == 0 ? 1 : 0][column_class(mc)];
         const int stg = tn.stages;
-        const bool fast = A->f32.Et && k % 8 == 0 && k <= 64 && mc % 4 == 0 && A->T.leaf_size <= 64;
+        // the transfer passes as lists of pairs (q = 2, 3, 4), with the columns padded to
+        // a multiple of 4
+        const bool fast = A->pairs_built && A->use_kron;
         bool want_flow = !fast;
         if (tn.path == kPathTcOwn || tn.path == kPathTcHybrid) want_flow = false;
         if (tn.path == kPathTcFlow || tn.path == kPathTcFused) want_flow = true;
         if (A->use_flow >= 0) want_flow = A->use_flow == 1;
         const bool capturing = stream_capture_active(st);
         const bool flow = kind == 1 && D.flow && want_flow && !capturing && !cx;
-        // hybrid: the subtree passes stop at the upward cut, and the clusters above it
+        // hybrid: the upward lists stop at their first cut, and the clusters above it
         // are transfer items of the coupling launch (k_tc_gemm<4, KIND>), which waits
         // for them only where a coupling reads them
         bool want_hybrid = tn.path == kPathTcHybrid || (tn.path == kPathDefault && D.h_default);
         if (A->use_hybrid >= 0) want_hybrid = A->use_hybrid == 1;
         const bool lists = kind == 1 ? D.hybrid : D.hybrid_bf16;
         const bool hybrid = fast && !flow && !trans && !mf && !cx && lists && want_hybrid && !capturing;
+        const int ml = fast && !flow ? pad4(mc) : mc;  // columns of the coefficient blocks and of Z
+        const size_t bXp = align_up((size_t)n * ml * 4), bC = align_up((size_t)nc * k * ml * 4);
         int rc = ensure_workspace(A, bXp + 2 * bC + bXcm + 3 * bAct, st);
         if (rc) return rc;
         char* base = (char*)A->ws.base;
@@ -1635,31 +878,26 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
         const unsigned gy = (unsigned)((mc + NT - 1) / NT), gzk = (unsigned)((k + MT - 1) / MT);
         PhaseMarks marks(A, st);
         marks.mark();
-        // the subtree passes' arrival counters and task counters, and the hybrid
-        // launch's ready flags, are zeroed by the gather
-        const bool reset_in_gather = fast && !flow && sbc.claim2;
-        {
+        const int32_t* zid = trans ? D.ct_zero : D.c_zero;
+        const int nzid = trans ? D.ct_nzero : D.c_nzero;
+        if (fast && !flow) {
+            // one chain of launches: gather and leaves, then the upward pass (the leaves'
+            // launch also clears the hybrid launch's ready flags and ŷ of the clusters
+            // without couplings)
+            if ((rc = launch_forward(A, X + c0, ldx, mc, ml, xhat, xcm, Xcm, R, es, hybrid, sbc.fflag,
+                                     hybrid ? (int)nc : 0, zid, nzid, yhat, st)))
+                return rc;
+        } else {
             const int64_t total = n * mc;
             const unsigned g = (unsigned)std::min<int64_t>((total + 255) / 256, 152 * 32);
-            // claim2 follows the claim counters in the same allocation: zero them all
-            // with the hybrid pass (no climb, so nothing writes ŷ before the coupling
-            // launch) also ŷ of the clusters without couplings
-            if (reset_in_gather)
-                k_gather<float><<<g, 256, 0, st>>>(X + c0, ldx, A->d_perm, n, mc, Xp, sbc.cnt, (int)nc, sbc.claim,
-                                                   (int)(sbc.claim2 - sbc.claim) + 1, hybrid ? sbc.fflag : nullptr,
-                                                   hybrid ? (int)nc : 0, hybrid ? D.c_zero : nullptr,
-                                                   hybrid ? D.c_nzero : 0, yhat, k, mc, mc);
-            else
-                k_gather<float><<<g, 256, 0, st>>>(X + c0, ldx, A->d_perm, n, mc, Xp);
+            k_gather<float><<<g, 256, 0, st>>>(X + c0, ldx, A->d_perm, n, mc, Xp);
             H2_LAUNCH_CHECK();
         }
-        // (fast: the subtree-owning CUDA-core transfer passes apply, rows of 16-byte
-        // multiples; they also write the split tiles of X (leaves), x̂ and leaf ŷ)
+        // (the lists of pairs also write the split tiles of X (leaves), x̂ and leaf ŷ)
         if ((!fast || flow) &&
             (rc = launch_pack_act(Xp, mc, NL, nullptr, D.leaf_base, D.leaf_kdim, 0, D.xkoff, 0, mc, R, Xcm, es, st)))
             return rc;
         marks.mark();
-        const int fcn = mc <= 16 ? 1 : (mc <= 32 ? 2 : 4);
         if (flow) {
             // Both transfer passes on the tensor cores.  With A (and the stored
             // couplings) the upward pass shares one launch with the coupling phase
@@ -1763,32 +1001,14 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
                 lp.ldc = mc;
                 if ((rc = launch_tc_gemm(1, 1, lp, st, stg))) return rc;
             }
-            const int64_t total = n * mc;
-            const unsigned g = (unsigned)std::min<int64_t>((total + 255) / 256, 152 * 32);
             if ((rc = wait_y_staged(A->ws, st))) return rc;
-            k_scatter_y<<<g, 256, 0, st>>>(Xp, mc, A->d_perm, n, mc, X + c0, ldx, Y + c0, ldy, alpha, A->sigma,
-                                           overwrite ? 1 : 0);
+            launch_scatter_y(Xp, mc, A->d_perm, n, mc, X + c0, ldx, Y + c0, ldy, alpha, A->sigma, overwrite, st);
             H2_LAUNCH_CHECK();
             marks.mark();
             if ((rc = marks.commit())) return rc;
             continue;
         }
         if (fast) {
-            if ((rc = fast_prepare())) return rc;
-            const PackOut pk{xcm, Xcm, D.xkoff, KP, R, es};
-            const int usm = up_own_smem_bytes(fcn, A->up_entries);
-            const unsigned g = (unsigned)std::min(A->up_ntasks, 152 * std::max(1, (227 * 1024) / (usm + 2048)));
-            if (!reset_in_gather) {
-                H2_CUDA_TRY(cudaMemsetAsync(sbc.cnt, 0, (size_t)nc * sizeof(unsigned), st));
-                H2_CUDA_TRY(cudaMemsetAsync(sbc.claim, 0, sizeof(unsigned), st));
-            }
-            const int climb = hybrid ? 0 : 1;
-            // q = 4: the inner steps and the climb apply E_sᵀ as Kronecker products
-            const float* ukron = (k == 64 && A->use_kron) ? (const float*)A->f32.kron : nullptr;
-            if (fcn == 1) k_up_own<1><<<g, 64, usm, st>>>(A->d_up_task_ptr, A->up_ntasks, A->d_up_steps, A->d_cl_off, A->d_cl_size, A->d_parent, A->d_son0, A->d_son1, V, E, Xp, xhat, yhat, sbc.cnt, sbc.claim, sbc.err, A->up_entries, k, mc, pk, climb, ukron);
-            else if (fcn == 2) k_up_own<2><<<g, 128, usm, st>>>(A->d_up_task_ptr, A->up_ntasks, A->d_up_steps, A->d_cl_off, A->d_cl_size, A->d_parent, A->d_son0, A->d_son1, V, E, Xp, xhat, yhat, sbc.cnt, sbc.claim, sbc.err, A->up_entries, k, mc, pk, climb, ukron);
-            else k_up_own<4><<<g, 256, usm, st>>>(A->d_up_task_ptr, A->up_ntasks, A->d_up_steps, A->d_cl_off, A->d_cl_size, A->d_parent, A->d_son0, A->d_son1, V, E, Xp, xhat, yhat, sbc.cnt, sbc.claim, sbc.err, A->up_entries, k, mc, pk, climb, ukron);
-            H2_LAUNCH_CHECK();
             marks.mark();
             marks.mark();
         } else if ((rc = forward_pass<float, RM, CN>(A, V, E, Xp, xhat, mc, gy, gzk, st, sbc, marks))) {
@@ -1800,10 +1020,7 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
         // Aᵀ: the coupling runs over column clusters with S_bᵀ, the leaf phase over
         // column leaves with G_bᵀ (tiles and lists of build_tc_transposed)
         const uint8_t* bmat = trans ? (kind == 0 ? D.matT : D.matT32) : (kind == 0 ? D.mat : D.mat32);
-        if (!(reset_in_gather && hybrid) &&
-            (rc = launch_zero_clusters(trans ? D.ct_zero : D.c_zero, trans ? D.ct_nzero : D.c_nzero, yhat, k, mc, mc,
-                                       st)))
-            return rc;
+        if (!fast && (rc = launch_zero_clusters(zid, nzid, yhat, k, mc, mc, st))) return rc;
         TcGemmParams cp{};
         cp.n_items = trans ? D.ct_nitems : D.c_nitems;
         cp.items = trans ? D.ct_items : D.c_items;
@@ -1812,10 +1029,10 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
         cp.act1 = xcm;
         cp.bmat = bmat;
         cp.R = R;
-        cp.mc = mc;
+        cp.mc = ml;
         cp.yhat = yhat;
         cp.k = k;
-        cp.ldc = mc;
+        cp.ldc = ml;
         cp.err = A->err_dev;
         cp.nodes = D.nodes4;
         cp.KP = KP;
@@ -1827,7 +1044,6 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
             cp.out_act = xcm;  // the transfer items' split tiles
             cp.flag = sbc.fflag;
             cp.epoch = 1;
-            if (!reset_in_gather) H2_CUDA_TRY(cudaMemsetAsync(sbc.fflag, 0, (size_t)nc * sizeof(int), st));
         }
         marks.kernel_begin();
         if (cp.n_items > 0 &&
@@ -1835,39 +1051,13 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
             return rc;
         marks.kernel_end();
         marks.mark();
-        bool leaf_y_packed = false;
         if (fast) {
-            const int n_items = (int)A->down_ptr[A->depth + 1];
-            if (n_items > 0) {
-                const PackOut pk{ycm, nullptr, nullptr, KP, R, es};
-                leaf_y_packed = true;
-                // the task counter of this pass: claim2, zeroed by the gather (else claim again)
-                unsigned* dclaim = reset_in_gather ? sbc.claim2 : sbc.claim;
-                if (!reset_in_gather) H2_CUDA_TRY(cudaMemsetAsync(sbc.claim, 0, sizeof(unsigned), st));
-                const float* Et = (const float*)A->f32.Et;
-                const int smem = down_own_smem_bytes(fcn, A->dn_entries);
-                const unsigned g = (unsigned)std::min(A->dn_ntasks, 152 * std::max(1, (227 * 1024) / (smem + 4096)));
-                const float* kron = (const float*)A->f32.kron;
-                if (kron && k == 64 && A->use_kron && fcn >= 2) {
-                    // q = 4: each step as three 4×4 mode products (E_c = F_z ⊗ F_y ⊗ F_x); with
-                    // 16 columns or fewer half its threads would idle, and the dense pass is faster
-                    const int ksm = down_kron_smem_bytes(fcn, A->dn_entries);
-                    const unsigned gk =
-                        (unsigned)std::min(A->dn_ntasks, 152 * std::max(1, (227 * 1024) / (ksm + 4096)));
-                    if (fcn == 1) k_down_kron<1><<<gk, 128, ksm, st>>>(A->d_dn_task_ptr, A->dn_ntasks, A->d_dn_steps, kron, yhat, dclaim, sbc.err, mc, pk);
-                    else if (fcn == 2) k_down_kron<2><<<gk, 128, ksm, st>>>(A->d_dn_task_ptr, A->dn_ntasks, A->d_dn_steps, kron, yhat, dclaim, sbc.err, mc, pk);
-                    else k_down_kron<4><<<gk, 128, ksm, st>>>(A->d_dn_task_ptr, A->dn_ntasks, A->d_dn_steps, kron, yhat, dclaim, sbc.err, mc, pk);
-                } else if (fcn == 1) k_down_own<1><<<g, 128, smem, st>>>(A->d_dn_task_ptr, A->dn_ntasks, A->d_dn_steps, Et, yhat, dclaim, sbc.err, k, mc, pk);
-                else if (fcn == 2) k_down_own<2><<<g, 128, smem, st>>>(A->d_dn_task_ptr, A->dn_ntasks, A->d_dn_steps, Et, yhat, dclaim, sbc.err, k, mc, pk);
-                else k_down_own<4><<<g, 128, smem, st>>>(A->d_dn_task_ptr, A->dn_ntasks, A->d_dn_steps, Et, yhat, dclaim, sbc.err, k, mc, pk);
-                H2_LAUNCH_CHECK();
-            }
-        } else if ((rc = backward_pass<float, RM, CN>(A, E, yhat, mc, gy, gzk, st, sbc))) {
-            return rc;
+            if ((rc = launch_backward(A, yhat, ycm, ml, R, es, st))) return rc;
+        } else {
+            if ((rc = backward_pass<float, RM, CN>(A, E, yhat, mc, gy, gzk, st, sbc))) return rc;
+            if ((rc = launch_pack_act(yhat, mc, NL, A->d_leaves, nullptr, nullptr, k, nullptr, KP, mc, R, ycm, es, st)))
+                return rc;
         }
-        if (!leaf_y_packed &&
-            (rc = launch_pack_act(yhat, mc, NL, A->d_leaves, nullptr, nullptr, k, nullptr, KP, mc, R, ycm, es, st)))
-            return rc;
         marks.mark();
         TcGemmParams lp{};
         lp.n_items = trans ? D.lt_nitems : D.l_nitems;
@@ -1877,13 +1067,13 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
         lp.act1 = ycm;
         lp.bmat = bmat;
         lp.R = R;
-        lp.mc = mc;
+        lp.mc = ml;
         lp.leaves = A->d_leaves;
         lp.cl_off = A->d_cl_off;
         lp.cl_size = A->d_cl_size;
         lp.err = A->err_dev;
         lp.zp = Xp;  // the gathered FP32 X is no longer read after the forward pass and its packing
-        lp.ldc = mc;
+        lp.ldc = ml;
         lp.cplx = cx ? 1 : 0;
         if ((rc = launch_tc_gemm(1, kind, lp, st, stg))) return rc;
         {
@@ -1891,11 +1081,10 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
             const unsigned g = (unsigned)std::min<int64_t>((total + 255) / 256, 152 * 32);
             if ((rc = wait_y_staged(A->ws, st))) return rc;
             if (cx)
-                k_scatter_yc<<<g, 256, 0, st>>>(Xp, mc, A->d_perm, n, mc, X + c0, ldx, Y + c0, ldy, alpha, *alpha_im,
+                k_scatter_yc<<<g, 256, 0, st>>>(Xp, ml, A->d_perm, n, mc, X + c0, ldx, Y + c0, ldy, alpha, *alpha_im,
                                                 A->sigma, overwrite ? 1 : 0);
             else
-                k_scatter_y<<<g, 256, 0, st>>>(Xp, mc, A->d_perm, n, mc, X + c0, ldx, Y + c0, ldy, alpha, A->sigma,
-                                               overwrite ? 1 : 0);
+                launch_scatter_y(Xp, ml, A->d_perm, n, mc, X + c0, ldx, Y + c0, ldy, alpha, A->sigma, overwrite, st);
             H2_LAUNCH_CHECK();
         }
         marks.mark();
@@ -1943,20 +1132,18 @@ int ensure_sync(h2_matrix* A, int64_t tiles, cudaStream_t st, SyncBufs* sb) {
         A->sync_cnt = nullptr;
         A->sync_tiles = 0;
         const size_t per = (size_t)A->nc * tiles;
-        // claim: `tiles` counters and one more (the tensor-core chain's downward pass)
-        const size_t bytes = per * (sizeof(unsigned) + sizeof(int)) + (tiles + 1) * sizeof(unsigned) +
+        const size_t bytes = per * (sizeof(unsigned) + sizeof(int)) + tiles * sizeof(unsigned) +
                              2 * (size_t)A->nc * sizeof(int);
         H2_CUDA_TRY(cudaMalloc(&A->sync_cnt, bytes));
         H2_CUDA_TRY(cudaMemsetAsync(A->sync_cnt, 0, bytes, st));
         A->sync_flag = (int*)(A->sync_cnt + per);
         A->sync_claim = (unsigned*)(A->sync_flag + per);
-        A->sync_fflag = (int*)(A->sync_claim + tiles + 1);
+        A->sync_fflag = (int*)(A->sync_claim + tiles);
         A->sync_tiles = tiles;
     }
     sb->cnt = A->sync_cnt;
     sb->flag = A->sync_flag;
     sb->claim = A->sync_claim;
-    sb->claim2 = A->sync_claim + A->sync_tiles;
     sb->fflag = A->sync_fflag;
     sb->epoch = 1;  // flags are cleared before every downward pass
     sb->err = A->err_dev;
@@ -2058,7 +1245,7 @@ int product_prepare(h2_matrix* A, int64_t m, int32_t dtype, cudaStream_t st) {
         const int es = dtype == H2_BF16 ? 2 : 4;
         const int mc = (int)std::min<int64_t>(64, m);
         const int R = round16(2 * mc);
-        need = align_up((size_t)n * mc * 4) + 2 * align_up((size_t)nc * k * mc * 4) +
+        need = align_up((size_t)n * pad4(mc) * 4) + 2 * align_up((size_t)nc * k * pad4(mc) * 4) +
                align_up((size_t)R * D.xk_total * es) + 3 * align_up((size_t)nc * R * D.KP * es);
         if ((rc = tc_prepare())) return rc;
     } else {
@@ -2118,11 +1305,7 @@ int flow_pre(h2_matrix* A, const double* X, int64_t ldx, const FlowBufs& fb, cud
 // After them: Y += α(Z + σX) in the caller's order (Y = α(Z + σX) with overwrite).
 int flow_post(h2_matrix* A, double alpha, const double* X, int64_t ldx, double* Y, int64_t ldy, const FlowBufs& fb,
               bool overwrite, cudaStream_t st) {
-    const int64_t n = A->n;
-    const int mc = fb.mc;
-    const int64_t total = n * mc;
-    const unsigned g = (unsigned)std::min<int64_t>((total + 255) / 256, 152 * 32);
-    k_scatter_y<<<g, 256, 0, st>>>(fb.Xp, mc, A->d_perm, n, mc, X, ldx, Y, ldy, alpha, A->sigma, overwrite ? 1 : 0);
+    launch_scatter_y(fb.Xp, fb.mc, A->d_perm, A->n, fb.mc, X, ldx, Y, ldy, alpha, A->sigma, overwrite, st);
     H2_LAUNCH_CHECK();
     return 0;
 }
