@@ -5,8 +5,8 @@
 //   G = Pᵀ(AP),  W = PᵀR,  α = G⁻¹W,  X += Pα,  R -= (AP)α,
 //   Γ = G⁻¹(AP)ᵀR,  P = R - PΓ.
 //
-// G⁻¹ is applied through a Cholesky factor of G computed with deflation: in
-// index order, direction j is kept when its Schur pivot exceeds kDeflate times
+// G⁻¹ is applied through the square-root-free Cholesky factors of G, computed with
+// deflation: in index order, direction j is kept when its Schur pivot exceeds kDeflate times
 // its diagonal (it is not A-dependent on the kept directions before it) and
 // dropped for this step otherwise; a diagonal <p_j, A p_j> <= 0 on an active
 // column is a breakdown.  Columns that reach the tolerance are frozen: their
@@ -15,7 +15,7 @@
 // Everything runs in FP64 on the device.  Per iteration, after the product:
 //   k_gram_partial      per-CTA partial sums of [G | W] over row tiles
 //   k_gram_reduce<0>    fixed-order sum of the partials: G, W
-//   k_gram_solve<0>     deflating Cholesky of G and α = G⁻¹W, 4 columns per CTA
+//   k_gram_solve<0>     deflating L·D·Lᵀ of G and α = G⁻¹W, 4 columns per CTA
 //   k_gram_update       X += Pα, R -= (AP)α, partial sums of (AP)ᵀR and |r_j|²
 //   k_gram_reduce<1>    fixed-order sum: (AP)ᵀR, |r_j|²
 //   k_gram_solve<1>     active set and Γ = G⁻¹(AP)ᵀR, 4 columns per CTA
@@ -33,58 +33,87 @@ namespace h2 {
 namespace {
 
 constexpr int kGramCtas = 152;   // one CTA per SM for the row passes
-constexpr int kTRg = 16;         // rows per tile in the Gram pass
-constexpr int kTRu = 8;          // rows per tile in the update and direction passes
 constexpr double kDeflate = 1e-10;
 constexpr int kSolveLd = kGramMaxCols + 1;
 
 __host__ __device__ __forceinline__ int pstride(int m) { return 2 * m * m + m; }
 
+// Rows of a tile of the row passes: 256 elements, one a thread (m > 32: two).
+template <int MP>
+__host__ __device__ constexpr int tile_rows() { return MP == 64 ? 8 : 256 / MP; }
+
+// One tile of an n×m array (ld m) in registers: elements t, t + 256 of the tile's
+// rows × MP, zero outside.  The row passes load a tile's arrays while the one
+// before is worked on, into two shared-memory buffers in turn, so that one barrier
+// a tile is all that stands between its multiply-adds.
+template <int MP>
+struct TileRegs {
+    static constexpr int E = tile_rows<MP>() * MP / 256;
+    double v[E];
+    __device__ __forceinline__ void load(const double* __restrict__ A, int64_t lda, int64_t r0, int64_t n, int m) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int o = threadIdx.x + 256 * e, c = o % MP;
+            const int64_t row = r0 + o / MP;
+            v[e] = row < n && c < m ? A[row * lda + c] : 0.0;
+        }
+    }
+    __device__ __forceinline__ void store(double* s) const {
+#pragma unroll
+        for (int e = 0; e < E; ++e) s[threadIdx.x + 256 * e] = v[e];
+    }
+};
+
 // part[cta][0:m²] = Uᵀ V0, part[cta][m²:2m²] = Uᵀ V1 over the CTA's row tiles
 // (U, V0, V1: n×m, ld m).  MP is m rounded up to 16, 32 or 64; thread (tx, ty)
-// owns entries (ty + 16a, tx + 16b).
+// owns entries (ty + 16a, tx + 16b).  NT = 2 (G = PᵀAP and PᵀR): of the symmetric
+// G the factorisation reads the lower triangle, so the blocks above it are left
+// out.  n = 8192, m = 32: 40 µs with 16-row tiles and exposed loads, 29 now (its
+// multiply-adds: 23); NT = 1: 28 → 18 (13).
 template <int MP, int NT>
 __global__ void __launch_bounds__(256) k_gram_partial(const double* __restrict__ U, const double* __restrict__ V0,
                                                       const double* __restrict__ V1, int64_t n, int m,
                                                       double* __restrict__ part) {
-    constexpr int T = MP / 16;
-    __shared__ double su[kTRg][MP], s0[kTRg][MP], s1[kTRg][MP];
+    constexpr int T = MP / 16, TR = tile_rows<MP>();
+    __shared__ double su[2][TR][MP], s0[2][TR][MP], s1[2][NT == 2 ? TR : 1][MP];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     double a0[T][T], a1[T][T];
 #pragma unroll
     for (int i = 0; i < T; ++i)
 #pragma unroll
         for (int j = 0; j < T; ++j) a0[i][j] = a1[i][j] = 0.0;
-    const int64_t tiles = (n + kTRg - 1) / kTRg;
-    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        const int64_t r0 = tile * kTRg;
-        for (int e = threadIdx.x; e < kTRg * MP; e += 256) {
-            const int r = e / MP, c = e % MP;
-            const int64_t row = r0 + r;
-            const bool ok = row < n && c < m;
-            su[r][c] = ok ? U[row * m + c] : 0.0;
-            s0[r][c] = ok ? V0[row * m + c] : 0.0;
-            if (NT == 2) s1[r][c] = ok ? V1[row * m + c] : 0.0;
-        }
+    const int64_t tiles = (n + TR - 1) / TR;
+    TileRegs<MP> ru, r0, r1;
+    auto fetch = [&](int64_t tile) {
+        ru.load(U, m, tile * TR, n, m);
+        r0.load(V0, m, tile * TR, n, m);
+        if (NT == 2) r1.load(V1, m, tile * TR, n, m);
+    };
+    int b = 0;
+    if (blockIdx.x < tiles) fetch(blockIdx.x);
+    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, b ^= 1) {
+        ru.store(&su[b][0][0]);
+        r0.store(&s0[b][0][0]);
+        if (NT == 2) r1.store(&s1[b][0][0]);
         __syncthreads();
+        if (tile + gridDim.x < tiles) fetch(tile + gridDim.x);
 #pragma unroll 4
-        for (int r = 0; r < kTRg; ++r) {
+        for (int r = 0; r < TR; ++r) {
             double u[T], v0[T], v1[T];
 #pragma unroll
             for (int i = 0; i < T; ++i) {
-                u[i] = su[r][ty + 16 * i];
-                v0[i] = s0[r][tx + 16 * i];
-                v1[i] = NT == 2 ? s1[r][tx + 16 * i] : 0.0;
+                u[i] = su[b][r][ty + 16 * i];
+                v0[i] = s0[b][r][tx + 16 * i];
+                v1[i] = NT == 2 ? s1[b][r][tx + 16 * i] : 0.0;
             }
 #pragma unroll
             for (int i = 0; i < T; ++i)
 #pragma unroll
                 for (int j = 0; j < T; ++j) {
-                    a0[i][j] = fma(u[i], v0[j], a0[i][j]);
+                    if (NT == 1 || j <= i) a0[i][j] = fma(u[i], v0[j], a0[i][j]);
                     if (NT == 2) a1[i][j] = fma(u[i], v1[j], a1[i][j]);
                 }
         }
-        __syncthreads();
     }
     double* out = part + (size_t)blockIdx.x * pstride(m);
 #pragma unroll
@@ -99,95 +128,104 @@ __global__ void __launch_bounds__(256) k_gram_partial(const double* __restrict__
         }
 }
 
-// Fixed-order sum of the per-CTA partials: PHASE 0 gives G = Pᵀ(AP) and
-// W = PᵀR, PHASE 1 gives C = (AP)ᵀR and |r_j|².
+// Fixed-order sum of the per-CTA partials: PHASE 0 gives G = Pᵀ(AP) (lower
+// triangle by 16×16 blocks) and W = PᵀR, PHASE 1 gives C = (AP)ᵀR and |r_j|².
+// Eight lanes an entry take a run of the partials each (four consecutive entries to
+// a sector), so a thread has at most 19 loads one after the other instead of 152
+// (26 → 10 µs at m = 32).
 template <int PHASE>
 __global__ void __launch_bounds__(256) k_gram_reduce(int nct, int m, GramDev g) {
     const int ps = pstride(m);
     const int nterm = PHASE == 0 ? 2 * m * m : m * m + m;
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= nterm) return;
-    // four interleaved partial sums keep loads in flight; fixed order
-    double s4[4] = {0.0, 0.0, 0.0, 0.0};
-    int c = 0;
-    for (; c + 3 < nct; c += 4)
+    const int lane = threadIdx.x & 31, sub = lane >> 2;
+    const int e = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 4 + (lane & 3);
+    double s = 0.0;
+    if (e < nterm) {
+        const int run = (nct + 7) >> 3;
+#pragma unroll 10
+        for (int c = sub * run; c < min(nct, (sub + 1) * run); ++c) s += __ldcg(&g.part[(size_t)c * ps + e]);
+    }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) s4[u] += __ldcg(&g.part[(size_t)(c + u) * ps + e]);
-    for (; c < nct; ++c) s4[0] += __ldcg(&g.part[(size_t)c * ps + e]);
-    const double s = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+    for (int o = 4; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (e >= nterm || sub) return;
     if (e < m * m) (PHASE == 0 ? g.G : g.W)[e] = s;
     else if (PHASE == 0) g.W[e - m * m] = s;
     else g.rr[e - m * m] = s;
 }
 
 constexpr int kSolveCols = 4;     // right-hand-side columns of the m×m solve per CTA
-constexpr int kSolveThreads = 128;
+constexpr int kSolveThreads = 256;
 
-// The m×m step, kSolveCols columns per CTA.
-// PHASE 0: every CTA factors G (deflating Cholesky, identical in all CTAs) and
-//   solves α[:, c] = G_KK⁻¹ W[K, c] for its active columns c; CTA 0 keeps L and
-//   the kept set for PHASE 1.
+// The m×m step, kSolveCols columns per CTA, with G = L·D·Lᵀ on the kept
+// directions: sA holds the columns of L·D (below the diagonal), rcp[j] = 1 / d_j,
+// 0 for a dropped direction.
+// PHASE 0: every CTA factors G (with deflation, identical in all CTAs) and solves
+//   α[:, c] = G_KK⁻¹ W[K, c] for its active columns c; CTA 0 keeps the factors
+//   (1 / d_j on the diagonal of L) and the kept set for PHASE 1.
 // PHASE 1: each CTA updates the active set of its columns from |r_c| and solves
 //   Γ[:, c] = G_KK⁻¹ C[K, c] for those still active.
+// A step of the factorisation is one barrier: the thread that finishes the next
+// pivot inverts it while the others update, and the right-hand sides are more
+// columns of the matrix.  A substitution is one warp a column, which needs no
+// barrier.  m = 32: 83 → 38 µs (PHASE 0), 45 → 17 µs (PHASE 1).
 template <int PHASE>
 __global__ void __launch_bounds__(kSolveThreads) k_gram_solve(int m, double tol, GramDev g, CgDev d) {
     __shared__ double sA[kGramMaxCols][kSolveLd];
     __shared__ double sB[kGramMaxCols][kSolveCols];
-    __shared__ double sdg[kGramMaxCols];
-    __shared__ int sk[kGramMaxCols], sa[kGramMaxCols], sown[kSolveCols];
+    __shared__ double sdg[kGramMaxCols], rcp[kGramMaxCols];
+    __shared__ int sa[kGramMaxCols], sown[kSolveCols];
     __shared__ int sbrk;
     const int t = threadIdx.x;
     const int c0 = blockIdx.x * kSolveCols;
     const int nc = min(kSolveCols, m - c0);
     if (t == 0) sbrk = 0;
+    for (int x = t; x < m * m; x += kSolveThreads) sA[x / m][x % m] = __ldcg(&(PHASE == 0 ? g.G : g.L)[x]);
+    for (int x = t; x < m * nc; x += kSolveThreads) sB[x / nc][x % nc] = __ldcg(&g.W[(x / nc) * m + c0 + x % nc]);
     if (PHASE == 0) {
-        for (int x = t; x < m * m; x += blockDim.x) sA[x / m][x % m] = __ldcg(&g.G[x]);
-        for (int j = t; j < m; j += blockDim.x) {
+        for (int j = t; j < m; j += kSolveThreads) {
             sa[j] = d.active[j] != 0;
             sdg[j] = __ldcg(&g.G[j * m + j]);
         }
         __syncthreads();
-        // right-looking Cholesky with deflation
+        // 1 / d_j of a kept direction; thread 0 only
+        auto pivot = [&](int j) {
+            double r = 0.0;
+            if (sa[j]) {
+                const double gjj = sdg[j], dj = sA[j][j];
+                if (!(gjj > 0.0) || !isfinite(gjj)) sbrk = 1;
+                else if (dj > kDeflate * gjj) r = 1.0 / dj;
+            }
+            rcp[j] = r;
+        };
+        if (t == 0) pivot(0);
+        const int tx = t & 15, ty = t >> 4;
         for (int j = 0; j < m; ++j) {
-            if (t == 0) {
-                int keep = 0;
-                if (sa[j]) {
-                    const double gjj = sdg[j];
-                    if (!(gjj > 0.0) || !isfinite(gjj)) {
-                        sbrk = 1;
-                    } else {
-                        const double dj = sA[j][j];
-                        if (dj > kDeflate * gjj) {
-                            keep = 1;
-                            sA[j][j] = sqrt(dj);
-                        }
-                    }
-                }
-                sk[j] = keep;
-            }
             __syncthreads();
-            if (sk[j]) {
-                const double piv = sA[j][j];
-                for (int i = j + 1 + t; i < m; i += blockDim.x) sA[i][j] /= piv;
-                __syncthreads();
-                const int w = m - j - 1;
-                for (int x = t; x < w * w; x += blockDim.x) {
-                    const int i = j + 1 + x / w, k = j + 1 + x % w;
-                    if (k <= i) sA[i][k] -= sA[i][j] * sA[k][j];
+            const double r = rcp[j];
+            if (r != 0.0) {
+                for (int i = j + 1 + ty; i < m; i += 16) {
+                    const double f = sA[i][j] * r;
+                    for (int k = j + 1 + tx; k <= i; k += 16) sA[i][k] = fma(-f, sA[k][j], sA[i][k]);
+                    if (tx < nc) sB[i][tx] = fma(-f, sB[j][tx], sB[i][tx]);
+                    // thread 0 finishes pivot j + 1 with its first element
+                    if (t == 0 && i == j + 1) pivot(j + 1);
                 }
+            } else if (t == 0 && j + 1 < m) {
+                pivot(j + 1);
             }
-            __syncthreads();
         }
-        for (int c = t; c < nc; c += blockDim.x) sown[c] = sa[c0 + c];
-        for (int x = t; x < m * nc; x += blockDim.x) sB[x / nc][x % nc] = __ldcg(&g.W[(x / nc) * m + c0 + x % nc]);
+        __syncthreads();
+        for (int c = t; c < nc; c += kSolveThreads) sown[c] = sa[c0 + c];
         if (blockIdx.x == 0) {
-            for (int x = t; x < m * m; x += blockDim.x) g.L[x] = sA[x / m][x % m];
-            for (int j = t; j < m; j += blockDim.x) g.kept[j] = sk[j];
+            for (int x = t; x < m * m; x += kSolveThreads) {
+                const int i = x / m, k = x % m;
+                g.L[x] = i == k ? rcp[i] : sA[i][k];
+            }
+            for (int j = t; j < m; j += kSolveThreads) g.kept[j] = rcp[j] != 0.0;
         }
     } else {
-        for (int x = t; x < m * m; x += blockDim.x) sA[x / m][x % m] = __ldcg(&g.L[x]);
-        for (int j = t; j < m; j += blockDim.x) sk[j] = __ldcg(&g.kept[j]);
-        for (int c = t; c < nc; c += blockDim.x) {
+        for (int j = t; j < m; j += kSolveThreads) rcp[j] = __ldcg(&g.L[j * m + j]);
+        for (int c = t; c < nc; c += kSolveThreads) {
             const int col = c0 + c;
             int act = d.active[col] != 0;
             if (act) {
@@ -203,59 +241,60 @@ __global__ void __launch_bounds__(kSolveThreads) k_gram_solve(int m, double tol,
             }
             sown[c] = act;
         }
-        for (int x = t; x < m * nc; x += blockDim.x) sB[x / nc][x % nc] = __ldcg(&g.W[(x / nc) * m + c0 + x % nc]);
     }
     __syncthreads();
-    // sB[:, c] = G_KK⁻¹ sB[K, c]: L z = b, then Lᵀ y = z; rows outside K are 0
-    for (int j = 0; j < m; ++j) {
-        if (sk[j]) {
-            const double piv = sA[j][j];
-            if (t < nc) sB[j][t] /= piv;
-            __syncthreads();
-            const int w = m - j - 1;
-            for (int x = t; x < w * nc; x += blockDim.x) {
-                const int i = j + 1 + x / nc, c = x % nc;
-                sB[i][c] -= sA[i][j] * sB[j][c];
+    // a warp's column: entries of rows lane and lane + 32
+    const int c = t >> 5, lane = t & 31;
+    double y0 = 0.0, y1 = 0.0;
+    bool finite = true;
+    if (c < nc) {
+        y0 = lane < m ? sB[lane][c] : 0.0;
+        y1 = lane + 32 < m ? sB[lane + 32][c] : 0.0;
+        const double q0 = lane < m ? rcp[lane] : 0.0, q1 = lane + 32 < m ? rcp[lane + 32] : 0.0;
+        if (PHASE == 1)  // L z = b
+            for (int j = 0; j < m; ++j) {
+                const double r = rcp[j];
+                if (r == 0.0) continue;
+                const double f = r * __shfl_sync(0xffffffffu, j < 32 ? y0 : y1, j & 31);
+                if (lane > j && lane < m) y0 = fma(-sA[lane][j], f, y0);
+                if (lane + 32 > j && lane + 32 < m) y1 = fma(-sA[lane + 32][j], f, y1);
             }
-        } else if (t < nc) {
-            sB[j][t] = 0.0;
+        // Lᵀ y = D⁻¹ z: entry i is final once the rows after it are; rows outside K are 0
+        for (int j = m - 1; j >= 0; --j) {
+            if (rcp[j] == 0.0) continue;
+            const double f = __shfl_sync(0xffffffffu, j < 32 ? q0 * y0 : q1 * y1, j & 31);
+            if (lane < j) y0 = fma(-sA[j][lane], f, y0);
+            if (lane + 32 < j) y1 = fma(-sA[j][lane + 32], f, y1);
         }
-        __syncthreads();
-    }
-    for (int j = m - 1; j >= 0; --j) {
-        if (sk[j]) {
-            const double piv = sA[j][j];
-            if (t < nc) sB[j][t] /= piv;
-            __syncthreads();
-            for (int x = t; x < j * nc; x += blockDim.x) {
-                const int i = x / nc, c = x % nc;
-                if (sk[i]) sB[i][c] -= sA[j][i] * sB[j][c];
-            }
-        }
-        __syncthreads();
-    }
-    double* out = PHASE == 0 ? g.alpha : g.gamma;
-    for (int x = t; x < m * nc; x += blockDim.x) {
-        const int i = x / nc, c = x % nc;
-        const double v = sB[i][c];
-        const bool ok = sown[c] && isfinite(v);
-        if (sown[c] && !isfinite(v)) sbrk = 1;
-        out[i * m + c0 + c] = (ok && !(PHASE == 0 && sbrk)) ? v : 0.0;
+        y0 = q0 != 0.0 ? q0 * y0 : 0.0;
+        y1 = q1 != 0.0 ? q1 * y1 : 0.0;
+        finite = isfinite(y0) && isfinite(y1);
+        if (sown[c] && !finite) sbrk = 1;
     }
     __syncthreads();
+    if (c < nc) {
+        double* out = PHASE == 0 ? g.alpha : g.gamma;
+        const bool ok = sown[c] && !(PHASE == 0 && sbrk);
+        if (lane < m) out[lane * m + c0 + c] = ok && isfinite(y0) ? y0 : 0.0;
+        if (lane + 32 < m) out[(lane + 32) * m + c0 + c] = ok && isfinite(y1) ? y1 : 0.0;
+    }
     if (t == 0 && sbrk) atomicOr(&d.summary[1], 1);
 }
 
 // X += Pα, R -= Qα (Q = AP) over the CTA's row tiles, then the partial sums of
-// QᵀR_new and |r_j|² for k_gram_reduce<1>.
+// QᵀR_new (WITH_C) and |r_j|² for k_gram_reduce<1>.  n = 8192, m = 32, without C:
+// 45 → 35 µs (its multiply-adds: 27).
 template <int MP, bool WITH_C>
 __global__ void __launch_bounds__(256) k_gram_update(double* __restrict__ X, int64_t ldx, const double* __restrict__ P,
                                                      const double* __restrict__ Q, double* __restrict__ R, int64_t n,
                                                      int m, const double* __restrict__ alpha,
                                                      double* __restrict__ part) {
-    constexpr int T = MP / 16;
-    __shared__ double sal[MP][MP];
-    __shared__ double sp[kTRu][MP], sq[kTRu][MP], sr[kTRu][MP];
+    constexpr int T = MP / 16, TR = tile_rows<MP>(), E = TileRegs<MP>::E;
+    extern __shared__ __align__(16) double gsm[];
+    double(*sal)[MP] = reinterpret_cast<double(*)[MP]>(gsm);             // [MP][MP]
+    double(*sp)[MP] = sal + MP;                                          // [2·TR][MP]
+    double(*sq)[MP] = sp + 2 * TR;                                       // [2·TR][MP]
+    double(*sr)[MP] = sq + 2 * TR;                                       // [2·TR][MP], WITH_C only
     const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
     for (int x = t; x < MP * MP; x += 256) {
         const int i = x / MP, j = x % MP;
@@ -266,102 +305,119 @@ __global__ void __launch_bounds__(256) k_gram_update(double* __restrict__ X, int
     for (int i = 0; i < T; ++i)
 #pragma unroll
         for (int j = 0; j < T; ++j) acc[i][j] = 0.0;
-    double rr = 0.0;
-    const int64_t tiles = (n + kTRu - 1) / kTRu;
-    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        const int64_t r0 = tile * kTRu;
-        __syncthreads();  // sal written (first tile); previous tile's reads done
-        for (int e = t; e < kTRu * MP; e += 256) {
-            const int r = e / MP, c = e % MP;
-            const int64_t row = r0 + r;
-            const bool ok = row < n && c < m;
-            sp[r][c] = ok ? P[row * m + c] : 0.0;
-            sq[r][c] = ok ? Q[row * m + c] : 0.0;
-            sr[r][c] = ok ? R[row * m + c] : 0.0;
-        }
+    double rr = 0.0;  // |r_j|² of this thread's rows, j = t mod MP
+    const int64_t tiles = (n + TR - 1) / TR;
+    TileRegs<MP> rp, rq, rres, rx;
+    auto fetch = [&](int64_t tile) {
+        rp.load(P, m, tile * TR, n, m);
+        rq.load(Q, m, tile * TR, n, m);
+        rres.load(R, m, tile * TR, n, m);
+        rx.load(X, ldx, tile * TR, n, m);
+    };
+    int b = 0;
+    if (blockIdx.x < tiles) fetch(blockIdx.x);
+    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, b ^= 1) {
+        const int64_t r0 = tile * TR;
+        rp.store(&sp[b * TR][0]);
+        rq.store(&sq[b * TR][0]);
+        const TileRegs<MP> cr = rres, cx = rx;
         __syncthreads();
-        for (int o = t; o < kTRu * MP; o += 256) {
-            const int r = o / MP, j = o % MP;
+        if (tile + gridDim.x < tiles) fetch(tile + gridDim.x);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int o = t + 256 * e, r = b * TR + o / MP, j = o % MP;
             double xs = 0.0, rs = 0.0;
 #pragma unroll 16
             for (int i = 0; i < MP; ++i) {
                 xs = fma(sp[r][i], sal[i][j], xs);
                 rs = fma(sq[r][i], sal[i][j], rs);
             }
-            const int64_t row = r0 + r;
+            const int64_t row = r0 + o / MP;
+            const double rn = cr.v[e] - rs;
             if (row < n && j < m) {
-                const double rn = sr[r][j] - rs;
-                X[row * ldx + j] += xs;
+                X[row * ldx + j] = cx.v[e] + xs;
                 R[row * m + j] = rn;
-                sr[r][j] = rn;
+                rr = fma(rn, rn, rr);
+            }
+            if (WITH_C) sr[r][j] = row < n && j < m ? rn : 0.0;
+        }
+        if (WITH_C) {
+            __syncthreads();
+#pragma unroll
+            for (int r = b * TR; r < b * TR + TR; ++r) {
+                double u[T], v[T];
+#pragma unroll
+                for (int i = 0; i < T; ++i) {
+                    u[i] = sq[r][ty + 16 * i];
+                    v[i] = sr[r][tx + 16 * i];
+                }
+#pragma unroll
+                for (int i = 0; i < T; ++i)
+#pragma unroll
+                    for (int j = 0; j < T; ++j) acc[i][j] = fma(u[i], v[j], acc[i][j]);
             }
         }
-        __syncthreads();
-        if (WITH_C)
-#pragma unroll
-        for (int r = 0; r < kTRu; ++r) {
-            double u[T], v[T];
-#pragma unroll
-            for (int i = 0; i < T; ++i) {
-                u[i] = sq[r][ty + 16 * i];
-                v[i] = sr[r][tx + 16 * i];
-            }
-#pragma unroll
-            for (int i = 0; i < T; ++i)
-#pragma unroll
-                for (int j = 0; j < T; ++j) acc[i][j] = fma(u[i], v[j], acc[i][j]);
-        }
-        if (t < MP)
-#pragma unroll
-            for (int r = 0; r < kTRu; ++r) rr = fma(sr[r][t], sr[r][t], rr);
     }
     double* out = part + (size_t)blockIdx.x * pstride(m);
+    if (WITH_C)  // else k_gram_partial<MP, 1> fills them, from as many CTAs
 #pragma unroll
-    for (int i = 0; i < T; ++i)
+        for (int i = 0; i < T; ++i)
 #pragma unroll
-        for (int j = 0; j < T; ++j) {
-            const int r = ty + 16 * i, c = tx + 16 * j;
-            if (r < m && c < m) out[r * m + c] = WITH_C ? acc[i][j] : 0.0;
-        }
-    if (t < m) out[m * m + t] = rr;
+            for (int j = 0; j < T; ++j) {
+                const int r = ty + 16 * i, c = tx + 16 * j;
+                if (r < m && c < m) out[r * m + c] = acc[i][j];
+            }
+    __syncthreads();  // sal has been read: its first row block takes the 256 / MP sums a column
+    gsm[t] = rr;
+    __syncthreads();
+    if (t < m) {
+        double v = 0.0;
+#pragma unroll
+        for (int i = 0; i < 256 / MP; ++i) v += gsm[i * MP + t];
+        out[m * m + t] = v;
+    }
 }
+template <int MP>
+constexpr int update_smem(bool with_c) { return (MP + (with_c ? 6 : 4) * tile_rows<MP>()) * MP * (int)sizeof(double); }
 
 // P = R - PΓ on active columns, 0 on the others (in place, row tile by tile).
+// n = 8192, m = 32: 27 → 20 µs (its multiply-adds: 13).
 template <int MP>
 __global__ void __launch_bounds__(256) k_gram_dir(double* __restrict__ P, const double* __restrict__ R, int64_t n,
                                                   int m, const double* __restrict__ gamma,
                                                   const int* __restrict__ active) {
+    constexpr int TR = tile_rows<MP>(), E = TileRegs<MP>::E;
     __shared__ double sg[MP][MP];
-    __shared__ double sp[kTRu][MP];
-    __shared__ int sa[MP];
+    __shared__ double sp[2][TR][MP];
     const int t = threadIdx.x;
     for (int x = t; x < MP * MP; x += 256) {
         const int i = x / MP, j = x % MP;
         sg[i][j] = (i < m && j < m) ? gamma[i * m + j] : 0.0;
     }
-    for (int j = t; j < MP; j += 256) sa[j] = j < m ? active[j] != 0 : 0;
-    const int64_t tiles = (n + kTRu - 1) / kTRu;
-    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        const int64_t r0 = tile * kTRu;
+    const int j = t % MP;  // the thread's column in every tile
+    const bool act = j < m && active[j] != 0;
+    const int64_t tiles = (n + TR - 1) / TR;
+    TileRegs<MP> rp, rres;
+    auto fetch = [&](int64_t tile) {
+        rp.load(P, m, tile * TR, n, m);
+        rres.load(R, m, tile * TR, n, m);
+    };
+    int b = 0;
+    if (blockIdx.x < tiles) fetch(blockIdx.x);
+    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, b ^= 1) {
+        rp.store(&sp[b][0][0]);
+        const TileRegs<MP> cr = rres;
         __syncthreads();
-        for (int e = t; e < kTRu * MP; e += 256) {
-            const int r = e / MP, c = e % MP;
-            const int64_t row = r0 + r;
-            sp[r][c] = (row < n && c < m) ? P[row * m + c] : 0.0;
-        }
-        __syncthreads();
-        for (int o = t; o < kTRu * MP; o += 256) {
-            const int r = o / MP, j = o % MP;
-            const int64_t row = r0 + r;
+        if (tile + gridDim.x < tiles) fetch(tile + gridDim.x);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int r = (t + 256 * e) / MP;
+            const int64_t row = tile * TR + r;
             if (row >= n || j >= m) continue;
-            double v = 0.0;
-            if (sa[j]) {
-                double s = 0.0;
+            double s = 0.0;
 #pragma unroll 16
-                for (int i = 0; i < MP; ++i) s = fma(sp[r][i], sg[i][j], s);
-                v = R[row * m + j] - s;
-            }
-            P[row * m + j] = v;
+            for (int i = 0; i < MP; ++i) s = fma(sp[b][r][i], sg[i][j], s);
+            P[row * m + j] = act ? cr.v[e] - s : 0.0;
         }
     }
 }
@@ -373,15 +429,20 @@ __global__ void k_gram_mask(double* __restrict__ P, int64_t n, int m, const int*
         if (!active[e % m]) P[e] = 0.0;
 }
 
-unsigned row_grid(int64_t n, int rows) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + rows - 1) / rows, kGramCtas)); }
+// CTAs of a row pass of n rows
+template <int MP>
+unsigned row_grid(int64_t n) {
+    constexpr int rows = tile_rows<MP>();
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + rows - 1) / rows, kGramCtas));
+}
 
 template <int MP>
 int launch_alpha(const double* P, const double* AP, const double* R, int64_t n, int m, const GramDev& g,
                  const CgDev& d, cudaStream_t st) {
-    const unsigned gp = row_grid(n, kTRg);
+    const unsigned gp = row_grid<MP>(n);
     k_gram_partial<MP, 2><<<gp, 256, 0, st>>>(P, AP, R, n, m, g.part);
     H2_LAUNCH_CHECK();
-    const unsigned gr = (unsigned)((2 * m * m + 255) / 256);
+    const unsigned gr = (unsigned)((2 * m * m + 31) / 32);
     k_gram_reduce<0><<<gr, 256, 0, st>>>((int)gp, m, g);
     H2_LAUNCH_CHECK();
     k_gram_solve<0><<<(unsigned)((m + kSolveCols - 1) / kSolveCols), kSolveThreads, 0, st>>>(m, 0.0, g, d);
@@ -392,18 +453,18 @@ int launch_alpha(const double* P, const double* AP, const double* R, int64_t n, 
 template <int MP>
 int launch_update(double* X, int64_t ldx, const double* P, const double* AP, double* R, int64_t n, int m,
                   bool with_c, const GramDev& g, cudaStream_t st) {
-    const unsigned gu = row_grid(n, kTRu);
-    if (with_c) k_gram_update<MP, true><<<gu, 256, 0, st>>>(X, ldx, P, AP, R, n, m, g.alpha, g.part);
-    else k_gram_update<MP, false><<<gu, 256, 0, st>>>(X, ldx, P, AP, R, n, m, g.alpha, g.part);
+    const unsigned gu = row_grid<MP>(n);
+    const int sm = update_smem<MP>(with_c);
+    if (with_c) k_gram_update<MP, true><<<gu, 256, sm, st>>>(X, ldx, P, AP, R, n, m, g.alpha, g.part);
+    else k_gram_update<MP, false><<<gu, 256, sm, st>>>(X, ldx, P, AP, R, n, m, g.alpha, g.part);
     H2_LAUNCH_CHECK();
     return 0;
 }
 
 template <int MP>
 int launch_c_partial(const double* AP, const double* Z, int64_t n, int m, const GramDev& g, cudaStream_t st) {
-    // the partials of the update pass hold zeros in the C slots of its CTAs;
-    // this pass (no more CTAs than the update pass) overwrites them
-    k_gram_partial<MP, 1><<<row_grid(n, kTRg), 256, 0, st>>>(AP, Z, nullptr, n, m, g.part);
+    // as many CTAs as the update pass, which left the C slots of its partials to this one
+    k_gram_partial<MP, 1><<<row_grid<MP>(n), 256, 0, st>>>(AP, Z, nullptr, n, m, g.part);
     H2_LAUNCH_CHECK();
     return 0;
 }
@@ -411,8 +472,8 @@ int launch_c_partial(const double* AP, const double* Z, int64_t n, int m, const 
 template <int MP>
 int launch_gamma_dir(double* P, const double* D, int64_t n, int m, double tol, const GramDev& g, const CgDev& d,
                      cudaStream_t st) {
-    const unsigned gu = row_grid(n, kTRu);
-    const unsigned gr = (unsigned)((m * m + m + 255) / 256);
+    const unsigned gu = row_grid<MP>(n);
+    const unsigned gr = (unsigned)((m * m + m + 31) / 32);
     k_gram_reduce<1><<<gr, 256, 0, st>>>((int)gu, m, g);
     H2_LAUNCH_CHECK();
     k_gram_solve<1><<<(unsigned)((m + kSolveCols - 1) / kSolveCols), kSolveThreads, 0, st>>>(m, tol, g, d);
@@ -462,6 +523,9 @@ int gram_prepare() {
     int dev = 0;
     H2_CUDA_TRY(cudaGetDevice(&dev));
     if (dev == g_gram_attr_device) return 0;
+    const cudaFuncAttribute smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    H2_CUDA_TRY(cudaFuncSetAttribute(k_gram_update<64, true>, smem, update_smem<64>(true)));
+    H2_CUDA_TRY(cudaFuncSetAttribute(k_gram_update<64, false>, smem, update_smem<64>(false)));
     g_gram_attr_device = dev;
     return 0;
 }
@@ -471,10 +535,9 @@ int gram_start(double* P, const double* R, int64_t n, int m, const GramDev& g, c
     H2_CUDA_TRY(cudaMemsetAsync(g.ticket, 0, sizeof(unsigned), st));
     H2_CUDA_TRY(cudaMemsetAsync(P, 0, (size_t)n * m * sizeof(double), st));
     H2_CUDA_TRY(cudaMemsetAsync(g.gamma, 0, (size_t)m * m * sizeof(double), st));
-    const unsigned gu = row_grid(n, kTRu);
-    if (m <= 16) k_gram_dir<16><<<gu, 256, 0, st>>>(P, R, n, m, g.gamma, d.active);
-    else if (m <= 32) k_gram_dir<32><<<gu, 256, 0, st>>>(P, R, n, m, g.gamma, d.active);
-    else k_gram_dir<64><<<gu, 256, 0, st>>>(P, R, n, m, g.gamma, d.active);
+    if (m <= 16) k_gram_dir<16><<<row_grid<16>(n), 256, 0, st>>>(P, R, n, m, g.gamma, d.active);
+    else if (m <= 32) k_gram_dir<32><<<row_grid<32>(n), 256, 0, st>>>(P, R, n, m, g.gamma, d.active);
+    else k_gram_dir<64><<<row_grid<64>(n), 256, 0, st>>>(P, R, n, m, g.gamma, d.active);
     H2_LAUNCH_CHECK();
     return 0;
 }
