@@ -79,6 +79,15 @@ __device__ __forceinline__ void bulk_g2s_hint(void* dst, const void* src, uint32
         : "memory");
 }
 
+// Programmatic dependent launch: a kernel launched with launch_chained may start
+// while its predecessor on the stream still runs.  Every thread of such a kernel
+// calls chain_release(), after which the successor's CTAs may be scheduled (they take
+// what this grid leaves free), and chain_wait(), after which everything that earlier
+// kernels wrote is visible; only work on data that no kernel writes stands before it.
+// Every kernel waits, so completion passes down the chain.
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Byte offset of element (row r, column c) of a core-matrix tile whose rows hold
 // kp values of es bytes (kp·es a multiple of 16): 8-row groups outermost, then
 // 16-byte column chunks, then the 8 rows of 16 bytes of one core matrix.

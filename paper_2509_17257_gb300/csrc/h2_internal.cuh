@@ -50,6 +50,25 @@ struct MatData {
     bool built = false;
 };
 
+// Launch with (overlap) or without programmatic dependent launch; the kernel calls
+// chain_release() and chain_wait() (h2_async.cuh).
+template <typename... KArgs, typename... Args>
+int launch_chained(bool overlap, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                   Args... args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = overlap ? 1 : 0;
+    H2_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...));
+    return 0;
+}
+
 // Per-phase event timing of the product (h2_timing_enable / h2_timing_query).
 struct TimingRecord {
     std::vector<cudaEvent_t> ev;       // phase boundaries (7 per product)
@@ -589,7 +608,7 @@ int tc_prepare();
 // transfer-pass bookkeeping, kernel attributes), so that the product itself
 // allocates nothing (e.g. while it is captured into a CUDA graph).
 int product_prepare(h2_matrix* A, int64_t m, int32_t dtype, cudaStream_t st);
-int launch_tc_gemm(int mode, int kind, TcGemmParams p, cudaStream_t st, int stages = 0);
+int launch_tc_gemm(int mode, int kind, TcGemmParams p, cudaStream_t st, int stages = 0, bool overlap = false);
 // Rebuild the CUDA-core transfer passes' lists of pairs for other cut targets.
 int set_transfer_targets(h2_matrix* A, int up_target, int down_target, cudaStream_t st);
 // Work list of the coupling launch with the clusters above the upward cut (TcData::h_*).
@@ -605,11 +624,11 @@ int build_tc(h2_matrix* A, bool bf16, bool tf32, cudaStream_t st);
 // The transfer passes as lists of pairs (h2_transfer.cu), q = 2, 3, 4.
 int build_pairs(h2_matrix* A, cudaStream_t st);
 int launch_pairs(h2_matrix* A, const PairPass& ps, int s0, int s1, bool up, const float* in, float* out, uint8_t* act,
-                 int m, int R, int es, cudaStream_t st);
+                 int m, int R, int es, bool overlap, cudaStream_t st);
 int launch_forward(h2_matrix* A, const double* X, int64_t ldx, int mreal, int m, float* xhat, uint8_t* xcm,
                    uint8_t* Xcm, int R, int es, bool below, int* zflag, int nflag, const int32_t* zid, int nzid,
-                   float* yhat, cudaStream_t st);
-int launch_backward(h2_matrix* A, float* yhat, uint8_t* ycm, int m, int R, int es, cudaStream_t st);
+                   float* yhat, bool overlap, cudaStream_t st);
+int launch_backward(h2_matrix* A, float* yhat, uint8_t* ycm, int m, int R, int es, bool overlap, cudaStream_t st);
 // Tiles and work lists of the tensor-core product with Aᵀ (once per matrix; allocates).
 int build_tc_transposed(h2_matrix* A, cudaStream_t st);
 

@@ -19,6 +19,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "h2_async.cuh"
 #include "h2_internal.cuh"
 
 namespace h2 {
@@ -246,6 +247,8 @@ __global__ void k_gather(const double* __restrict__ X, int64_t ldx, const int32_
 __global__ void k_scatter_y(const float* __restrict__ Z, int ldz, const int32_t* __restrict__ perm, int64_t n, int m,
                             const double* __restrict__ X, int64_t ldx, double* __restrict__ Y, int64_t ldy,
                             double alpha, double sigma, int overwrite) {
+    chain_release();
+    chain_wait();
     const int P = row_lanes(m), R = 32 / P;
     const int lane = threadIdx.x & 31, sub = lane / P, cl = lane % P;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -261,10 +264,12 @@ __global__ void k_scatter_y(const float* __restrict__ Z, int ldz, const int32_t*
     }
 }
 
-void launch_scatter_y(const float* Z, int ldz, const int32_t* perm, int64_t n, int m, const double* X, int64_t ldx,
-                      double* Y, int64_t ldy, double alpha, double sigma, bool overwrite, cudaStream_t st) {
+int launch_scatter_y(const float* Z, int ldz, const int32_t* perm, int64_t n, int m, const double* X, int64_t ldx,
+                     double* Y, int64_t ldy, double alpha, double sigma, bool overwrite, bool overlap,
+                     cudaStream_t st) {
     const unsigned g = (unsigned)std::min<int64_t>((n * m + 255) / 256, 152 * 32);
-    k_scatter_y<<<g, 256, 0, st>>>(Z, ldz, perm, n, m, X, ldx, Y, ldy, alpha, sigma, overwrite ? 1 : 0);
+    return launch_chained(overlap, k_scatter_y, g, 256, 0, st, Z, ldz, perm, n, m, X, ldx, Y, ldy, alpha, sigma,
+                          overwrite ? 1 : 0);
 }
 
 // ---- the same over C: interleaved (real, imaginary) columns, m2 = 2·m_c, and
@@ -272,6 +277,8 @@ void launch_scatter_y(const float* Z, int ldz, const int32_t* perm, int64_t n, i
 __global__ void k_scatter_yc(const float* __restrict__ Z, int ldz, const int32_t* __restrict__ perm, int64_t n,
                              int m2, const double* __restrict__ X, int64_t ldx, double* __restrict__ Y, int64_t ldy,
                              double alpha_re, double alpha_im, double sigma, int overwrite) {
+    chain_release();
+    chain_wait();
     const int mc = m2 >> 1;
     const int P = row_lanes(mc), R = 32 / P;
     const int lane = threadIdx.x & 31, sub = lane / P, cl = lane % P;
@@ -864,6 +871,9 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
         const bool lists = kind == 1 ? D.hybrid : D.hybrid_bf16;
         const bool hybrid = fast && !flow && !trans && !mf && !cx && lists && want_hybrid && !capturing;
         const int ml = fast && !flow ? pad4(mc) : mc;  // columns of the coefficient blocks and of Z
+        // the chain's kernels start under the tail of the one before (not in a capture,
+        // whose branches are cut and joined by events, nor between timing events)
+        const bool overlap = fast && !flow && !capturing && !A->timing.on;
         const size_t bXp = align_up((size_t)n * ml * 4), bC = align_up((size_t)nc * k * ml * 4);
         int rc = ensure_workspace(A, bXp + 2 * bC + bXcm + 3 * bAct, st);
         if (rc) return rc;
@@ -885,7 +895,7 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
             // launch also clears the hybrid launch's ready flags and ŷ of the clusters
             // without couplings)
             if ((rc = launch_forward(A, X + c0, ldx, mc, ml, xhat, xcm, Xcm, R, es, hybrid, sbc.fflag,
-                                     hybrid ? (int)nc : 0, zid, nzid, yhat, st)))
+                                     hybrid ? (int)nc : 0, zid, nzid, yhat, overlap, st)))
                 return rc;
         } else {
             const int64_t total = n * mc;
@@ -1002,8 +1012,9 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
                 if ((rc = launch_tc_gemm(1, 1, lp, st, stg))) return rc;
             }
             if ((rc = wait_y_staged(A->ws, st))) return rc;
-            launch_scatter_y(Xp, mc, A->d_perm, n, mc, X + c0, ldx, Y + c0, ldy, alpha, A->sigma, overwrite, st);
-            H2_LAUNCH_CHECK();
+            if ((rc = launch_scatter_y(Xp, mc, A->d_perm, n, mc, X + c0, ldx, Y + c0, ldy, alpha, A->sigma, overwrite,
+                                       false, st)))
+                return rc;
             marks.mark();
             if ((rc = marks.commit())) return rc;
             continue;
@@ -1047,12 +1058,12 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
         }
         marks.kernel_begin();
         if (cp.n_items > 0 &&
-            (rc = launch_tc_gemm(hybrid ? 4 : (mf ? 2 : 0), kind, cp, st, stg)))
+            (rc = launch_tc_gemm(hybrid ? 4 : (mf ? 2 : 0), kind, cp, st, stg, overlap)))
             return rc;
         marks.kernel_end();
         marks.mark();
         if (fast) {
-            if ((rc = launch_backward(A, yhat, ycm, ml, R, es, st))) return rc;
+            if ((rc = launch_backward(A, yhat, ycm, ml, R, es, overlap, st))) return rc;
         } else {
             if ((rc = backward_pass<float, RM, CN>(A, E, yhat, mc, gy, gzk, st, sbc))) return rc;
             if ((rc = launch_pack_act(yhat, mc, NL, A->d_leaves, nullptr, nullptr, k, nullptr, KP, mc, R, ycm, es, st)))
@@ -1075,17 +1086,19 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
         lp.zp = Xp;  // the gathered FP32 X is no longer read after the forward pass and its packing
         lp.ldc = ml;
         lp.cplx = cx ? 1 : 0;
-        if ((rc = launch_tc_gemm(1, kind, lp, st, stg))) return rc;
+        if ((rc = launch_tc_gemm(1, kind, lp, st, stg, overlap))) return rc;
         {
             const int64_t total = n * mc;
             const unsigned g = (unsigned)std::min<int64_t>((total + 255) / 256, 152 * 32);
+            const bool staged = A->ws.y_wait;  // an event to wait for stands before the scatter
             if ((rc = wait_y_staged(A->ws, st))) return rc;
             if (cx)
-                k_scatter_yc<<<g, 256, 0, st>>>(Xp, ml, A->d_perm, n, mc, X + c0, ldx, Y + c0, ldy, alpha, *alpha_im,
-                                                A->sigma, overwrite ? 1 : 0);
+                rc = launch_chained(overlap && !staged, k_scatter_yc, g, 256, 0, st, Xp, ml, A->d_perm, n, mc, X + c0, ldx,
+                                    Y + c0, ldy, alpha, *alpha_im, A->sigma, overwrite ? 1 : 0);
             else
-                launch_scatter_y(Xp, ml, A->d_perm, n, mc, X + c0, ldx, Y + c0, ldy, alpha, A->sigma, overwrite, st);
-            H2_LAUNCH_CHECK();
+                rc = launch_scatter_y(Xp, ml, A->d_perm, n, mc, X + c0, ldx, Y + c0, ldy, alpha, A->sigma, overwrite,
+                                      overlap && !staged, st);
+            if (rc) return rc;
         }
         marks.mark();
         if ((rc = marks.commit())) return rc;
@@ -1305,9 +1318,7 @@ int flow_pre(h2_matrix* A, const double* X, int64_t ldx, const FlowBufs& fb, cud
 // After them: Y += α(Z + σX) in the caller's order (Y = α(Z + σX) with overwrite).
 int flow_post(h2_matrix* A, double alpha, const double* X, int64_t ldx, double* Y, int64_t ldy, const FlowBufs& fb,
               bool overwrite, cudaStream_t st) {
-    launch_scatter_y(fb.Xp, fb.mc, A->d_perm, A->n, fb.mc, X, ldx, Y, ldy, alpha, A->sigma, overwrite, st);
-    H2_LAUNCH_CHECK();
-    return 0;
+    return launch_scatter_y(fb.Xp, fb.mc, A->d_perm, A->n, fb.mc, X, ldx, Y, ldy, alpha, A->sigma, overwrite, false, st);
 }
 
 int forward_transform_f64(h2_matrix* A, const double* X, int64_t ldx, int64_t m, double* Xp, double* xhat,

@@ -341,6 +341,7 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
     __shared__ int stage_t[MF ? kSt : 1];  // MODE 2: target cluster
     __shared__ int abort_shared;
     volatile int& abort_flag = abort_shared;
+    chain_release();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int R = p.R;
     const int M = R <= 64 ? 64 : 128;
@@ -386,6 +387,9 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
+    // the barriers, TMEM and the item count (of static lists) are set up while the
+    // launch before still runs
+    chain_wait();
 
     if (warp == 0) {
         // ---------------- producer ----------------
@@ -1156,15 +1160,13 @@ NarrowFit& narrow_fit() {
 }
 
 template <int MODE, int KIND>
-int launch_one(const TcGemmParams& p, bool narrow, int smem, cudaStream_t st) {
+int launch_one(const TcGemmParams& p, bool narrow, int smem, bool overlap, cudaStream_t st) {
     // Every CTA has to be resident: those of modes 3 and 4 wait on each other's
     // ready flags (bounded).
     const int per_sm = narrow ? narrow_fit<MODE, KIND>().per_sm(tc_threads<KIND>(), smem) : 1;
     const int grid = std::min(p.n_items, per_sm * kTcGrid);
-    if (narrow) k_tc_gemm<MODE, KIND, true><<<grid, tc_threads<KIND>(), smem, st>>>(p);
-    else k_tc_gemm<MODE, KIND, false><<<grid, tc_threads<KIND>(), smem, st>>>(p);
-    H2_LAUNCH_CHECK();
-    return 0;
+    return launch_chained(overlap, narrow ? k_tc_gemm<MODE, KIND, true> : k_tc_gemm<MODE, KIND, false>, grid,
+                          tc_threads<KIND>(), smem, st, p);
 }
 template <int MODE, int KIND>
 int prepare_one(int dev) {
@@ -1201,7 +1203,7 @@ int tc_prepare() {
     return 0;
 }
 
-int launch_tc_gemm(int mode, int kind, TcGemmParams p, cudaStream_t st, int stages) {
+int launch_tc_gemm(int mode, int kind, TcGemmParams p, cudaStream_t st, int stages, bool overlap) {
     const bool narrow = p.R <= 64;
     TcGeometry g = tc_geometry(p.R, mode, kind, narrow);
     // a tuned stage count (h2_autotune) below the number that fits
@@ -1217,18 +1219,18 @@ int launch_tc_gemm(int mode, int kind, TcGemmParams p, cudaStream_t st, int stag
     if (rc) return rc;
     const int smem = g.nstages * g.stage_bytes + g.after + 128;
     if (kind == 0) {
-        if (mode == 0) return launch_one<0, 0>(p, narrow, smem, st);
-        if (mode == 1) return launch_one<1, 0>(p, narrow, smem, st);
-        if (mode == 4) return launch_one<4, 0>(p, narrow, smem, st);
+        if (mode == 0) return launch_one<0, 0>(p, narrow, smem, overlap, st);
+        if (mode == 1) return launch_one<1, 0>(p, narrow, smem, overlap, st);
+        if (mode == 4) return launch_one<4, 0>(p, narrow, smem, overlap, st);
         set_error(mode == 2 ? "matrix-free coupling runs on the TF32 path only"
                             : "the tensor-core transfer passes run on the TF32 path only");
         return H2_E_UNSUPPORTED;
     }
-    if (mode == 2) return launch_one<2, 1>(p, narrow, smem, st);
-    if (mode == 3) return launch_one<3, 1>(p, narrow, smem, st);
-    if (mode == 4) return launch_one<4, 1>(p, narrow, smem, st);
-    if (mode == 0) return launch_one<0, 1>(p, narrow, smem, st);
-    return launch_one<1, 1>(p, narrow, smem, st);
+    if (mode == 2) return launch_one<2, 1>(p, narrow, smem, overlap, st);
+    if (mode == 3) return launch_one<3, 1>(p, narrow, smem, overlap, st);
+    if (mode == 4) return launch_one<4, 1>(p, narrow, smem, overlap, st);
+    if (mode == 0) return launch_one<0, 1>(p, narrow, smem, overlap, st);
+    return launch_one<1, 1>(p, narrow, smem, overlap, st);
 }
 
 int launch_pack_tiles(const TcPackTile* tiles, int64_t count, const double* src, uint8_t* dst, int es,

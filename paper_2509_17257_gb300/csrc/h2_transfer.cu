@@ -149,6 +149,7 @@ __global__ void __launch_bounds__(CN == 4 ? 256 : 128) k_leaf_up(const LeafUp p)
     __shared__ __align__(16) float sx[64 * 16 * CN];  // X|_t̂
     __shared__ __align__(16) float sh[H == 2 ? 64 * 16 : 4];  // the second half's sums
     __shared__ int s_perm[64];
+    chain_release();
     const int4 rec = p.rec[blockIdx.x];
     const int t = rec.x, off = rec.y, nt = rec.z;
     if (threadIdx.x < nt) s_perm[threadIdx.x] = p.perm[off + threadIdx.x];
@@ -163,6 +164,7 @@ __global__ void __launch_bounds__(CN == 4 ? 256 : 128) k_leaf_up(const LeafUp p)
 #pragma unroll 4
         for (int e = threadIdx.x; e < nt * k; e += T) sv[(e / k) * ldv + e % k] = __ldg(V + e);
     }
+    chain_wait();
     {
         const int64_t i0 = blockIdx.x * (int64_t)T + threadIdx.x, n = (int64_t)gridDim.x * T;
         for (int64_t i = i0; i < p.nflag; i += n) p.zflag[i] = 0;
@@ -270,7 +272,9 @@ __global__ void __launch_bounds__(32 * W, W == 4 ? 4 : 2) k_pairs(const Pairs p)
     const int logP = LOGP ? LOGP : p.logP, P = 1 << logP, m = LOGP ? P : p.m;
     const int col0 = LOGP ? 0 : P * blockIdx.y, mc = LOGP ? P : min(P, m - col0);
     const int grp = threadIdx.x >> logP, col = threadIdx.x & (P - 1), NG = 32 * W >> logP;
+    chain_release();
     const PairItem it = p.items[blockIdx.x];
+    chain_wait();
     const int np = it.p1 - it.p0;
     float* mine = red + grp * K * P + col;
     float* fs = red + K * 32 * W + grp * FL;
@@ -348,15 +352,14 @@ int cut_level(const Tree& T, int64_t n_leaves, int target, int usual) {
 }
 
 template <int Q, bool UP, int W, int LOGP>
-int launch_pairs_w(const Pairs& p, int n_items, cudaStream_t st) {
+int launch_pairs_w(const Pairs& p, int n_items, bool overlap, cudaStream_t st) {
     constexpr int K = Q * Q * Q, FL = (3 * Q * Q + 3) & ~3;
     const dim3 grid((unsigned)n_items, (unsigned)((p.m + p.P - 1) / p.P));
-    k_pairs<Q, UP, W, LOGP><<<grid, 32 * W, (32 * W * K + (32 * W >> p.logP) * FL) * (int)sizeof(float), st>>>(p);
-    H2_LAUNCH_CHECK();
-    return 0;
+    return launch_chained(overlap, k_pairs<Q, UP, W, LOGP>, grid, 32 * W,
+                          (32 * W * K + (32 * W >> p.logP) * FL) * sizeof(float), st, p);
 }
 template <int Q, bool UP>
-int launch_stage(const PairPass& ps, int s, Pairs p, cudaStream_t st) {
+int launch_stage(const PairPass& ps, int s, Pairs p, bool overlap, cudaStream_t st) {
     const PairPass::Stage& g = ps.stages[s];
     if (g.i1 == g.i0) return 0;
     p.items = ps.items + g.i0;
@@ -371,10 +374,10 @@ int launch_stage(const PairPass& ps, int s, Pairs p, cudaStream_t st) {
     auto few = [&](int lp) { return n * ((p.m + (1 << lp) - 1) >> lp) < 152; };
     while (p.logP > 3 && g.longest > (128 >> p.logP) && few(p.logP)) --p.logP;
     p.P = 1 << p.logP;
-    if (g.longest > (128 >> p.logP) && few(p.logP)) return launch_pairs_w<Q, UP, 8, 0>(p, n, st);
-    if (Q == 4 && p.m == p.P && p.logP == 5) return launch_pairs_w<Q, UP, 4, 5>(p, n, st);
-    if (Q == 4 && p.m == p.P && p.logP == 4) return launch_pairs_w<Q, UP, 4, 4>(p, n, st);
-    return launch_pairs_w<Q, UP, 4, 0>(p, n, st);
+    if (g.longest > (128 >> p.logP) && few(p.logP)) return launch_pairs_w<Q, UP, 8, 0>(p, n, overlap, st);
+    if (Q == 4 && p.m == p.P && p.logP == 5) return launch_pairs_w<Q, UP, 4, 5>(p, n, overlap, st);
+    if (Q == 4 && p.m == p.P && p.logP == 4) return launch_pairs_w<Q, UP, 4, 4>(p, n, overlap, st);
+    return launch_pairs_w<Q, UP, 4, 0>(p, n, overlap, st);
 }
 
 int g_pairs_device = -1;
@@ -540,7 +543,7 @@ int build_pairs(h2_matrix* A, cudaStream_t st) {
 // multiple of 4), with `below` only of the clusters at or below the cut.
 int launch_forward(h2_matrix* A, const double* X, int64_t ldx, int mreal, int m, float* xhat, uint8_t* xcm,
                    uint8_t* Xcm, int R, int es, bool below, int* zflag, int nflag, const int32_t* zid, int nzid,
-                   float* yhat, cudaStream_t st) {
+                   float* yhat, bool overlap, cudaStream_t st) {
     int rc = pairs_prepare();
     if (rc) return rc;
     const int NL = (int)A->leaves.size();
@@ -565,24 +568,28 @@ int launch_forward(h2_matrix* A, const double* X, int64_t ldx, int mreal, int m,
     p.nzid = nzid;
     p.yhat = yhat;
     const bool full = A->k == 64;
-    if (m == 16 && full) k_leaf_up<1, true><<<NL, 128, 0, st>>>(p);
-    else if (m <= 16) k_leaf_up<1, false><<<NL, 128, 0, st>>>(p);
-    else if (m == 32 && full) k_leaf_up<2, true><<<NL, 128, 0, st>>>(p);
-    else if (m <= 32) k_leaf_up<2, false><<<NL, 128, 0, st>>>(p);
-    else if (m == 64 && full) k_leaf_up<4, true><<<NL, 256, 0, st>>>(p);
-    else k_leaf_up<4, false><<<NL, 256, 0, st>>>(p);
-    H2_LAUNCH_CHECK();
+    auto leaves = [&](void (*kernel)(const LeafUp), int threads) {
+        return launch_chained(overlap, kernel, NL, threads, 0, st, p);
+    };
+    if (m == 16 && full) rc = leaves(k_leaf_up<1, true>, 128);
+    else if (m <= 16) rc = leaves(k_leaf_up<1, false>, 128);
+    else if (m == 32 && full) rc = leaves(k_leaf_up<2, true>, 128);
+    else if (m <= 32) rc = leaves(k_leaf_up<2, false>, 128);
+    else if (m == 64 && full) rc = leaves(k_leaf_up<4, true>, 256);
+    else rc = leaves(k_leaf_up<4, false>, 256);
+    if (rc) return rc;
     const int stages = below ? A->up_pairs.below_cut : (int)A->up_pairs.stages.size();
-    return launch_pairs(A, A->up_pairs, 0, stages, true, xhat, xhat, xcm, m, R, es, st);
+    return launch_pairs(A, A->up_pairs, 0, stages, true, xhat, xhat, xcm, m, R, es, overlap, st);
 }
 
 // Backward transfer pass: ŷ of the leaves as split tiles, from ŷ after the coupling.
-int launch_backward(h2_matrix* A, float* yhat, uint8_t* ycm, int m, int R, int es, cudaStream_t st) {
-    return launch_pairs(A, A->down_pairs, 0, (int)A->down_pairs.stages.size(), false, yhat, yhat, ycm, m, R, es, st);
+int launch_backward(h2_matrix* A, float* yhat, uint8_t* ycm, int m, int R, int es, bool overlap, cudaStream_t st) {
+    return launch_pairs(A, A->down_pairs, 0, (int)A->down_pairs.stages.size(), false, yhat, yhat, ycm, m, R, es,
+                        overlap, st);
 }
 
 int launch_pairs(h2_matrix* A, const PairPass& ps, int s0, int s1, bool up, const float* in, float* out, uint8_t* act,
-                 int m, int R, int es, cudaStream_t st) {
+                 int m, int R, int es, bool overlap, cudaStream_t st) {
     int rc = pairs_prepare();
     if (rc) return rc;
     Pairs p{};
@@ -594,9 +601,9 @@ int launch_pairs(h2_matrix* A, const PairPass& ps, int s0, int s1, bool up, cons
     p.R = R;
     p.es = es;
     for (int s = s0; s < s1 && !rc; ++s)
-        if (A->q == 4) rc = up ? launch_stage<4, true>(ps, s, p, st) : launch_stage<4, false>(ps, s, p, st);
-        else if (A->q == 3) rc = up ? launch_stage<3, true>(ps, s, p, st) : launch_stage<3, false>(ps, s, p, st);
-        else rc = up ? launch_stage<2, true>(ps, s, p, st) : launch_stage<2, false>(ps, s, p, st);
+        if (A->q == 4) rc = up ? launch_stage<4, true>(ps, s, p, overlap, st) : launch_stage<4, false>(ps, s, p, overlap, st);
+        else if (A->q == 3) rc = up ? launch_stage<3, true>(ps, s, p, overlap, st) : launch_stage<3, false>(ps, s, p, overlap, st);
+        else rc = up ? launch_stage<2, true>(ps, s, p, overlap, st) : launch_stage<2, false>(ps, s, p, overlap, st);
     return rc;
 }
 
