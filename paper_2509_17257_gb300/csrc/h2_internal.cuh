@@ -591,15 +591,16 @@ int matmul_in_scratch(h2_matrix* A, double alpha, const double* X, int64_t ldx, 
                       int64_t m, int32_t dtype, cudaStream_t st, void* scratch);
 
 // The FP64 phases (h2_mm64.cu): k <= 64 for the two transfer passes, kron the
-// factors of E for q = 4 or null; m columns, row stride m, except Y's.
+// factors of E for q = 4 or null; m columns, row stride m, except Y's.  The upward
+// pass also clears the flags and tickets of the downward pass.
 int launch_up64(h2_matrix* A, const double* V, const double* E, const double* kron, const double* Xp, double* xhat,
-                int m, const SyncBufs& sb, cudaStream_t st);
+                int m, const SyncBufs& sb, bool overlap, cudaStream_t st);
 int launch_down64(h2_matrix* A, const double* E, const double* kron, double* yhat, int m, const SyncBufs& sb,
-                  cudaStream_t st);
+                  bool overlap, cudaStream_t st);
 int launch_coupling64(h2_matrix* A, const double* S, const double* xhat, double* yhat, int m, bool trans,
-                      cudaStream_t st);
+                      bool overlap, cudaStream_t st);
 int launch_leaf64(h2_matrix* A, const double* V, const double* G, const double* yhat, const double* Xp, double* Y,
-                  int64_t ldy, double alpha, int m, bool trans, bool overwrite, cudaStream_t st);
+                  int64_t ldy, double alpha, int m, bool trans, bool overwrite, bool overlap, cudaStream_t st);
 
 // tcgen05 BF16 kernels (h2_tc.cu)
 int tc_smem_bytes();

@@ -233,6 +233,8 @@ __device__ __forceinline__ int row_lanes(int m) {
 template <typename T>
 __global__ void k_gather(const double* __restrict__ X, int64_t ldx, const int32_t* __restrict__ perm, int64_t n,
                          int m, T* __restrict__ Xp) {
+    chain_release();
+    chain_wait();
     const int P = row_lanes(m), R = 32 / P;
     const int lane = threadIdx.x & 31, sub = lane / P, cl = lane % P;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -662,12 +664,12 @@ struct PhaseMarks {
 // level otherwise).  Records the leaf-forward and upward phase marks.
 template <typename T, int RM, int CN>
 int forward_pass(h2_matrix* A, const T* V, const T* E, const T* Xp, T* xhat, int m, unsigned gy, unsigned gzk,
-                 cudaStream_t st, const SyncBufs& sb, PhaseMarks& marks, const T* kron = nullptr) {
+                 cudaStream_t st, const SyncBufs& sb, PhaseMarks& marks, const T* kron = nullptr, bool overlap = false) {
     const int k = A->k;
     const unsigned NL = (unsigned)A->leaves.size();
     if (gzk == 1) {
         if constexpr (std::is_same_v<T, double>) {
-            const int rc = launch_up64(A, V, E, kron, Xp, xhat, m, sb, st);
+            const int rc = launch_up64(A, V, E, kron, Xp, xhat, m, sb, overlap, st);
             if (rc) return rc;
         } else {
             k_up_fused<T, RM, CN><<<dim3(NL, gy), kThreads, 0, st>>>(A->d_leaves, A->d_cl_off, A->d_cl_size,
@@ -697,12 +699,12 @@ int forward_pass(h2_matrix* A, const T* V, const T* E, const T* Xp, T* xhat, int
 // Backward transfer pass ŷ_{t'} += E_{t'} ŷ_t (one launch when k <= 64).
 template <typename T, int RM, int CN>
 int backward_pass(h2_matrix* A, const T* E, T* yhat, int m, unsigned gy, unsigned gzk, cudaStream_t st,
-                  const SyncBufs& sb, const T* kron = nullptr) {
+                  const SyncBufs& sb, const T* kron = nullptr, bool overlap = false) {
     const int k = A->k;
     const int n_items = (int)A->down_ptr[A->depth + 1];
     if (n_items == 0) return 0;
     if (gzk == 1) {
-        if constexpr (std::is_same_v<T, double>) return launch_down64(A, E, kron, yhat, m, sb, st);
+        if constexpr (std::is_same_v<T, double>) return launch_down64(A, E, kron, yhat, m, sb, overlap, st);
         // ready flags and claim tickets start at zero for every product (graph-replay safe)
         H2_CUDA_TRY(cudaMemsetAsync(sb.flag, 0, (size_t)A->nc * gy * sizeof(int), st));
         H2_CUDA_TRY(cudaMemsetAsync(sb.claim, 0, gy * sizeof(unsigned), st));
@@ -742,16 +744,20 @@ int run_chain(h2_matrix* A, const MatData& D, double alpha, const double* X, int
     const T* kron = (k == 64 && RM == 4 && A->use_kron) ? (const T*)D.kron : nullptr;
     PhaseMarks marks(A, st);
     int rc = 0;
+    // the FP64 kernels start under the tail of the one before, as in run_chain_tc
+    // (n = 4096, q = 3, m = 8: 174 → 166 µs; n = 32768, q = 4, m = 16: 2909 → 2877).
+    // The solvers' own kernels are launched plainly: with them in the chain too an
+    // iteration of the Gram block CG (n = 8192, m = 32) took 660 µs instead of 440.
+    const bool overlap = std::is_same_v<T, double> && !A->timing.on && !stream_capture_active(st);
     marks.mark();
     {
         const int64_t total = A->n * m;
         const unsigned g = (unsigned)std::min<int64_t>((total + 255) / 256, 152 * 32);
-        k_gather<T><<<g, 256, 0, st>>>(X, ldx, A->d_perm, A->n, m, Xp);
-        H2_LAUNCH_CHECK();
+        if ((rc = launch_chained(overlap, k_gather<T>, g, 256, 0, st, X, ldx, A->d_perm, A->n, m, Xp))) return rc;
     }
     marks.mark();
     const unsigned NL = (unsigned)A->leaves.size();
-    if ((rc = forward_pass<T, RM, CN>(A, V, E, Xp, xhat, m, gy, gzk, st, sb, marks, kron))) return rc;
+    if ((rc = forward_pass<T, RM, CN>(A, V, E, Xp, xhat, m, gy, gzk, st, sb, marks, kron, overlap))) return rc;
     marks.kernel_begin();
     if (alpha_im) {
         if constexpr (CN % 2 == 0) {
@@ -762,7 +768,7 @@ int run_chain(h2_matrix* A, const MatData& D, double alpha, const double* X, int
             return H2_E_UNSUPPORTED;
         }
     } else if constexpr (std::is_same_v<T, double>) {
-        if ((rc = launch_coupling64(A, S, xhat, yhat, m, transposed, st))) return rc;
+        if ((rc = launch_coupling64(A, S, xhat, yhat, m, transposed, overlap, st))) return rc;
     } else if (transposed)
         k_coupling<T, RM, CN, true><<<dim3((unsigned)A->nc, gy, gzk), kThreads, 0, st>>>(
             A->d_admT_rowptr, A->d_admT_row, A->d_admT_blk, S, xhat, yhat, k, m);
@@ -772,8 +778,9 @@ int run_chain(h2_matrix* A, const MatData& D, double alpha, const double* X, int
     H2_LAUNCH_CHECK();
     marks.kernel_end();
     marks.mark();
-    if ((rc = backward_pass<T, RM, CN>(A, E, yhat, m, gy, gzk, st, sb, kron))) return rc;
+    if ((rc = backward_pass<T, RM, CN>(A, E, yhat, m, gy, gzk, st, sb, kron, overlap))) return rc;
     marks.mark();
+    const bool staged = A->ws.y_wait;  // an event to wait for stands before the last phase
     if ((rc = wait_y_staged(A->ws, st))) return rc;
     if (alpha_im) {
         if constexpr (CN % 2 == 0) {
@@ -785,7 +792,8 @@ int run_chain(h2_matrix* A, const MatData& D, double alpha, const double* X, int
             return H2_E_UNSUPPORTED;
         }
     } else if constexpr (std::is_same_v<T, double>) {
-        if ((rc = launch_leaf64(A, V, G, yhat, Xp, Y, ldy, alpha, m, transposed, overwrite, st))) return rc;
+        if ((rc = launch_leaf64(A, V, G, yhat, Xp, Y, ldy, alpha, m, transposed, overwrite, overlap && !staged, st)))
+            return rc;
     } else if (transposed)
         k_leaf_bwd_near<T, RM, CN, true><<<dim3(NL, gy, gzl), kThreads, 0, st>>>(
             A->d_leaves, A->d_cl_off, A->d_cl_size, A->d_perm, V, yhat, A->d_nearT_ptr, A->d_nearT_row,

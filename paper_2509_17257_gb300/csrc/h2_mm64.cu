@@ -20,6 +20,7 @@
 
 #include <algorithm>
 
+#include "h2_async.cuh"
 #include "h2_internal.cuh"
 
 namespace h2 {
@@ -119,6 +120,8 @@ __global__ void __launch_bounds__(32 * kSplitWarps64) k_coupling64(int chunks, c
                                                    const int32_t* __restrict__ blk, const double* __restrict__ S,
                                                    const double* __restrict__ xhat, double* __restrict__ yhat, int k,
                                                    int m) {
+    chain_release();
+    chain_wait();
     const int pos = blockIdx.x / chunks;
     Pair p;
     const bool live = my_pair(k, m, blockIdx.x - pos * chunks, p);
@@ -150,6 +153,8 @@ __global__ void __launch_bounds__(32 * kSplitWarps64) k_leaf64(
     const int32_t* __restrict__ nblk, const int64_t* __restrict__ near_off, const double* __restrict__ G,
     const double* __restrict__ Xp, double* __restrict__ Y, int64_t ldy, double alpha, double sigma, int k, int m,
     int overwrite) {
+    chain_release();
+    chain_wait();
     const int pos = blockIdx.x / chunks;
     const int lp = order[pos];
     const int t = leaves[lp];
@@ -188,7 +193,14 @@ __global__ void __launch_bounds__(32) k_leaf_fwd64(int chunks, const int32_t* __
                                                    const int32_t* __restrict__ cl_off,
                                                    const int32_t* __restrict__ cl_size,
                                                    const double* __restrict__ V, const double* __restrict__ Xp,
-                                                   double* __restrict__ xhat, int k, int m) {
+                                                   double* __restrict__ xhat, int k, int m, int* __restrict__ flag,
+                                                   int64_t nflag, unsigned* __restrict__ claim, int nclaim) {
+    chain_release();
+    chain_wait();
+    // the downward pass starts from cleared flags and claim tickets
+    const int64_t cta = blockIdx.y * (int64_t)gridDim.x + blockIdx.x, ctas = (int64_t)gridDim.x * gridDim.y;
+    for (int64_t e = cta * 32 + threadIdx.x; e < nflag; e += ctas * 32) flag[e] = 0;
+    for (int64_t e = cta * 32 + threadIdx.x; e < nclaim; e += ctas * 32) claim[e] = 0u;
     const int lp = blockIdx.x / chunks;
     Pair p;
     if (!my_pair(k, m, blockIdx.x - lp * chunks, p)) return;
@@ -273,6 +285,8 @@ __global__ void __launch_bounds__(kT) k_up64(const int32_t* __restrict__ leaves,
                                              const int32_t* __restrict__ son1, const double* __restrict__ E,
                                              const double* __restrict__ kron, double* xhat,
                                              unsigned* __restrict__ cnt, int k, int m) {
+    chain_release();
+    chain_wait();
     __shared__ double xs[2 * 64 * CS], ys[2 * 64 * CS], F[96];
     __shared__ int s_go;
     double fv = 0.0;
@@ -368,14 +382,16 @@ __global__ void __launch_bounds__(kT) k_up64(const int32_t* __restrict__ leaves,
 // item (atomic ticket), waits until its parent's ŷ is final (the parent's item
 // has a smaller ticket, so a running CTA holds it; the wait is bounded and
 // reports a timeout through err), adds E_{t'} ŷ_parent and sets its own bit of
-// the cluster's ready flags (one word per 64-column tile, cleared before each
-// launch).  n = 4096, q = 3, m = 8: 99 → 34 µs; n = 32768, q = 4, m = 16: 121 → 71.
+// the cluster's ready flags (one word per 64-column tile, cleared by
+// k_leaf_fwd64).  n = 4096, q = 3, m = 8: 99 → 34 µs; n = 32768, q = 4, m = 16: 121 → 71.
 template <int CS>
 __global__ void __launch_bounds__(kT) k_down64(const int32_t* __restrict__ order, int n_items, int slices,
                                                const int32_t* __restrict__ parent, const double* __restrict__ E,
                                                const double* __restrict__ kron, double* yhat,
                                                unsigned* __restrict__ claim, unsigned* flag, int* __restrict__ err,
                                                int k, int m, long long spin_limit) {
+    chain_release();
+    chain_wait();
     __shared__ double xs[64 * CS], ys[4 * 64 * CS], F[48];
     __shared__ int s_item, s_ok;
     const int tile = blockIdx.y, tiles = gridDim.y;
@@ -490,73 +506,47 @@ int list_threads(const dim3& g) { return (int64_t)g.x * g.y <= 152 * 8 ? 32 * kS
 }  // namespace
 
 int launch_up64(h2_matrix* A, const double* V, const double* E, const double* kron, const double* Xp, double* xhat,
-                int m, const SyncBufs& sb, cudaStream_t st) {
+                int m, const SyncBufs& sb, bool overlap, cudaStream_t st) {
     const int NL = (int)A->leaves.size(), CS = slice_cols(m, NL);
     const int tiles = (m + 63) / 64, slices = (std::min(m, 64) + CS - 1) / CS, chunks = chunks_of(A->k, m);
-    k_leaf_fwd64<<<chunk_grid(NL, chunks, m), 32, 0, st>>>(chunks, A->d_leaves, A->d_cl_off, A->d_cl_size, V, Xp,
-                                                           xhat, A->k, m);
-    H2_LAUNCH_CHECK();
-    if (A->nc == 1) return 0;
+    int rc = launch_chained(overlap, k_leaf_fwd64, chunk_grid(NL, chunks, m), 32, 0, st, chunks, A->d_leaves,
+                            A->d_cl_off, A->d_cl_size, V, Xp, xhat, A->k, m, sb.flag, A->nc * (int64_t)tiles, sb.claim,
+                            tiles);
+    if (rc || A->nc == 1) return rc;
     const dim3 g((unsigned)(NL * slices), (unsigned)tiles);
-#define UP64(CS_)                                                                                               \
-    k_up64<CS_><<<g, kT, 0, st>>>(A->d_leaves, NL, A->d_parent, A->d_son0, A->d_son1, E, kron, xhat, sb.cnt, A->k, m)
-    if (CS == 1) UP64(1);
-    else if (CS == 2) UP64(2);
-    else UP64(4);
-#undef UP64
-    H2_LAUNCH_CHECK();
-    return 0;
+    return launch_chained(overlap, CS == 1 ? k_up64<1> : (CS == 2 ? k_up64<2> : k_up64<4>), g, kT, 0, st, A->d_leaves, NL,
+                          A->d_parent, A->d_son0, A->d_son1, E, kron, xhat, sb.cnt, A->k, m);
 }
 
 int launch_down64(h2_matrix* A, const double* E, const double* kron, double* yhat, int m, const SyncBufs& sb,
-                  cudaStream_t st) {
+                  bool overlap, cudaStream_t st) {
     const int n_items = (int)A->down_ptr[A->depth + 1], CS = slice_cols(m, (int64_t)A->leaves.size());
     if (n_items == 0) return 0;
     const int tiles = (m + 63) / 64, slices = (std::min(m, 64) + CS - 1) / CS;
-    // ready flags and claim tickets start at zero for every product (graph-replay safe)
-    H2_CUDA_TRY(cudaMemsetAsync(sb.flag, 0, (size_t)A->nc * tiles * sizeof(int), st));
-    H2_CUDA_TRY(cudaMemsetAsync(sb.claim, 0, tiles * sizeof(unsigned), st));
     const dim3 g((unsigned)std::min<int64_t>((int64_t)n_items * slices, 152 * 12), (unsigned)tiles);
-#define DOWN64(CS_)                                                                                         \
-    k_down64<CS_><<<g, kT, 0, st>>>(A->d_down_list, n_items, slices, A->d_parent, E, kron, yhat, sb.claim,    \
-                                    (unsigned*)sb.flag, sb.err, A->k, m, wait_limit())
-    if (CS == 1) DOWN64(1);
-    else if (CS == 2) DOWN64(2);
-    else DOWN64(4);
-#undef DOWN64
-    H2_LAUNCH_CHECK();
-    return 0;
+    return launch_chained(overlap, CS == 1 ? k_down64<1> : (CS == 2 ? k_down64<2> : k_down64<4>), g, kT, 0, st,
+                          A->d_down_list, n_items, slices, A->d_parent, E, kron, yhat, sb.claim, (unsigned*)sb.flag,
+                          sb.err, A->k, m, wait_limit());
 }
 
 int launch_coupling64(h2_matrix* A, const double* S, const double* xhat, double* yhat, int m, bool trans,
-                      cudaStream_t st) {
+                      bool overlap, cudaStream_t st) {
     const int chunks = chunks_of(A->k, m);
     const dim3 g = chunk_grid(A->nc, chunks, m);
-    if (trans)
-        k_coupling64<true><<<g, list_threads(g), 0, st>>>(chunks, A->d_admT_order, A->d_admT_rowptr, A->d_admT_row, A->d_admT_blk, S, xhat,
-                                             yhat, A->k, m);
-    else
-        k_coupling64<false><<<g, list_threads(g), 0, st>>>(chunks, A->d_adm_order, A->d_adm_rowptr, A->d_adm_col, nullptr, S, xhat, yhat,
-                                              A->k, m);
-    H2_LAUNCH_CHECK();
-    return 0;
+    return launch_chained(overlap, trans ? k_coupling64<true> : k_coupling64<false>, g, list_threads(g), 0, st, chunks,
+                          trans ? A->d_admT_order : A->d_adm_order, trans ? A->d_admT_rowptr : A->d_adm_rowptr,
+                          trans ? A->d_admT_row : A->d_adm_col, trans ? A->d_admT_blk : nullptr, S, xhat, yhat, A->k, m);
 }
 
 int launch_leaf64(h2_matrix* A, const double* V, const double* G, const double* yhat, const double* Xp, double* Y,
-                  int64_t ldy, double alpha, int m, bool trans, bool overwrite, cudaStream_t st) {
+                  int64_t ldy, double alpha, int m, bool trans, bool overwrite, bool overlap, cudaStream_t st) {
     const int chunks = chunks_of((int)A->T.leaf_size, m);
     const dim3 g = chunk_grid((int64_t)A->leaves.size(), chunks, m);
-    const int ow = overwrite ? 1 : 0;
-    if (trans)
-        k_leaf64<true><<<g, list_threads(g), 0, st>>>(chunks, A->d_nearT_order, A->d_leaves, A->d_cl_off, A->d_cl_size, A->d_perm, V, yhat,
-                                         A->d_nearT_ptr, A->d_nearT_row, A->d_nearT_blk, A->d_near_off, G, Xp, Y, ldy,
-                                         alpha, A->sigma, A->k, m, ow);
-    else
-        k_leaf64<false><<<g, list_threads(g), 0, st>>>(chunks, A->d_near_order, A->d_leaves, A->d_cl_off, A->d_cl_size, A->d_perm, V, yhat,
-                                          A->d_near_ptr, A->d_near_col, nullptr, A->d_near_off, G, Xp, Y, ldy, alpha,
-                                          A->sigma, A->k, m, ow);
-    H2_LAUNCH_CHECK();
-    return 0;
+    return launch_chained(overlap, trans ? k_leaf64<true> : k_leaf64<false>, g, list_threads(g), 0, st, chunks,
+                          trans ? A->d_nearT_order : A->d_near_order, A->d_leaves, A->d_cl_off, A->d_cl_size, A->d_perm, V,
+                          yhat, trans ? A->d_nearT_ptr : A->d_near_ptr, trans ? A->d_nearT_row : A->d_near_col,
+                          trans ? A->d_nearT_blk : nullptr, A->d_near_off, G, Xp, Y, ldy, alpha, A->sigma, A->k, m,
+                          overwrite ? 1 : 0);
 }
 
 }  // namespace h2
