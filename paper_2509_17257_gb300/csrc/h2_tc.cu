@@ -66,11 +66,14 @@ constexpr int kSplitWarps = 4;  // KIND 1: warps 6..9 write [B; B_lo] into TMEM,
 template <int KIND>
 __host__ __device__ constexpr int tc_issuer2() { return KIND == 1 ? 6 + kSplitWarps : 6; }
 template <int KIND>
-__host__ __device__ constexpr int tc_threads() { return 32 * (tc_issuer2<KIND>() + 1); }
+__host__ __device__ constexpr int tc_producer2() { return KIND == 1 ? tc_issuer2<KIND>() + 1 : 6; }
+template <int KIND>
+__host__ __device__ constexpr int tc_threads() { return 32 * (tc_producer2<KIND>() + 1); }
 constexpr int kAccCols = 64;                // output columns of one term (the matrix tile's rows)
 constexpr int kAccBufs = 4;                 // accumulator buffers: MMAs of a term overlap the epilogue of the 3 before
 // TF32 epilogue: remainder sums handed over, two items deep (64 rows of 64 columns, NARROW 32)
 constexpr int xch_bytes(bool narrow) { return 2 * 64 * (narrow ? 32 : 64) * 4; }
+constexpr int kTermBatch = 8;  // terms that a producer reads at once
 constexpr int kNodeBytes = 64 * 16;        // MODE 2: the source cluster's nodes, in the stage after its activation tile
 // MODE 2: evaluated tiles, two terms deep, rows of 68 floats (16-byte accesses of
 // eight consecutive rows touch all 32 banks once)
@@ -89,38 +92,69 @@ __device__ __forceinline__ uint32_t idesc_for(int M, int N) {
     const uint32_t fmt = KIND == 0 ? 1u : 2u;
     return (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-// One tcgen05.mma (D = A·Bᵀ, or D += A·Bᵀ when acc != 0) from a converged warp:
-// elect.sync hands it to the lowest active lane, so every MMA and commit of the
-// warp comes from one thread, as tcgen05.commit requires.
-template <int KIND>
-__device__ __forceinline__ void mma_issue_elect(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    if (KIND == 0)
-        asm volatile(
-            "{ .reg .pred p, e; setp.ne.b32 p, %4, 0; elect.sync _|e, 0xffffffff;\n"
-            "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p; }" ::"r"(d),
-            "l"(a), "l"(b), "r"(idesc), "r"(acc)
-            : "memory");
-    else
-        asm volatile(
-            "{ .reg .pred p, e; setp.ne.b32 p, %4, 0; elect.sync _|e, 0xffffffff;\n"
-            "@e tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p; }" ::"r"(d),
-            "l"(a), "l"(b), "r"(idesc), "r"(acc)
-            : "memory");
-}
-// The TF32 MMA with its A operand (M = 128 rows, K = 8 columns) in TMEM at
-// column address a_tmem, lanes 0..127.
-__device__ __forceinline__ void mma_tf32_ta_elect(uint32_t d, uint32_t a_tmem, uint64_t b, uint32_t idesc,
-                                                  uint32_t acc) {
+// The MMAs of one term (D = A·Bᵀ, or D += A·Bᵀ when acc != 0) over nk <= 64 / K steps,
+// then up to two commits, from a converged warp: one elect.sync hands them to the
+// lowest active lane, so every MMA and commit of the warp comes from one thread, as
+// tcgen05.commit requires.  One block of code: an elect.sync and fresh descriptors for
+// every MMA cost 80 cycles each.  The descriptors move by 256 bytes a step (two core
+// matrices along K, 16 in their 16-byte units).  bar2 = 0: one commit.
+__device__ __forceinline__ void mma_term_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc, int nk,
+                                              uint32_t bar1, uint32_t bar2) {
+#define H2_STEP(K_)                                                                        \
+    "add.s64 a, a, 16; add.s64 b, b, 16; setp.gt.and.s32 q, %5, " #K_ ", e;\n"             \
+    "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n"
     asm volatile(
-        "{ .reg .pred p, e; setp.ne.b32 p, %4, 0; elect.sync _|e, 0xffffffff;\n"
-        "@e tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p; }" ::"r"(d),
-        "r"(a_tmem), "l"(b), "r"(idesc), "r"(acc)
+        "{ .reg .pred p, e, q, t; .reg .b64 a, b;\n"
+        "elect.sync _|e, 0xffffffff;\n"
+        "setp.ne.b32 p, %4, 0; setp.ge.s32 t, %5, 0; mov.b64 a, %1; mov.b64 b, %2;\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n" H2_STEP(1) H2_STEP(2) H2_STEP(3)
+        "setp.ne.and.b32 q, %7, 0, e;\n"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%6];\n"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%7]; }" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(nk), "r"(bar1), "r"(bar2)
         : "memory");
+#undef H2_STEP
+}
+// The TF32 MMAs with their A operand (M = 128 rows, K = 8 columns a step) in TMEM at
+// column address a, lanes 0..127, from zero; three commits.
+__device__ __forceinline__ void mma_term_tf32(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, int nk, uint32_t bar1,
+                                              uint32_t bar2, uint32_t bar3) {
+#define H2_STEP(K_)                                                                        \
+    "add.s32 a, a, 8; add.s64 b, b, 16; setp.gt.and.s32 q, %4, " #K_ ", e;\n"              \
+    "@q tcgen05.mma.cta_group::1.kind::tf32 [%0], [a], b, %3, t;\n"
+    asm volatile(
+        "{ .reg .pred f, e, q, t; .reg .b64 b; .reg .b32 a;\n"
+        "elect.sync _|e, 0xffffffff;\n"
+        "setp.lt.s32 f, %4, 0; setp.ge.s32 t, %4, 0; mov.b32 a, %1; mov.b64 b, %2;\n"
+        "@e tcgen05.mma.cta_group::1.kind::tf32 [%0], [a], b, %3, f;\n" H2_STEP(1) H2_STEP(2) H2_STEP(3) H2_STEP(4)
+            H2_STEP(5) H2_STEP(6) H2_STEP(7)
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%6];\n"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%7]; }" ::"r"(d),
+        "r"(a), "l"(b), "r"(idesc), "r"(nk), "r"(bar1), "r"(bar2), "r"(bar3)
+        : "memory");
+#undef H2_STEP
 }
 __device__ __forceinline__ void mma_commit_elect(uint64_t* bar) {
     asm volatile(
         "{ .reg .pred e; elect.sync _|e, 0xffffffff;\n"
         "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0]; }" ::"r"(smem_u32(bar))
+        : "memory");
+}
+// One stage from a converged warp (one elected lane): its metadata, the bytes that its
+// barrier expects, and the two bulk copies.
+__device__ __forceinline__ void stage_copy_elect(uint32_t meta, int m0, int m1, int m2, int m3, uint32_t bar, uint32_t dst_a,
+                                                 const void* src_a, uint32_t bytes_a, uint64_t pol_a, uint32_t dst_b,
+                                                 const void* src_b, uint32_t bytes_b, uint64_t pol_b) {
+    asm volatile(
+        "{ .reg .pred e; elect.sync _|e, 0xffffffff;\n"
+        "@e st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n"
+        "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%5], %6;\n"
+        "@e cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%7], [%8], %9, [%5], %10;\n"
+        "@e cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%11], [%12], %13, [%5], "
+        "%14; }" ::"r"(meta),
+        "r"(m0), "r"(m1), "r"(m2), "r"(m3), "r"(bar), "r"(bytes_a + bytes_b), "r"(dst_a), "l"(src_a), "r"(bytes_a),
+        "l"(pol_a), "r"(dst_b), "l"(src_b), "r"(bytes_b), "l"(pol_b)
         : "memory");
 }
 // Named barrier over `count` threads that also ORs a predicate across them.
@@ -318,7 +352,7 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
     const bool COUP_SPLIT = (MODE == 0 || MODE == 2) && p.out_act != nullptr;
     constexpr int ES = KIND == 0 ? 2 : 4;
     constexpr int KSTEP = KIND == 0 ? 16 : 8;  // K of one MMA instruction
-    constexpr int F_FIRST = 1, F_LAST = 2, F_END = 4;
+    constexpr int F_FIRST = 1, F_LAST = 2, F_END = 4, F_PARITY = 8;
     // TMEM: KIND 0 has kAccBufs accumulators of 64 columns.  KIND 1 has
     // accumulators of R columns (64 or 128: 4 or 2 of them, 256 columns) and
     // after them kASlots (4) slots of 64 columns for the MMA's A operand [B; B_lo].
@@ -337,8 +371,10 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
     __shared__ __align__(8) uint64_t accf_bar[kAccBufs], acce_bar[kAccBufs], drain_bar[2], aempty_bar[kASlots];
     __shared__ int s_total;  // terms of this CTA
     __shared__ uint32_t tmem_slot;
-    __shared__ int stage_kp[kSt], stage_np[kSt], stage_fl[kSt], stage_R[kSt];
-    __shared__ int stage_t[MF ? kSt : 1];  // MODE 2: target cluster
+    // a stage's contraction length, flags | output width << 8 (-1: never used), activation
+    // rows, target cluster (MODE 2)
+    __shared__ __align__(16) int4 stage_meta[kSt];
+    __shared__ __align__(16) int4 s_term[2][kTermBatch];  // the producers' current terms
     __shared__ int abort_shared;
     volatile int& abort_flag = abort_shared;
     chain_release();
@@ -351,11 +387,13 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
     const int G = gridDim.x;
     // TMEM columns of one accumulator, and accumulator buffers
     const int acc_cols = KIND == 1 ? (NARROW ? (R <= 32 ? 32 : 64) : (R <= 64 ? 64 : 128)) : kAccCols;
-    const int nacc = KIND == 1 ? A_BASE / acc_cols : kAccBufs;
+    const int nacc = KIND == 1 ? A_BASE / acc_cols : kAccBufs;  // 2 or 4
+    const int lacc = nacc >> 1;                                 // its logarithm
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < nst; ++s) {
             mbar_init(&full_bar[s], 1);
+            stage_meta[s] = make_int4(0, -1, 0, 0);
             mbar_init(&split_bar[s], kSplitWarps);
             mbar_init(&empty_bar[s], 1);
         }
@@ -391,135 +429,121 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
     // launch before still runs
     chain_wait();
 
-    if (warp == 0) {
-        // ---------------- producer ----------------
-        // Item and term descriptors are packed 16-byte records; the next item's
-        // descriptors are loaded while the current item's copies are issued,
-        // so no dependent global load sits between two stages.  Stage
-        // metadata (contraction length, output width, first/last/end flags)
-        // goes to the MMA thread through shared memory, published by the
-        // mbarrier arrive.
-        int stage = 0;
+    if (warp == 0 || warp == tc_producer2<KIND>()) {
+        // ---------------- producers ----------------
+        // Two warps issue the copies, of the terms with an even and with an odd index
+        // among the CTA's: a warp's instructions a term bound the kernel where the copies
+        // do not (one producer with six shuffles a term: 1070 cycles a term at KIND 0,
+        // 2100 at KIND 1, unchanged when the copies were halved).  A batch of term
+        // descriptors (16 bytes each) is loaded while the batch before is issued, and
+        // parked in shared memory: a term costs one read of its descriptor, a wait for its
+        // stage, one store of the stage's metadata (published to the other roles by the
+        // mbarrier arrive) and the copies, all from a converged warp, which keeps the
+        // stage's addresses uniform.  A producer is never more than a stage's use ahead of
+        // the other, so a phase parity names one use.
+        const int me = warp == 0 ? 0 : 1;
+        int stage = me;
         uint32_t phase = 0;
-        uint32_t pend_mask = 0, pend_par = 0;
-        bool aborted = false;
+        bool dead = false;
         const uint64_t pol_keep = l2_policy_evict_last(), pol_stream = l2_policy_evict_first();
         // an item's system: its terms, buffers and sizes (PSYS reads a field of the
         // system table of a multi-system launch, else of the launch's own arguments)
 #define PSYS(it_, f_) ((FLOW && p.sys) ? p.sys[item_sys(it_)].f_ : p.f_)
-        TcItem cur = blockIdx.x < p.n_items ? p.items[blockIdx.x] : TcItem{-1, 0, 0, 0};
-        TcTerm tcur{};
-        if (cur.id >= 0 && lane < cur.e1 - cur.e0) tcur = PSYS(cur, terms)[cur.e0 + lane];
-        for (int w = blockIdx.x; w < p.n_items && !aborted; w += G) {
-            aborted = abort_flag != 0;
-            const int wn = w + G;
-            const TcItem nxt = wn < p.n_items ? p.items[wn] : TcItem{-1, 0, 0, 0};
-            const int nterms = cur.e1 - cur.e0;
-            const int Ri = PSYS(cur, R);
-            for (int base = 0; base < nterms && !aborted; base += 32) {
-                TcTerm t = tcur;
-                if (base > 0) {
-                    t = TcTerm{};
-                    if (base + lane < nterms) t = PSYS(cur, terms)[cur.e0 + base + lane];
-                }
-                const int cnt = min(32, nterms - base);
+        const TcItem none{-1, 0, 0, 0};
+        auto item_at = [&](int w) { return w < p.n_items ? p.items[w] : none; };
+        // the lane's term of the item's terms first, first + 2, ... from the base-th of them
+        auto term_at = [&](const TcItem& it, int first, int base) {
+            const int e = it.e0 + first + 2 * (base + lane);
+            return it.id >= 0 && lane < kTermBatch && e < it.e1 ? __ldg((const int4*)(PSYS(it, terms) + e))
+                                                                : make_int4(0, 0, 0, 0);
+        };
+        TcItem cur = item_at(blockIdx.x), nxt = item_at(blockIdx.x + G);
+        int first = me;  // this producer's first term of the item
+        int4 tnext = term_at(cur, first, 0);
+        for (int w = blockIdx.x; w < p.n_items && !dead; w += G) {
+            if (__any_sync(0xffffffffu, abort_flag != 0)) break;
+            const TcItem after = item_at(w + 2 * G);
+            const int nterms = cur.e1 - cur.e0, own = (nterms - first + 1) >> 1;
+            const int first_n = (first ^ nterms) & 1;
+            const int Ri = PSYS(cur, R), npi = item_np(cur), row_bytes = Ri * ES;
+            const uint8_t *a0 = PSYS(cur, act0), *a1 = PSYS(cur, act1), *a2 = PSYS(cur, act2), *bm = PSYS(cur, bmat);
+            if (own <= 0) tnext = term_at(nxt, first_n, 0);
+            for (int base = 0; base < own && !dead; base += kTermBatch) {
+                const int4 t = tnext;
+                tnext = base + kTermBatch < own ? term_at(cur, first, base + kTermBatch) : term_at(nxt, first_n, 0);
+                const int cnt = min(kTermBatch, own - base);
+                __syncwarp();
+                if (lane < kTermBatch) s_term[me][lane] = t;
                 // Terms that read a tile of this launch wait for its ready flag.  The
                 // lanes poll the flags of the batch's terms together (one round trip
-                // for all), and lane 0 issues a term's copies once its bit is set.
+                // for all), and a term's copies are issued once its bit is set.
                 uint32_t ready_mask = 0xffffffffu;
                 const int* my_flag = nullptr;
                 if (LIST) {
-                    if (lane < cnt && (t.asrc & kTermWait)) my_flag = PSYS(cur, flag) + t.akoff / PSYS(cur, KP);
+                    if (lane < cnt && ((t.w >> 16) & kTermWait)) my_flag = PSYS(cur, flag) + t.z / PSYS(cur, KP);
                     ready_mask = __ballot_sync(0xffffffffu, !my_flag || flag_acquire(my_flag) == p.epoch);
-                    __syncwarp();
                 }
-                const uint64_t t_batch = LIST ? global_ns() : 0;
+                __syncwarp();
+                int4 tj = s_term[me][0];
                 for (int j = 0; j < cnt; ++j) {
-                    const int kpj = __shfl_sync(0xffffffffu, (int)t.kp, j);
-                    const int asj = __shfl_sync(0xffffffffu, (int)t.asrc, j);
-                    const int64_t bj = __shfl_sync(0xffffffffu, t.boff, j);
-                    const int akj = __shfl_sync(0xffffffffu, t.akoff, j);
-                    const int64_t aj = (int64_t)akj * Ri * ES;
-                    bool ready = true;
+                    const int kpj = (int16_t)tj.w, asj = tj.w >> 16, akj = tj.z;
+                    const int64_t bj = (int64_t)(((uint64_t)(uint32_t)tj.y << 32) | (uint32_t)tj.x);
+                    if (j + 1 < cnt) tj = s_term[me][j + 1];
                     if (LIST && !((ready_mask >> j) & 1u)) {
                         // poll again (bounded: gives up after about one second)
+                        const uint64_t t0 = global_ns();
                         while (true) {
                             __nanosleep(32);
                             ready_mask |= __ballot_sync(0xffffffffu, my_flag && flag_acquire(my_flag) == p.epoch);
                             __syncwarp();
                             if ((ready_mask >> j) & 1u) break;
-                            if (__any_sync(0xffffffffu, abort_flag || global_ns() - t_batch > 1000000000ull)) {
-                                ready = false;  // warp-uniform: every lane leaves together
+                            if (__any_sync(0xffffffffu, abort_flag || global_ns() - t0 > 1000000000ull)) {
+                                dead = true;  // warp-uniform: every lane leaves together
                                 break;
                             }
                         }
                     }
-                    int bad = 0;
-                    if (lane == 0) {
-                        // the flags acquired by the warp order the tiles' writes before this copy
-                        if (LIST && (asj & kTermWait)) fence_proxy_async_global();
-                        if (!ready || !mbar_wait(&empty_bar[stage], phase ^ 1)) {
-                            bad = 1;
-                        } else {
-                            const uint32_t ab = (uint32_t)(Ri * kpj * ES);
-                            const uint32_t bb = (uint32_t)(item_np(cur) * kpj * ES);
-                            uint8_t* sA = smem + stage * stage_bytes;
-                            uint8_t* sB = sA + a_bytes;
-                            stage_kp[stage] = kpj;
-                            stage_np[stage] = item_np(cur);
-                            stage_R[stage] = Ri;
-                            stage_fl[stage] = (base + j == 0 ? F_FIRST : 0) | (base + j == nterms - 1 ? F_LAST : 0);
-                            if (MF) {
-                                // the source cluster's nodes: cluster s's rows and nodes start at s·KP
-                                const uint32_t nb = (uint32_t)(p.KP * 16);
-                                stage_t[stage] = cur.id;
-                                mbar_expect_tx(&full_bar[stage], ab + nb);
-                                bulk_g2s(sA, (asj ? p.act1 : p.act0) + aj, ab, &full_bar[stage]);
-                                bulk_g2s(sB, p.nodes + akj, nb, &full_bar[stage]);
-                            } else {
-                                mbar_expect_tx(&full_bar[stage], ab + bb);
-                                const uint8_t* asrc = (asj & 3) == 0 ? PSYS(cur, act0)
-                                                                     : ((asj & 3) == 1 ? PSYS(cur, act1) : PSYS(cur, act2));
-                                // the activation tiles are read by many terms, the matrix tiles once
-                                bulk_g2s_hint(sA, asrc + aj, ab, &full_bar[stage], pol_keep);
-                                bulk_g2s_hint(sB, PSYS(cur, bmat) + bj * (ES / 2), bb, &full_bar[stage], pol_stream);
-                            }
-                            pend_mask |= 1u << stage;
-                            pend_par = (pend_par & ~(1u << stage)) | (phase << stage);
-                        }
-                    }
-                    if (__shfl_sync(0xffffffffu, bad, 0)) {
+                    // the flags acquired by the warp order the tiles' writes before this copy
+                    if (LIST && (asj & kTermWait)) fence_proxy_async_global();
+                    if (dead || !__any_sync(0xffffffffu, mbar_wait(&empty_bar[stage], phase ^ 1))) {
+                        dead = true;
                         if (lane == 0) atomicExch(p.err, 1);
                         abort_flag = 1;
-                        aborted = true;
                         break;
                     }
-                    if (++stage == nst) { stage = 0; phase ^= 1; }
+                    const uint32_t ab = (uint32_t)(row_bytes * kpj);
+                    const uint32_t sA = smem_u32(smem + stage * stage_bytes), bar = smem_u32(&full_bar[stage]);
+                    const int term = first + 2 * (base + j);
+                    const int fl = (term == 0 ? F_FIRST : 0) | (term == nterms - 1 ? F_LAST : 0) | (phase ? F_PARITY : 0);
+                    const int64_t aj = (int64_t)akj * row_bytes;
+                    // the activation tiles are read by many terms, the matrix tiles once; MODE 2
+                    // copies the source cluster's nodes (its rows and nodes start at s·KP)
+                    const uint8_t* asrc = ((asj & 3) == 0 ? a0 : ((asj & 3) == 1 ? a1 : a2)) + aj;
+                    const uint8_t* bsrc = MF ? (const uint8_t*)(p.nodes + akj) : bm + bj * (ES / 2);
+                    const uint32_t bb = MF ? (uint32_t)(p.KP * 16) : (uint32_t)(npi * kpj * ES);
+                    stage_copy_elect(smem_u32(&stage_meta[stage]), kpj, fl | (npi << 8), Ri, cur.id, bar, sA, asrc, ab,
+                                     pol_keep, sA + a_bytes, bsrc, bb, MF ? pol_keep : pol_stream);
+                    stage += 2;
+                    if (stage >= nst) { stage -= nst; phase ^= 1; }
                 }
             }
-            tcur = TcTerm{};
-            if (nxt.id >= 0 && lane < nxt.e1 - nxt.e0) tcur = PSYS(nxt, terms)[nxt.e0 + lane];
             cur = nxt;
+            nxt = after;
+            first = first_n;
         }
-        if (lane == 0) {
-            // end marker for the MMA thread (and the splitters): a stage without data
+        __syncwarp();
+        // the splitters' end marker, a stage without data, comes from the next term's producer
+        if (lane == 0 && !dead && (s_total & 1) == me) {
             if (mbar_wait(&empty_bar[stage], phase ^ 1)) {
-                // the stage is free, so its earlier copy has landed and been consumed;
-                // the marker moves its barrier on, so it leaves the drain set
-                pend_mask &= ~(1u << stage);
-                stage_fl[stage] = F_END;
+                stage_meta[stage] = make_int4(0, F_END | (phase ? F_PARITY : 0), 0, 0);
                 mbar_arrive(&full_bar[stage]);
             } else {
                 atomicExch(p.err, 1);
                 abort_flag = 1;
             }
-            // every copy issued by this CTA lands before the CTA exits
-            for (int s2 = 0; s2 < nst; ++s2)
-                if ((pend_mask >> s2) & 1u)
-                    if (!mbar_wait(&full_bar[s2], (pend_par >> s2) & 1u)) atomicExch(p.err, 2);
         }
 #undef PSYS
-    } else if (warp == 1 || warp == tc_issuer2<KIND>()) {
+    } else if (warp == 1 || (KIND == 1 && warp == tc_issuer2<KIND>())) {
         // ---------------- MMA issuers: driven by the stage metadata ----------------
         // Two warps take the terms by parity (term t uses stage t mod nst,
         // accumulator t mod nacc and A slot t mod kASlots), so one warp's waits
@@ -535,16 +559,16 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
             // an item in one TMEM accumulator (an item's first term starts it from
             // zero); the epilogue reads each accumulator once per item.  The FP32
             // accumulation of the tensor cores is far finer than the BF16 operands.
-            int item_idx = 0, acc = 0;
+            int item_idx = 0, acc = 0, stage = 0;
+            uint32_t phase = 0;
             for (int it = 0; it < T; ++it) {
-                const int stage = it % nst;
-                const uint32_t phase = (uint32_t)(it / nst) & 1u;
                 if (!__any_sync(0xffffffffu, mbar_wait(&full_bar[stage], phase))) {
                     abort_flag = 1;
                     if (lane == 0) atomicExch(p.err, 4);
                     break;
                 }
-                const int fl = stage_fl[stage];
+                const int4 mt = stage_meta[stage];
+                const int fl = mt.y;
                 if (fl & F_FIRST) {
                     acc = item_idx % kAccBufs;
                     if (!__any_sync(0xffffffffu, mbar_wait(&acce_bar[acc], ((item_idx / kAccBufs) & 1) ^ 1))) {
@@ -555,26 +579,15 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
                 }
                 tc_fence_after();
                 const uint32_t d = tmem + (uint32_t)(acc * acc_cols);
-                const int kp = stage_kp[stage];
+                const int kp = mt.x;
                 const uint32_t sA = smem_u32(smem + stage * stage_bytes);
-                const uint32_t sB = sA + a_bytes;
                 const uint32_t sbo = (uint32_t)(kp * ES / 16) * 128;
-                const uint32_t idesc = idesc_for<KIND>(M, stage_np[stage]);
-                const uint64_t ad0 = smem_desc(sA, 128, sbo);
-                const uint64_t bd0 = smem_desc(sB, 128, sbo);
-                const int nk = kp / KSTEP;
-#pragma unroll
-                for (int kk = 0; kk < 64 / KSTEP; ++kk) {
-                    if (kk >= nk) break;
-                    const uint64_t off = (uint64_t)(kk * 16);
-                    mma_issue_elect<KIND>(d, ad0 + off, bd0 + off, idesc, (kk == 0 && (fl & F_FIRST)) ? 0u : 1u);
-                }
+                mma_term_bf16(d, smem_desc(sA, 128, sbo), smem_desc(sA + a_bytes, 128, sbo), idesc_for<KIND>(M, (fl >> 8) & 255),
+                              (fl & F_FIRST) ? 0u : 1u, kp / KSTEP, smem_u32(&empty_bar[stage]),
+                              (fl & F_LAST) ? smem_u32(&accf_bar[acc]) : 0u);
                 issued = true;
-                mma_commit_elect(&empty_bar[stage]);
-                if (fl & F_LAST) {
-                    mma_commit_elect(&accf_bar[acc]);
-                    ++item_idx;
-                }
+                if (fl & F_LAST) ++item_idx;
+                if (++stage == nst) { stage = 0; phase ^= 1; }
             }
             if (issued) {
                 mma_commit_elect(&drain_bar[0]);
@@ -582,10 +595,11 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
                 issued = false;  // drained
             }
         }
+        int stage = j;
+        uint32_t phase = 0;
+        if (stage >= nst) { stage -= nst; phase ^= 1; }
         for (int it = j; it < T && KIND == 1; it += 2) {
-            const int stage = it % nst;
-            const uint32_t phase = (uint32_t)(it / nst) & 1u;
-            if (!__any_sync(0xffffffffu, mbar_wait(KIND == 1 ? &split_bar[stage] : &full_bar[stage], phase))) {
+            if (!__any_sync(0xffffffffu, mbar_wait(&split_bar[stage], phase))) {
                 abort_flag = 1;
                 if (lane == 0) atomicExch(p.err, 4);
                 break;
@@ -593,46 +607,28 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
             // every term accumulates from zero in its own TMEM buffer; the epilogue
             // adds the terms of an item in FP32 registers (round to nearest), so
             // the tensor-core accumulator never sums more than one term's K steps
-            const int acc = it % nacc;
-            if (!__any_sync(0xffffffffu, mbar_wait(&acce_bar[acc], ((it / nacc) & 1) ^ 1))) {
+            const int acc = it & (nacc - 1);
+            if (!__any_sync(0xffffffffu, mbar_wait(&acce_bar[acc], ((it >> lacc) & 1) ^ 1))) {
                 abort_flag = 1;
                 if (lane == 0) atomicExch(p.err, 3);
                 break;
             }
             tc_fence_after();
             const uint32_t d = tmem + (uint32_t)(acc * acc_cols);
-            const int kp = stage_kp[stage];
-            const uint32_t sA = smem_u32(smem + stage * stage_bytes);
-            const uint32_t sB = sA + a_bytes;
-            const uint32_t sbo = (uint32_t)(kp * ES / 16) * 128;
-            // KIND 0: D[r, n] = act · matᵀ (M = activation rows, N = the tile's rows),
-            // both operands in shared memory.
-            // KIND 1: D[n, r] = [mat; mat_lo] · actᵀ: M = 128, the tile (rows 0..63)
-            // and its TF32 remainder (rows 64..127), which the splitter warps have
-            // put into TMEM slot `as`; N = R activation rows from shared memory.
-            // The MMA time grows with N, not with M up to 128, so the remainder
-            // costs no extra instructions.  Rows np..63 of either part hold stale
-            // data whose TMEM lanes the epilogue ignores.
-            const uint32_t idesc = KIND == 1 ? idesc_for<KIND>(128, stage_R[stage]) : idesc_for<KIND>(M, stage_np[stage]);
-            // descriptors of K step kk: the start address field moves by 256 bytes
-            // (two core matrices along K), i.e. 16 in its 16-byte units; a TMEM
-            // operand moves by KSTEP columns
-            const uint64_t ad0 = smem_desc(sA, 128, sbo);
-            const uint64_t bd0 = smem_desc(sB, 128, sbo);
+            const int4 mt = stage_meta[stage];
+            const uint32_t sbo = (uint32_t)(mt.x * ES / 16) * 128;
+            // D[n, r] = [mat; mat_lo] · actᵀ: M = 128, the tile (rows 0..63) and its TF32
+            // remainder (rows 64..127), which the splitter warps have put into TMEM slot
+            // `as`; N = R activation rows from shared memory.  The MMA time grows with N,
+            // not with M up to 128, so the remainder costs no extra instructions.  Rows
+            // np..63 of either part hold stale data whose TMEM lanes the epilogue ignores.
             const int as = it % kASlots;
-            const uint32_t a_tmem = tmem + (uint32_t)(A_BASE + 64 * as);
-            const int nk = kp / KSTEP;
-#pragma unroll
-            for (int kk = 0; kk < 64 / KSTEP; ++kk) {
-                if (kk >= nk) break;
-                const uint64_t off = (uint64_t)(kk * 16);
-                if (KIND == 1) mma_tf32_ta_elect(d, a_tmem + (uint32_t)(kk * KSTEP), ad0 + off, idesc, kk == 0 ? 0u : 1u);
-                else mma_issue_elect<KIND>(d, ad0 + off, bd0 + off, idesc, kk == 0 ? 0u : 1u);
-            }
+            mma_term_tf32(d, tmem + (uint32_t)(A_BASE + 64 * as), smem_desc(smem_u32(smem + stage * stage_bytes), 128, sbo),
+                          idesc_for<KIND>(128, mt.z), mt.x / KSTEP, smem_u32(&empty_bar[stage]), smem_u32(&aempty_bar[as]),
+                          smem_u32(&accf_bar[acc]));
             issued = true;
-            mma_commit_elect(&empty_bar[stage]);
-            if (KIND == 1) mma_commit_elect(&aempty_bar[as]);
-            mma_commit_elect(&accf_bar[acc]);
+            stage += 2;
+            while (stage >= nst) { stage -= nst; phase ^= 1; }
         }
         if (issued) {
             mma_commit_elect(&drain_bar[j]);
@@ -692,8 +688,8 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
                     imask = __ballot_sync(0xffffffffu, tt < nterms && (p.terms[cur.e0 + tt].asrc & kTermImag));
                 }
                 const bool imag = (imask >> (term & 31)) & 1u;
-                const int acc = it % nacc;
-                if (!__any_sync(0xffffffffu, mbar_wait(&accf_bar[acc], (it / nacc) & 1))) {
+                const int acc = it & (nacc - 1);
+                if (!__any_sync(0xffffffffu, mbar_wait(&accf_bar[acc], (it >> lacc) & 1))) {
                     failed = true;
                     break;
                 }
@@ -995,14 +991,15 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
         int xt_of = -1;
         while (true) {
             bool ok = pre || __any_sync(0xffffffffu, mbar_wait(&full_bar[stage], phase));
-            const int fl = ok ? stage_fl[stage] : 0;
+            const int4 mt = ok ? stage_meta[stage] : make_int4(0, 0, 0, 0);
+            const int fl = mt.y;
             const bool end = ok && (fl & F_END);
             const int as = sit % kASlots;
             // the slot is free once the MMAs of term sit - kASlots have completed
             if (ok && !end && !pre) ok = __any_sync(0xffffffffu, mbar_wait(&aempty_bar[as], ((sit / kASlots) & 1) ^ 1));
             pre = false;
             if (ok && !end) tc_fence_after();
-            const int kp = ok ? stage_kp[stage] : 0;
+            const int kp = mt.x;
             // MODE 2: row n of the evaluated tile, two terms deep (a warp is past the
             // barrier of term t + 1 only when its partner has read term t's tile)
             float* xrow = (float*)(smem + nst * stage_bytes + (sit & 1) * (kEvalBytes / 2)) + n * kEvalLd;
@@ -1020,8 +1017,8 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
                 // with scaled nodes, a square root and 16-byte exchanges.
                 if (ok && !end) {
                     const bool rv = n < p.k;
-                    if (stage_t[stage] != xt_of) {
-                        xt_of = stage_t[stage];
+                    if (mt.w != xt_of) {
+                        xt_of = mt.w;
                         xt = p.nodes[(int64_t)xt_of * p.KP + (rv ? n : 0)];
                     }
                     const int half = p.KP >> 1, mu0 = lo_part ? half : 0;
@@ -1097,6 +1094,10 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    // every copy lands before the CTA exits: the last use of each stage, whose parity
+    // its metadata holds
+    if (threadIdx.x < nst && stage_meta[threadIdx.x].y != -1)
+        if (!mbar_wait(&full_bar[threadIdx.x], (stage_meta[threadIdx.x].y & F_PARITY) ? 1u : 0u)) atomicExch(p.err, 2);
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
 }
