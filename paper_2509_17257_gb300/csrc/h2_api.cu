@@ -319,7 +319,7 @@ int h2_info(const h2_matrix* A, h2_info_t* info) {
     // both passes, coupling, leaf phase, scatter into Y.  Without: gather, upward pass, coupling,
     // downward pass, leaf phase, scatter, three packing launches, + zeroing of clusters without couplings
     const bool pairs = A->pairs_built && A->use_kron;
-    const bool hybrid = pairs && (A->tc.hybrid || A->tc.hybrid_bf16) && A->tc.h_default;
+    const bool hybrid = pairs && A->tc.hybrid && A->tc.h_default;
     info->launches_tc = 0;
     if (A->tc.built && pairs)
         info->launches_tc = 4 + (int32_t)(A->down_pairs.stages.size() +

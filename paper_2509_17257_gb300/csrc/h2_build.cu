@@ -232,22 +232,6 @@ int upload(h2_matrix* A, T** dst, const std::vector<T>& src, cudaStream_t st) {
     return 0;
 }
 
-// Lays out a work list sorted by decreasing cost for a kernel whose CTA b
-// takes positions b, b + G, b + 2G, ...: round r of G items goes to the CTAs
-// in order for even r and in reverse for odd r (the last, partial round in
-// order), so no CTA takes the largest item of every round.
-void snake_order(std::vector<TcItem>& v, int G) {
-    const size_t n = v.size();
-    if (G < 2 || n <= (size_t)G) return;
-    std::vector<TcItem> out(n);
-    for (size_t i = 0; i < n; ++i) {
-        const size_t r = i / G, j = i % G;
-        const bool full = (r + 1) * G <= n;
-        out[r * G + ((r & 1) && full ? G - 1 - j : j)] = v[i];
-    }
-    v.swap(out);
-}
-
 // A term's fixed cost in the balance of the tensor-core work lists, in units of
 // tile elements (a full 64×64 tile adds a third of it): a term's copies and
 // hand-offs take nearly as long whatever its tile's size.
@@ -781,27 +765,38 @@ void flow_tiles(h2_matrix* A, std::vector<TcPackTile>& tiles, int64_t& off, Flow
     off += (int64_t)NP * KP * 2;
 }
 
-// Items with their sort keys, dealt in snake order over the CTAs within each key.
+// Items with their sort keys, in order of the keys; the items of one key do not wait
+// for each other.  Position r·G + c of the list runs on CTA c of G: every stretch of
+// one key within a round is dealt largest item first to the CTA with the fewest
+// terms so far.
 struct KeyedItem {
     int32_t key;
     TcItem it;
 };
 void order_by_key(std::vector<KeyedItem>& v, std::vector<TcItem>& out) {
+    constexpr size_t G = kTcDeal;
     std::stable_sort(v.begin(), v.end(), [](const KeyedItem& a, const KeyedItem& b) { return a.key < b.key; });
-    out.clear();
-    std::vector<TcItem> group;
+    out.resize(v.size());
+    std::vector<int64_t> load(G, 0);
+    std::vector<size_t> cta, src;
     for (size_t i = 0; i < v.size();) {
         size_t j = i;
-        group.clear();
-        while (j < v.size() && v[j].key == v[i].key) group.push_back(v[j++].it);
-        snake_order(group, kTcGrid);
-        out.insert(out.end(), group.begin(), group.end());
+        while (j < v.size() && v[j].key == v[i].key && j / G == i / G) ++j;
+        cta.clear();
+        src.clear();
+        for (size_t e = i; e < j; ++e) { cta.push_back(e % G); src.push_back(e); }
+        auto terms = [&](size_t e) { return (int64_t)v[e].it.e1 - v[e].it.e0; };
+        std::stable_sort(cta.begin(), cta.end(), [&](size_t a, size_t b) { return load[a] < load[b]; });
+        std::stable_sort(src.begin(), src.end(), [&](size_t a, size_t b) { return terms(a) > terms(b); });
+        for (size_t e = 0; e < cta.size(); ++e) {
+            out[i / G * G + cta[e]] = v[src[e]].it;
+            load[cta[e]] += terms(src[e]);
+        }
         i = j;
     }
 }
 
-// Items of several work lists merged by key (snake order over the CTAs within a
-// key), for the multi-system launches of h2_batch_matmul.
+// Items of several work lists merged by key (dealt as in order_by_key), for the multi-system launches of h2_batch_matmul.
 void merge_by_key(const std::vector<int32_t>& keys, const std::vector<TcItem>& items, std::vector<TcItem>& out) {
     std::vector<KeyedItem> v(keys.size());
     for (size_t i = 0; i < keys.size(); ++i) v[i] = KeyedItem{keys[i], items[i]};
@@ -942,7 +937,11 @@ constexpr int kHybridRoundTerms = 16;  // H2_HYBRID_ROUND_TERMS overrides it (1.
 // The product takes the hybrid upward pass by default when the coupling work
 // that reads no cluster above the cut gives every CTA at least this many terms
 // per height above the cut: then the chain of transfer items (a few
-// microseconds per height) runs under that work instead of after it.
+// microseconds per height) runs under that work instead of after it.  FP32, q = 4,
+// m = 32, without → with (µs): 8 terms per height (n = 20011) 120 → 123, 10 (24000)
+// 132 → 130, 13 (24000, ellipsoid) 142 → 136, 17 (32768) 175 → 170, 27 (65536)
+// 296 → 291.  The BF16 product does not take it: its coupling terms are as short as
+// the chain's steps (n = 16384: 79 → 91, 65536: 191 → 194, 262144, m = 16: 525 → 526).
 constexpr int kHybridTermsPerHeight = 12;
 
 int hybrid_lists(h2_matrix* A, cudaStream_t st) {
@@ -1022,7 +1021,7 @@ int hybrid_lists(h2_matrix* A, cudaStream_t st) {
             }
         }
         // the rest, and the coupling items that read clusters above the cut: largest
-        // first (snake-dealt within the key)
+        // first
         std::vector<Free> rest(free_items.begin() + (long)i, free_items.end());
         rest.insert(rest.end(), late.begin(), late.end());
         std::stable_sort(rest.begin(), rest.end(), [](const Free& a, const Free& b) { return a.cost > b.cost; });
@@ -1201,7 +1200,7 @@ int build_tc(h2_matrix* A, bool bf16, bool tf32, cudaStream_t st) {
         else c_zero.push_back((int32_t)c);
     }
     // longest lists first, each to the CTA with the least work so far
-    balance_order(c_items, [](const TcItem& a) { return (int64_t)(a.e1 - a.e0); }, kTcGrid);
+    balance_order(c_items, [](const TcItem& a) { return (int64_t)(a.e1 - a.e0); }, kTcDeal);
     // ---- leaf schedule: outputs = leaf positions; terms = V_t ŷ_t, then G_b X|_ŝ ----
     std::vector<int64_t> xkoff(NL + 1, 0);
     std::vector<int32_t> leaf_base(NL), leaf_kdim(NL);
@@ -1234,7 +1233,7 @@ int build_tc(h2_matrix* A, bool bf16, bool tf32, cudaStream_t st) {
             l_items[lp] = TcItem{(int32_t)lp, e0, (int32_t)l_terms.size(), l_np[lp]};
         }
     }
-    balance_order(l_items, [&](const TcItem& a) { return l_cost[a.id]; }, kTcGrid);
+    balance_order(l_items, [&](const TcItem& a) { return l_cost[a.id]; }, kTcDeal);
     D.s_off_host = s_off;
     D.et_off_host.clear();
     if (flow) {
@@ -1346,7 +1345,7 @@ int build_tc_transposed(h2_matrix* A, cudaStream_t st) {
             else c_zero.push_back((int32_t)sc);
         }
     }
-    balance_order(c_items, [](const TcItem& a) { return (int64_t)(a.e1 - a.e0); }, kTcGrid);
+    balance_order(c_items, [](const TcItem& a) { return (int64_t)(a.e1 - a.e0); }, kTcDeal);
     // ---- leaf list over column leaves: item s, terms V_s ŷ_s, then G_bᵀ x|_t̂ ----
     std::vector<int64_t> xkoff(NL + 1, 0);
     for (int64_t lp = 0; lp < NL; ++lp) xkoff[lp + 1] = xkoff[lp] + round16((int)T.size[A->leaves[lp]]);
@@ -1369,7 +1368,7 @@ int build_tc_transposed(h2_matrix* A, cudaStream_t st) {
         }
         l_items[lp] = TcItem{(int32_t)lp, e0, (int32_t)l_terms.size(), np};
     }
-    balance_order(l_items, [&](const TcItem& a) { return l_cost[a.id]; }, kTcGrid);
+    balance_order(l_items, [&](const TcItem& a) { return l_cost[a.id]; }, kTcDeal);
     D.ct_nitems = (int)c_items.size();
     D.ct_nzero = (int)c_zero.size();
     D.lt_nitems = (int)NL;

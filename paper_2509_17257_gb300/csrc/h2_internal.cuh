@@ -267,7 +267,11 @@ struct DownStep {
     int32_t c, rd, wr, flags;
 };
 constexpr int kDownLoad = 1, kDownStore = 2;
-constexpr int kTcGrid = 152;  // CTAs of the tensor-core kernels (one per SM); their work lists are laid out for it
+constexpr int kTcGrid = 152;  // CTAs of the tensor-core kernels, one per SM (narrow instances: two)
+// The work lists are laid out for two CTAs per SM; with one, CTA c takes the shares of
+// c and c + kTcGrid.  Dealt for one (m = 32, n = 65536, q = 4), the 304 CTAs of the
+// coupling had 105 to 131 terms and those of the leaf phase 62 to 80.
+constexpr int kTcDeal = 2 * kTcGrid;
 constexpr int kDownMaxSteps = 192;  // steps of one task at most (the schedule keeps to it)
 
 // One step of the upward subtree schedule (up_schedule): a leaf c (rd0 < 0, rd1 =

@@ -874,7 +874,7 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
         // hybrid: the upward lists stop at their first cut, and the clusters above it
         // are transfer items of the coupling launch (k_tc_gemm<4, KIND>), which waits
         // for them only where a coupling reads them
-        bool want_hybrid = tn.path == kPathTcHybrid || (tn.path == kPathDefault && D.h_default);
+        bool want_hybrid = tn.path == kPathTcHybrid || (tn.path == kPathDefault && kind == 1 && D.h_default);
         if (A->use_hybrid >= 0) want_hybrid = A->use_hybrid == 1;
         const bool lists = kind == 1 ? D.hybrid : D.hybrid_bf16;
         const bool hybrid = fast && !flow && !trans && !mf && !cx && lists && want_hybrid && !capturing;
