@@ -582,8 +582,8 @@ def run_ours(args):
             solve["speedup_fastest_mixed_vs_fastest_fp64"] = round(fp64[best_f] / mixed[best_m], 3)
 
     # the batch workload: 64 independent systems (ellipsoids, n log-uniform in [2048, 32768],
-    # m in 1..64, q in {3, 4}); one FP32 product of all of them per step, in two multi-system
-    # launches (upward + coupling, downward + leaf) between the systems' gathers and scatters
+    # m in 1..64, q in {3, 4}); one FP32 product of all of them per step, one CUDA graph with
+    # a branch per system
     batch = None
     if not args.no_batch and workload == WORKLOAD:
         batch = batch_products(P, torch, dev, steps=max(5, min(args.steps, 20)), dist=dist)
@@ -714,8 +714,7 @@ def batch_products(P, torch, dev, steps: int, dist=None) -> dict:
     out = {"systems": len(specs), "total_n": sum(sp["n"] for sp in specs),
            "total_columns": sum(sp["m"] for sp in specs), "gflop_per_product": round(flops / 1e9, 3),
            "ms_per_product": round(ms, 4), "value": round(flops / (ms * 1e-3) / 1e9, 1), "unit": "GFLOP/s",
-           "steps": steps, "launch": "two multi-system tensor-core launches per product (upward pass + coupling, "
-                                     "downward pass + leaf phase) plus per-system gathers and scatters, one CUDA graph"}
+           "steps": steps, "launch": "one CUDA graph with a branch per system"}
     Bt.close()
     for mm in mats:
         mm.close()

@@ -1,5 +1,5 @@
 // Batches of independent systems: products captured into one CUDA graph with
-// one branch per system, and the autotuner that picks the FP32 product path.
+// one branch per system or (flow_batch_ok) two launches over all systems, and the autotuner that picks the FP32 product path.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -184,10 +184,20 @@ int flow_capture(h2_batch* b, const std::vector<int>& sys, const TcGemmParams& p
     return 0;
 }
 
+// Whether a batch takes the multi-system launches: FP32, when some system has no lists
+// of transfer pairs (its own branch would pass level by level).  With the pairs a
+// branch per system is faster, branches running side by side with the column tiles
+// that suit each system (µs, multi-system → branches): 16 systems, n = 2048..32768,
+// m <= 64: 1081 → 867; 12, n <= 20619, m <= 6: 442 → 382; 8, n <= 11761, m <= 12:
+// 263 → 203; 2, n <= 14412, m <= 33: 117 → 79.
 bool flow_batch_ok(h2_batch* b, const std::vector<int>& sys, const int64_t* m, int32_t dtype) {
-    bool multi = dtype == H2_F32 && b->multi_launch;
-    for (int i : sys) multi = multi && flow_batchable(b->mats[i], m[i]) && b->mats[i]->use_flow != 0;
-    return multi;
+    bool multi = dtype == H2_F32 && b->multi_launch, pairs = true;
+    for (int i : sys) {
+        const h2_matrix* A = b->mats[i];
+        multi = multi && flow_batchable(b->mats[i], m[i]) && A->use_flow != 0;
+        pairs = pairs && A->pairs_built && A->use_kron && A->use_flow != 1;
+    }
+    return multi && !pairs;
 }
 
 namespace {
@@ -305,7 +315,7 @@ int h2_batch_matmul(h2_batch* b, double alpha, const double* const* X, const int
     if (sys.empty()) return 0;
     // the graph runs on the batch's own stream, ordered after and before the caller's stream
     H2_CUDA_TRY(cudaEventRecord(b->ev_in, st));
-    // FP32 with the tensor-core transfer passes on every system: multi-system launches
+    // FP32 with a system without transfer pairs: multi-system launches with the tensor-core transfer passes
     if (flow_batch_ok(b, sys, m, dtype)) {
         H2_CUDA_TRY(cudaStreamWaitEvent(b->origin, b->ev_in, 0));
         int rc = batch_flow_matmul(b, alpha, X, ldx, Y, ldy, m, sys);

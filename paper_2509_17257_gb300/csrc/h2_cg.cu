@@ -938,9 +938,9 @@ int batch_block_cg(h2_batch* b, const double* const* B, const int64_t* ldb, doub
     cudaGraphExec_t exec = nullptr;
     std::vector<int> in_graph;
     int status = 0, it = 0;
-    // FP32 products of every system in two multi-system launches per iteration
-    // (the upward pass with the coupling phase, the downward pass with the leaf
-    // phase), when every system can take them; their buffers are sized once here
+    // where flow_batch_ok says so, FP32 products of every system in two multi-system
+    // launches per iteration (the upward pass with the coupling phase, the downward
+    // pass with the leaf phase); their buffers are sized once here
     std::vector<int> all_active;
     for (int i = 0; i < count; ++i) if (!sys[i].done) all_active.push_back(i);
     const bool multi = !all_active.empty() && flow_batch_ok(b, all_active, m, dtype);

@@ -525,8 +525,9 @@ struct h2_batch {
     cudaGraphExec_t mm_exec = nullptr;  // cached product graph
     std::vector<int64_t> mm_key;
     // FP32 products whose upward/coupling and downward/leaf phases run as one
-    // launch each over the items of every system (multi-system work lists)
-    bool multi_launch = true;  // H2_BATCH_MULTI=0 at h2_batch_create: one graph branch per system instead
+    // launch each over the items of every system (multi-system work lists), where
+    // flow_batch_ok says so
+    bool multi_launch = true;  // H2_BATCH_MULTI=0 at h2_batch_create: always one graph branch per system
     cudaGraphExec_t flow_exec = nullptr;
     std::vector<int64_t> flow_key;
     void* flow_mem = nullptr;  // merged item lists and system tables on the device
@@ -578,8 +579,8 @@ int flow_prepare(h2_matrix* A, int m, cudaStream_t st, FlowBufs* fb);
 int flow_pre(h2_matrix* A, const double* X, int64_t ldx, const FlowBufs& fb, cudaStream_t st);
 int flow_post(h2_matrix* A, double alpha, const double* X, int64_t ldx, double* Y, int64_t ldy, const FlowBufs& fb,
               bool overwrite, cudaStream_t st);
-// Multi-system FP32 products of a batch (h2_batch.cu): whether every system of
-// sys can take them, their work lists and tables, and their graph capture.
+// Multi-system FP32 products of a batch (h2_batch.cu): whether the systems of
+// sys take them, their work lists and tables, and their graph capture.
 bool flow_batch_ok(h2_batch* b, const std::vector<int>& sys, const int64_t* m, int32_t dtype);
 int flow_tables(h2_batch* b, const std::vector<int>& sys, const std::vector<FlowBufs>& fb, void** mem, size_t* bytes,
                 TcGemmParams* p1, TcGemmParams* p2, cudaStream_t st);

@@ -1,0 +1,39 @@
+"""The two routes of an FP32 batch: a graph branch per system where every system has lists of transfer pairs, the
+multi-system launches where one has not (H2_KRON=0 leaves it without), and both kinds in one batch."""
+import pytest
+
+from _helpers import rel_fro, require_cuda
+from workloads import ellipsoid_points, gaussian_rhs
+
+pytestmark = pytest.mark.gpu
+
+SIZES = [(700, 3, 1), (1531, 4, 33), (900, 2, 64), (3001, 4, 16)]  # n, q, m
+
+
+@pytest.mark.parametrize("no_pairs", [(), (0, 1, 2, 3), (2,)], ids=["branches", "multi", "mixed"])
+def test_batch_routes_equal_single_fp64_products(no_pairs, monkeypatch):
+    torch = require_cuda()
+    import paper_2509_17257_gb300.build as bld
+    bld.build()
+    import paper_2509_17257_gb300 as P
+    mats = []
+    for i, (n, q, _) in enumerate(SIZES):
+        if i in no_pairs:
+            monkeypatch.setenv("H2_KRON", "0")
+        else:
+            monkeypatch.delenv("H2_KRON", raising=False)
+        mats.append(P.H2Matrix(ellipsoid_points(n, (1.0, 0.7, 0.5), 40 + i), q=q, leaf_size=64, eta=2.0, sigma=1e-2,
+                               precisions=("f32",)))
+    B = P.H2Batch(mats)
+    for seed in (1, 2):  # new buffers each time
+        X = [torch.from_numpy(gaussian_rhs(n, m, 10 * seed + i)).cuda() for i, (n, _, m) in enumerate(SIZES)]
+        Y = [torch.from_numpy(gaussian_rhs(n, m, 50 * seed + i)).cuda() for i, (n, _, m) in enumerate(SIZES)]
+        ref = [y.clone() for y in Y]
+        for A, x, y in zip(mats, X, ref):
+            A.matmul(x, y, alpha=0.5, dtype="f64")
+        B.matmul(X, Y, alpha=0.5, dtype="f32")
+        torch.cuda.synchronize()
+        for y, r in zip(Y, ref):
+            # a few FP32 roundings, as for the single products of the other batches' tests
+            assert rel_fro(y.cpu().numpy(), r.cpu().numpy()) <= 3e-6
+    B.close()
