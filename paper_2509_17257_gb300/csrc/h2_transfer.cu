@@ -148,23 +148,42 @@ __global__ void __launch_bounds__(CN == 4 ? 256 : 128) k_leaf_up(const LeafUp p)
     __shared__ __align__(16) float sv[64 * 64];       // V_t, then x̂_t
     __shared__ __align__(16) float sx[64 * 16 * CN];  // X|_t̂
     __shared__ __align__(16) float sh[H == 2 ? 64 * 16 : 4];  // the second half's sums
-    __shared__ int s_perm[64];
     chain_release();
     const int4 rec = p.rec[blockIdx.x];
     const int t = rec.x, off = rec.y, nt = rec.z;
-    if (threadIdx.x < nt) s_perm[threadIdx.x] = p.perm[off + threadIdx.x];
     const int k = FULL ? 64 : p.k, m = FULL ? 16 * CN : p.m;
+    // rows of X by the caller's order, a group of lanes along the columns: thread rows
+    // sub, sub + step, ... (at most 16: 64 points, groups of at most 32 lanes)
+    const int lg = m <= 4 ? 2 : (m <= 8 ? 3 : (m <= 16 ? 4 : 5));
+    const int sub = threadIdx.x >> lg, col = threadIdx.x & ((1 << lg) - 1), step = T >> lg;
+    constexpr int NR = 64 * 32 / T;
+    int row[NR];
+#pragma unroll
+    for (int u = 0; u < NR; ++u) row[u] = sub + u * step < nt ? __ldg(p.perm + off + sub + u * step) : 0;
     const int ldv = (k + 3) & ~3;
     const float* V = p.V + (int64_t)off * k;
     if (ldv == k) {
-#pragma unroll 4
+        // straight into shared memory, in flight beside the rows of X
         for (int e = threadIdx.x; e < nt * k / 4; e += T)
-            reinterpret_cast<float4*>(sv)[e] = __ldg(reinterpret_cast<const float4*>(V) + e);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(sv + 4 * e)), "l"(V + 4 * e) : "memory");
     } else {
 #pragma unroll 4
         for (int e = threadIdx.x; e < nt * k; e += T) sv[(e / k) * ldv + e % k] = __ldg(V + e);
     }
     chain_wait();
+    for (int c = col; c < m; c += 1 << lg) {
+        const bool real = c < p.mreal;
+        const double* X = p.X + c;
+#pragma unroll
+        for (int u0 = 0; u0 < NR; u0 += 8) {
+            double v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = real && sub + (u0 + u) * step < nt ? X[row[u0 + u] * p.ldx] : 0.0;
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (sub + (u0 + u) * step < nt) sx[(sub + (u0 + u) * step) * m + c] = (float)v[u];
+        }
+    }
     {
         const int64_t i0 = blockIdx.x * (int64_t)T + threadIdx.x, n = (int64_t)gridDim.x * T;
         for (int64_t i = i0; i < p.nflag; i += n) p.zflag[i] = 0;
@@ -172,27 +191,16 @@ __global__ void __launch_bounds__(CN == 4 ? 256 : 128) k_leaf_up(const LeafUp p)
         for (int64_t e = i0; e < p.nzid * blk; e += n)
             reinterpret_cast<float4*>(p.yhat)[p.zid[e / blk] * blk + e % blk] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    {
-        // rows of X by the caller's order, a group of lanes along the columns
-        const int lg = m <= 4 ? 2 : (m <= 8 ? 3 : (m <= 16 ? 4 : 5));
-        const double* X = p.X;
-        const int sub = threadIdx.x >> lg, col = threadIdx.x & ((1 << lg) - 1);
-        for (int c = col; c < m; c += 1 << lg) {
-            const bool real = c < p.mreal;
-#pragma unroll 8
-            for (int i = sub; i < nt; i += T >> lg)
-                sx[i * m + c] = real ? (float)X[(int64_t)s_perm[i] * p.ldx + c] : 0.f;
-        }
-    }
-    __syncthreads();
+    // X|_t̂ first: its stores drain under the contraction
+    pack_cols(p.leafX + (int64_t)rec.w * p.R * p.es, (nt + 15) & ~15, p.es, 0, p.R >> 1, sx, m, nt, m);
     const int h = threadIdx.x / (64 * CN), tt = threadIdx.x % (64 * CN);
     const int tx = tt % (4 * CN), ty = tt / (4 * CN);
     float acc[4][4] = {};
     const bool live = 4 * tx < m && 4 * ty < k;
     const int mid = H == 2 ? nt >> 1 : nt, k0 = h ? mid : 0;
     if (live) contract44(acc, sv + k0 * ldv, ldv, sx + k0 * m, m, h ? nt - mid : mid, tx, ty);
-    pack_cols(p.leafX + (int64_t)rec.w * p.R * p.es, (nt + 15) & ~15, p.es, 0, p.R >> 1, sx, m, nt, m);
     if (H == 2 && h && live) {
 #pragma unroll
         for (int r = 0; r < 4; ++r)
@@ -274,8 +282,8 @@ __global__ void __launch_bounds__(32 * W, W == 4 ? 4 : 2) k_pairs(const Pairs p)
     const int grp = threadIdx.x >> logP, col = threadIdx.x & (P - 1), NG = 32 * W >> logP;
     chain_release();
     const PairItem it = p.items[blockIdx.x];
-    chain_wait();
     const int np = it.p1 - it.p0;
+    if (np == 0) chain_wait();
     float* mine = red + grp * K * P + col;
     float* fs = red + K * 32 * W + grp * FL;
     const bool live = LOGP || col < mc;
@@ -292,6 +300,7 @@ __global__ void __launch_bounds__(32 * W, W == 4 ? 4 : 2) k_pairs(const Pairs p)
             const float* f = p.fac + (int64_t)(it.p0 + e) * 3 * Q2;
             for (int i = col; i < 3 * Q2; i += P) fs[i] = __ldg(f + i);
         }
+        if (e0 == 0) chain_wait();  // the first factors do not
         __syncwarp();
         if (e < np) {
             const float* s = p.in + (int64_t)src * K * m + col0 + col;
@@ -311,15 +320,20 @@ __global__ void __launch_bounds__(32 * W, W == 4 ? 4 : 2) k_pairs(const Pairs p)
         }
         __syncwarp();
     }
+    // the own block, in flight while the slower groups finish
+    constexpr int NO = LOGP ? (K * (1 << LOGP) + 128 * W - 1) / (128 * W) : 1;
+    float4 own[NO];
+#pragma unroll
+    for (int u = 0; u < NO; ++u) {
+        const int e = 4 * (threadIdx.x + 32 * W * u);
+        own[u] = LOGP && !UP && e < K * P ? __ldcg(reinterpret_cast<const float4*>(p.out + (int64_t)it.c * K * m + e))
+                                          : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
     __syncthreads();
     // the own block, then the groups that had a pair, in their order; four columns a
     // thread (P is a multiple of 4, and so is m)
     const int used = min(np, NG);
-    for (int e = 4 * threadIdx.x; e < K * P; e += 128 * W) {
-        const int r = e >> logP, c = e & (P - 1);
-        float4* g = reinterpret_cast<float4*>(p.out + ((int64_t)it.c * K + r) * m + col0 + c);
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (!UP && c < mc) v = __ldcg(g);
+    auto reduce4 = [&](int e, float4 v) {
         for (int i = 0; i < used; ++i) {
             const float4 w = *reinterpret_cast<const float4*>(red + i * K * P + e);
             v.x += w.x;
@@ -327,8 +341,22 @@ __global__ void __launch_bounds__(32 * W, W == 4 ? 4 : 2) k_pairs(const Pairs p)
             v.z += w.z;
             v.w += w.w;
         }
-        if ((it.flags & kOutF32) && c < mc) *g = v;
+        const int r = e >> logP, c = e & (P - 1);
+        if ((it.flags & kOutF32) && c < mc)
+            *reinterpret_cast<float4*>(p.out + ((int64_t)it.c * K + r) * m + col0 + c) = v;
         *reinterpret_cast<float4*>(red + e) = v;  // the first group's sums at e have been read, by this thread
+    };
+    if constexpr (LOGP > 0) {
+#pragma unroll
+        for (int u = 0; u < NO; ++u)
+            if (4 * (threadIdx.x + 32 * W * u) < K * P) reduce4(4 * (threadIdx.x + 32 * W * u), own[u]);
+    } else {
+        for (int e = 4 * threadIdx.x; e < K * P; e += 128 * W) {
+            const int c = e & (P - 1);
+            reduce4(e, !UP && c < mc ? __ldcg(reinterpret_cast<const float4*>(p.out + ((int64_t)it.c * K + (e >> logP)) * m +
+                                                                              col0 + c))
+                                     : make_float4(0.f, 0.f, 0.f, 0.f));
+        }
     }
     if (!(it.flags & kOutTile)) return;
     __syncthreads();
