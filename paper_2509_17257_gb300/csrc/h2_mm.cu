@@ -245,6 +245,16 @@ __global__ void k_gather(const double* __restrict__ X, int64_t ldx, const int32_
     }
 }
 
+// (double)x by the bit patterns: a conversion instruction holds the FP64 pipe (two
+// results a cycle and SM) as long as a multiply-add does.  Zeros, subnormals,
+// infinities and NaNs take the instruction.
+__device__ __forceinline__ double widen(float x) {
+    const uint32_t b = __float_as_uint(x);
+    if (((b >> 23) & 255u) - 1u < 254u)
+        return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(b << 29));
+    return (double)x;
+}
+
 // ---- scatter of the tensor-core leaf result: Y[perm[i], :] (+)= α (Z[i, :] + σ X[perm[i], :]) ----
 __global__ void k_scatter_y(const float* __restrict__ Z, int ldz, const int32_t* __restrict__ perm, int64_t n, int m,
                             const double* __restrict__ X, int64_t ldx, double* __restrict__ Y, int64_t ldy,
@@ -260,7 +270,7 @@ __global__ void k_scatter_y(const float* __restrict__ Z, int ldz, const int32_t*
         const double* x = X + g * ldx;
         double* y = Y + g * ldy;
         for (int c = cl; c < m; c += P) {
-            const double v = alpha * ((double)z[c] + sigma * x[c]);
+            const double v = alpha * (widen(z[c]) + sigma * x[c]);
             if (overwrite) y[c] = v; else y[c] += v;
         }
     }
@@ -291,7 +301,7 @@ __global__ void k_scatter_yc(const float* __restrict__ Z, int ldz, const int32_t
         const double* x = X + g * ldx;
         double* y = Y + g * ldy;
         for (int c = cl; c < mc; c += P) {
-            const double zr = (double)z[2 * c] + sigma * x[2 * c], zi = (double)z[2 * c + 1] + sigma * x[2 * c + 1];
+            const double zr = widen(z[2 * c]) + sigma * x[2 * c], zi = widen(z[2 * c + 1]) + sigma * x[2 * c + 1];
             const double vr = alpha_re * zr - alpha_im * zi, vi = alpha_re * zi + alpha_im * zr;
             if (overwrite) {
                 y[2 * c] = vr;

@@ -140,6 +140,21 @@ __device__ __forceinline__ void contract44(float (&acc)[4][4], const float* a, i
     }
 }
 
+// (float)x, rounded to nearest even, by the bit patterns: a conversion instruction
+// holds the FP64 pipe (two results a cycle and SM) as long as a multiply-add does.
+// What does not round to a normal number takes the instruction.
+__device__ __forceinline__ float narrow(double x) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t e = (hi >> 20) & 2047u;
+    if (e - 897u < 253u) {  // 2^-126 <= |x| < 2^127
+        // sign, exponent and 23 bits of the significand; the rest decides the rounding
+        const uint32_t t = (hi & 0x80000000u) | (((hi & 0x7FFFFFFFu) - 0x38000000u) << 3) | (lo >> 29);
+        const uint32_t rest = lo & 0x1FFFFFFFu;
+        return __uint_as_float(t + (rest + (t & 1u) > 0x10000000u ? 1u : 0u));
+    }
+    return (float)x;
+}
+
 // FULL: k = 64 and m = 16·CN, so that every stride is a constant.
 template <int CN, bool FULL>
 __global__ void __launch_bounds__(CN == 4 ? 256 : 128) k_leaf_up(const LeafUp p) {
@@ -181,7 +196,7 @@ __global__ void __launch_bounds__(CN == 4 ? 256 : 128) k_leaf_up(const LeafUp p)
             for (int u = 0; u < 8; ++u) v[u] = real && sub + (u0 + u) * step < nt ? X[row[u0 + u] * p.ldx] : 0.0;
 #pragma unroll
             for (int u = 0; u < 8; ++u)
-                if (sub + (u0 + u) * step < nt) sx[(sub + (u0 + u) * step) * m + c] = (float)v[u];
+                if (sub + (u0 + u) * step < nt) sx[(sub + (u0 + u) * step) * m + c] = narrow(v[u]);
         }
     }
     {
