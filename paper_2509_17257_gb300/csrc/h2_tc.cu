@@ -27,15 +27,16 @@
 // M = 128, so B_lo rides along in M at no cost.
 //
 // Kernel roles (one persistent CTA per SM, or two with at most 32 columns; 7 warps
-// for KIND 0, 11 for KIND 1):
-//   warp 0          bulk-copy producer (cp.async.bulk + mbarrier complete_tx)
+// for KIND 0, 12 for KIND 1):
+//   warp 0, last    bulk-copy producers (cp.async.bulk + mbarrier complete_tx), one
+//                   for the even stages and one for the odd
 //   warp 1          TMEM owner and MMA issuer (tcgen05.mma kind::f16 or
 //                   kind::tf32, FP32 accumulate): KIND 0 all terms, KIND 1 the
 //                   even terms; the converged warp runs the loop and elect.sync
 //                   issues, which keeps its operands warp-uniform
 //   warps 2..5      epilogue (tcgen05.ld, hi+lo combine, stores)
 //   warps 6..9      KIND 1 only: the splitter, [B; B_lo] into TMEM
-//   last warp       KIND 1: MMA issuer of the odd terms (warp 10); KIND 0: idle
+//   warp 10         KIND 1 only: MMA issuer of the odd terms
 // KIND 1: every term accumulates in its own TMEM buffer (round robin over the
 // accumulators), so the epilogue's FP32 sum of earlier terms overlaps the MMAs
 // of the next ones and keeps FP32 accuracy.  KIND 0 (BF16): all terms of an
@@ -61,8 +62,8 @@ constexpr int kSmemBudget = 225 * 1024;  // dynamic shared memory per CTA (one C
 // each CTA's 1 KiB reserve and about 0.7 KiB of static shared memory come off.
 constexpr int kSmemBudgetNarrow = 228 * 1024 / 2 - 1024 - 768;
 constexpr int kSplitWarps = 4;  // KIND 1: warps 6..9 write [B; B_lo] into TMEM, one lane quadrant each
-// warps: 0 producer, 1 and kIssuer2 MMA issuers (even and odd terms), 2..5
-// epilogue, KIND 1: 6..9 splitter
+// warps: 0 and the last producers (even and odd stages), 1 and KIND 1's issuer2 MMA
+// issuers (even and odd terms), 2..5 epilogue, KIND 1: 6..9 splitter
 template <int KIND>
 __host__ __device__ constexpr int tc_issuer2() { return KIND == 1 ? 6 + kSplitWarps : 6; }
 template <int KIND>
@@ -431,18 +432,19 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
 
     if (warp == 0 || warp == tc_producer2<KIND>()) {
         // ---------------- producers ----------------
-        // Two warps issue the copies, of the terms with an even and with an odd index
-        // among the CTA's: a warp's instructions a term bound the kernel where the copies
-        // do not (one producer with six shuffles a term: 1070 cycles a term at KIND 0,
-        // 2100 at KIND 1, unchanged when the copies were halved).  A batch of term
-        // descriptors (16 bytes each) is loaded while the batch before is issued, and
-        // parked in shared memory: a term costs one read of its descriptor, a wait for its
-        // stage, one store of the stage's metadata (published to the other roles by the
-        // mbarrier arrive) and the copies, all from a converged warp, which keeps the
-        // stage's addresses uniform.  A producer is never more than a stage's use ahead of
-        // the other, so a phase parity names one use.
+        // Two warps issue the copies, each into its own stages (even and odd): a warp's
+        // instructions a term bound the kernel where the copies do not (one producer with
+        // six shuffles a term: 1070 cycles a term at KIND 0, 2100 at KIND 1, unchanged when
+        // the copies were halved).  A batch of term descriptors (16 bytes each) is loaded
+        // while the batch before is issued, and parked in shared memory: a term costs one
+        // read of its descriptor, a wait for its stage, one store of the stage's metadata
+        // (published to the other roles by the mbarrier arrive) and the copies, all from a
+        // converged warp, which keeps the stage's addresses uniform.  Stages, not terms,
+        // are shared out: a stage's producer then waits for every one of its uses in turn,
+        // and a phase parity cannot be taken for that of the use two before (the two
+        // issuers may finish terms out of order).
         const int me = warp == 0 ? 0 : 1;
-        int stage = me;
+        int stage = 0;  // of the next term, whichever warp's
         uint32_t phase = 0;
         bool dead = false;
         const uint64_t pol_keep = l2_policy_evict_last(), pol_stream = l2_policy_evict_first();
@@ -451,27 +453,25 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
 #define PSYS(it_, f_) ((FLOW && p.sys) ? p.sys[item_sys(it_)].f_ : p.f_)
         const TcItem none{-1, 0, 0, 0};
         auto item_at = [&](int w) { return w < p.n_items ? p.items[w] : none; };
-        // the lane's term of the item's terms first, first + 2, ... from the base-th of them
-        auto term_at = [&](const TcItem& it, int first, int base) {
-            const int e = it.e0 + first + 2 * (base + lane);
+        // the lane's of the item's terms from base on
+        auto term_at = [&](const TcItem& it, int base) {
+            const int e = it.e0 + base + lane;
             return it.id >= 0 && lane < kTermBatch && e < it.e1 ? __ldg((const int4*)(PSYS(it, terms) + e))
                                                                 : make_int4(0, 0, 0, 0);
         };
         TcItem cur = item_at(blockIdx.x), nxt = item_at(blockIdx.x + G);
-        int first = me;  // this producer's first term of the item
-        int4 tnext = term_at(cur, first, 0);
+        int4 tnext = term_at(cur, 0);
         for (int w = blockIdx.x; w < p.n_items && !dead; w += G) {
             if (__any_sync(0xffffffffu, abort_flag != 0)) break;
             const TcItem after = item_at(w + 2 * G);
-            const int nterms = cur.e1 - cur.e0, own = (nterms - first + 1) >> 1;
-            const int first_n = (first ^ nterms) & 1;
+            const int nterms = cur.e1 - cur.e0;
             const int Ri = PSYS(cur, R), npi = item_np(cur), row_bytes = Ri * ES;
             const uint8_t *a0 = PSYS(cur, act0), *a1 = PSYS(cur, act1), *a2 = PSYS(cur, act2), *bm = PSYS(cur, bmat);
-            if (own <= 0) tnext = term_at(nxt, first_n, 0);
-            for (int base = 0; base < own && !dead; base += kTermBatch) {
+            if (nterms <= 0) tnext = term_at(nxt, 0);
+            for (int base = 0; base < nterms && !dead; base += kTermBatch) {
                 const int4 t = tnext;
-                tnext = base + kTermBatch < own ? term_at(cur, first, base + kTermBatch) : term_at(nxt, first_n, 0);
-                const int cnt = min(kTermBatch, own - base);
+                tnext = base + kTermBatch < nterms ? term_at(cur, base + kTermBatch) : term_at(nxt, 0);
+                const int cnt = min(kTermBatch, nterms - base);
                 __syncwarp();
                 if (lane < kTermBatch) s_term[me][lane] = t;
                 // Terms that read a tile of this launch wait for its ready flag.  The
@@ -480,12 +480,19 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
                 uint32_t ready_mask = 0xffffffffu;
                 const int* my_flag = nullptr;
                 if (LIST) {
-                    if (lane < cnt && ((t.w >> 16) & kTermWait)) my_flag = PSYS(cur, flag) + t.z / PSYS(cur, KP);
+                    int sl = stage + lane;  // the lane's term's stage
+                    while (sl >= nst) sl -= nst;
+                    if (lane < cnt && (sl & 1) == me && ((t.w >> 16) & kTermWait)) my_flag = PSYS(cur, flag) + t.z / PSYS(cur, KP);
                     ready_mask = __ballot_sync(0xffffffffu, !my_flag || flag_acquire(my_flag) == p.epoch);
                 }
                 __syncwarp();
                 int4 tj = s_term[me][0];
                 for (int j = 0; j < cnt; ++j) {
+                    if ((stage & 1) != me) {
+                        if (j + 1 < cnt) tj = s_term[me][j + 1];
+                        if (++stage == nst) { stage = 0; phase ^= 1; }
+                        continue;
+                    }
                     const int kpj = (int16_t)tj.w, asj = tj.w >> 16, akj = tj.z;
                     const int64_t bj = (int64_t)(((uint64_t)(uint32_t)tj.y << 32) | (uint32_t)tj.x);
                     if (j + 1 < cnt) tj = s_term[me][j + 1];
@@ -513,7 +520,7 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
                     }
                     const uint32_t ab = (uint32_t)(row_bytes * kpj);
                     const uint32_t sA = smem_u32(smem + stage * stage_bytes), bar = smem_u32(&full_bar[stage]);
-                    const int term = first + 2 * (base + j);
+                    const int term = base + j;
                     const int fl = (term == 0 ? F_FIRST : 0) | (term == nterms - 1 ? F_LAST : 0) | (phase ? F_PARITY : 0);
                     const int64_t aj = (int64_t)akj * row_bytes;
                     // the activation tiles are read by many terms, the matrix tiles once; MODE 2
@@ -523,17 +530,15 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
                     const uint32_t bb = MF ? (uint32_t)(p.KP * 16) : (uint32_t)(npi * kpj * ES);
                     stage_copy_elect(smem_u32(&stage_meta[stage]), kpj, fl | (npi << 8), Ri, cur.id, bar, sA, asrc, ab,
                                      pol_keep, sA + a_bytes, bsrc, bb, MF ? pol_keep : pol_stream);
-                    stage += 2;
-                    if (stage >= nst) { stage -= nst; phase ^= 1; }
+                    if (++stage == nst) { stage = 0; phase ^= 1; }
                 }
             }
             cur = nxt;
             nxt = after;
-            first = first_n;
         }
         __syncwarp();
-        // the splitters' end marker, a stage without data, comes from the next term's producer
-        if (lane == 0 && !dead && (s_total & 1) == me) {
+        // the splitters' end marker, a stage without data, comes from the next stage's producer
+        if (lane == 0 && !dead && (stage & 1) == me) {
             if (mbar_wait(&empty_bar[stage], phase ^ 1)) {
                 stage_meta[stage] = make_int4(0, F_END | (phase ? F_PARITY : 0), 0, 0);
                 mbar_arrive(&full_bar[stage]);
