@@ -325,12 +325,14 @@ int h2_batch_matmul(h2_batch* b, double alpha, const double* const* X, const int
         return 0;
     }
     H2_CUDA_TRY(cudaStreamWaitEvent(b->origin, b->ev_in, 0));
+    // the graph holds the workspaces' addresses: a product outside the batch may have grown them
+    for (int i : sys) {
+        int rc = product_prepare(b->mats[i], m[i], dtype, b->origin);
+        if (rc) return rc;
+        key.insert(key.end(), {(int64_t)(uintptr_t)b->mats[i]->ws.base, (int64_t)(uintptr_t)b->mats[i]->sync_cnt});
+    }
     if (!b->mm_exec || key != b->mm_key) {
         if (b->mm_exec) { cudaGraphExecDestroy(b->mm_exec); b->mm_exec = nullptr; }
-        for (int i : sys) {
-            int rc = product_prepare(b->mats[i], m[i], dtype, b->origin);
-            if (rc) return rc;
-        }
         H2_CUDA_TRY(cudaStreamSynchronize(b->origin));
         MmCtx ctx{b, alpha, X, ldx, Y, ldy, m, dtype};
         int rc = batch_capture(b, b->origin, sys, mm_body, &ctx, &b->mm_exec);
