@@ -273,6 +273,51 @@ void balance_order(std::vector<TcItem>& v, Cost cost, int G) {
     v.swap(out);
 }
 
+// Cuts the long items of a short list in two, so that their terms run on two CTAs:
+// each half adds its result to the cleared output, and a sum of two does not depend on
+// their order.  (The additions take place in memory, where FP32 subnormals count as
+// zero.)  Items of at least 4 terms and more than half of a CTA's share of the work, in
+// lists of at most max_items: where CTAs are left over, a launch takes as long as its
+// longest item; where they are not, the cuts only add results to store.  µs whole →
+// halves, q = 4: n = 2048, m = 1: 68 → 57 and q = 3: 55 → 46; n = 4096, m = 32: 82 → 70;
+// n = 6000: 86 → 73; n = 8192, m = 64: leaf list (195 items) 120 → 109, the coupling
+// list (375) as well 117; n = 12000, m = 64: leaf list (260) 123 → 128, both 139.
+// H2_TC_HALVES=0 at creation: no cuts.
+constexpr size_t kHalvesCoupling = kTcDeal, kHalvesLeaf = 2 * kTcDeal / 3;
+template <class Cost>
+int split_items(h2_matrix* A, const std::vector<TcItem>& items, size_t max_items, Cost cost,
+                const std::vector<int32_t>& zero, TcHalves* H, cudaStream_t st) {
+    const char* e = getenv("H2_TC_HALVES");
+    if (items.size() > max_items || (e && e[0] == '0')) return 0;
+    int64_t total = 0;
+    for (const TcItem& it : items) total += cost(it);
+    std::vector<TcItem> out;
+    std::vector<int32_t> z = zero;
+    for (TcItem it : items) {
+        const int32_t mid = it.e0 + (it.e1 - it.e0) / 2, e1 = it.e1;
+        if (it.e1 - it.e0 < 4 || 2 * kTcDeal * cost(it) <= total) {
+            out.push_back(it);
+            continue;
+        }
+        z.push_back(it.id);
+        it.np |= kItemHalf;
+        it.e1 = mid;
+        out.push_back(it);
+        it.e0 = mid;
+        it.e1 = e1;
+        out.push_back(it);
+    }
+    if (out.size() == items.size()) return 0;
+    balance_order(out, [&](const TcItem& a) { return cost(a) / ((a.np & kItemHalf) ? 2 : 1); }, kTcDeal);
+    int rc = upload(A, &H->items, out, st);
+    if (!rc) rc = upload(A, &H->zero, z, st);
+    if (!rc) H2_CUDA_TRY(cudaStreamSynchronize(st));  // out and z go out of scope
+    H->n = (int)out.size();
+    H->nzero = (int)z.size();
+    H->any = !rc;
+    return rc;
+}
+
 int cast_copy(h2_matrix* A, const double* src, void** dst, int64_t count, cudaStream_t st) {
     int rc = device_alloc(A, dst, (size_t)(count > 0 ? count : 1) * sizeof(float));
     if (rc) return rc;
@@ -1200,7 +1245,11 @@ int build_tc(h2_matrix* A, bool bf16, bool tf32, cudaStream_t st) {
         else c_zero.push_back((int32_t)c);
     }
     // longest lists first, each to the CTA with the least work so far
-    balance_order(c_items, [](const TcItem& a) { return (int64_t)(a.e1 - a.e0); }, kTcDeal);
+    std::vector<int64_t> c_cost(nc, 0);
+    for (const TcItem& it : c_items) c_cost[it.id] = it.e1 - it.e0;
+    auto cost_c = [&](const TcItem& a) { return c_cost[a.id]; };
+    balance_order(c_items, cost_c, kTcDeal);
+    if ((rc = split_items(A, c_items, kHalvesCoupling, cost_c, c_zero, &D.c_half, st))) return rc;
     // ---- leaf schedule: outputs = leaf positions; terms = V_t ŷ_t, then G_b X|_ŝ ----
     std::vector<int64_t> xkoff(NL + 1, 0);
     std::vector<int32_t> leaf_base(NL), leaf_kdim(NL);
@@ -1233,7 +1282,9 @@ int build_tc(h2_matrix* A, bool bf16, bool tf32, cudaStream_t st) {
             l_items[lp] = TcItem{(int32_t)lp, e0, (int32_t)l_terms.size(), l_np[lp]};
         }
     }
-    balance_order(l_items, [&](const TcItem& a) { return l_cost[a.id]; }, kTcDeal);
+    auto cost_l = [&](const TcItem& a) { return l_cost[a.id]; };
+    balance_order(l_items, cost_l, kTcDeal);
+    if ((rc = split_items(A, l_items, kHalvesLeaf, cost_l, {}, &D.l_half, st))) return rc;
     D.s_off_host = s_off;
     D.et_off_host.clear();
     if (flow) {
@@ -1345,7 +1396,11 @@ int build_tc_transposed(h2_matrix* A, cudaStream_t st) {
             else c_zero.push_back((int32_t)sc);
         }
     }
-    balance_order(c_items, [](const TcItem& a) { return (int64_t)(a.e1 - a.e0); }, kTcDeal);
+    std::vector<int64_t> c_cost(nc, 0);
+    for (const TcItem& it : c_items) c_cost[it.id] = it.e1 - it.e0;
+    auto cost_c = [&](const TcItem& a) { return c_cost[a.id]; };
+    balance_order(c_items, cost_c, kTcDeal);
+    if ((rc = split_items(A, c_items, kHalvesCoupling, cost_c, c_zero, &D.ct_half, st))) return rc;
     // ---- leaf list over column leaves: item s, terms V_s ŷ_s, then G_bᵀ x|_t̂ ----
     std::vector<int64_t> xkoff(NL + 1, 0);
     for (int64_t lp = 0; lp < NL; ++lp) xkoff[lp + 1] = xkoff[lp] + round16((int)T.size[A->leaves[lp]]);
@@ -1368,7 +1423,9 @@ int build_tc_transposed(h2_matrix* A, cudaStream_t st) {
         }
         l_items[lp] = TcItem{(int32_t)lp, e0, (int32_t)l_terms.size(), np};
     }
-    balance_order(l_items, [&](const TcItem& a) { return l_cost[a.id]; }, kTcDeal);
+    auto cost_l = [&](const TcItem& a) { return l_cost[a.id]; };
+    balance_order(l_items, cost_l, kTcDeal);
+    if ((rc = split_items(A, l_items, kHalvesLeaf, cost_l, {}, &D.lt_half, st))) return rc;
     D.ct_nitems = (int)c_items.size();
     D.ct_nzero = (int)c_zero.size();
     D.lt_nitems = (int)NL;

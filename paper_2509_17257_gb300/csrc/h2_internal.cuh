@@ -101,6 +101,8 @@ struct TcItem {
     int32_t id, e0, e1, np;
 };
 constexpr int32_t kRoleTransfer = 1, kRoleCoupling = 2, kRoleLeaf = 3;
+// Modes 0 to 2: the item is one of two halves of a list, added to its cleared output.
+constexpr int32_t kItemHalf = 1 << 16;
 __host__ __device__ inline int32_t item_np(const TcItem& t) { return t.np & 0xFFFF; }
 __host__ __device__ inline int32_t item_role(const TcItem& t) { return (t.np >> 16) & 3; }
 // One term: an activation tile (act0, act1 or act2 by asrc & 3, at akoff·R·es
@@ -177,6 +179,16 @@ struct TcGemmParams {
     int cplx;
 };
 
+// A coupling or leaf list with its long items in two halves (split_items); zero: the
+// clusters without couplings and those whose item is split (coupling).
+struct TcHalves {
+    bool any = false;
+    TcItem* items = nullptr;
+    int n = 0;
+    int32_t* zero = nullptr;
+    int nzero = 0;
+};
+
 // BF16 tensor-core copy of the matrix data and the schedules of its kernels.
 struct TcData {
     bool built = false;
@@ -196,6 +208,7 @@ struct TcData {
     TcItem* l_items = nullptr;
     TcTerm* l_terms = nullptr;
     int l_nitems = 0;
+    TcHalves c_half, l_half;
     int64_t* xkoff = nullptr;   // [n_leaves+1] prefix sums of round16(|leaf|)
     int64_t xk_total = 0;
     int32_t* leaf_base = nullptr;  // first point position of each leaf
@@ -217,6 +230,7 @@ struct TcData {
     TcItem* lt_items = nullptr;
     TcTerm* lt_terms = nullptr;
     int lt_nitems = 0;
+    TcHalves ct_half, lt_half;
     // the transfer passes on the tensor cores (built with the TF32 copy, k <= 64):
     // Eᵀ_s, V_tᵀ, E_s and an identity tile appended to mat32, and work lists in
     // dependency order: the upward and the downward pass alone (used with Aᵀ),
@@ -633,7 +647,7 @@ int launch_pairs(h2_matrix* A, const PairPass& ps, int s0, int s1, bool up, cons
                  int m, int R, int es, bool overlap, cudaStream_t st);
 int launch_forward(h2_matrix* A, const double* X, int64_t ldx, int mreal, int m, float* xhat, uint8_t* xcm,
                    uint8_t* Xcm, int R, int es, bool below, int* zflag, int nflag, const int32_t* zid, int nzid,
-                   float* yhat, bool overlap, cudaStream_t st);
+                   float* yhat, float* z, bool overlap, cudaStream_t st);
 int launch_backward(h2_matrix* A, float* yhat, uint8_t* ycm, int m, int R, int es, bool overlap, cudaStream_t st);
 // Tiles and work lists of the tensor-core product with Aᵀ (once per matrix; allocates).
 int build_tc_transposed(h2_matrix* A, cudaStream_t st);

@@ -829,7 +829,14 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
                     // coalesced pass, so the epilogue only stores
                     if (n < cur_nt) out = SYSF(cur, zp) + ((int64_t)cur_off + n) * ldci;
                 }
-                if (out) {
+                if (!LIST && (cur.np & kItemHalf)) {
+                    // one of two halves, onto zero
+                    if (out) {
+#pragma unroll
+                        for (int i = 0; i < kSums; ++i)
+                            if (i < mci) atomicAdd(out + i, sum[i]);
+                    }
+                } else if (out) {
                     if (vec4) {
 #pragma unroll
                         for (int i = 0; i < kSums; i += 4)
@@ -958,6 +965,13 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
                 if (lane == 0) atomicExch(p.err, 6);
                 abort_flag = 1;
                 break;
+            } else if (writer && !LIST && (cur.np & kItemHalf)) {
+                // one of two halves, onto zero
+                float* out = MODE == 1 ? p.zp + (int64_t)cur_off * p.ldc + i : p.yhat + (int64_t)id * p.k * p.ldc + i;
+                const int rows = MODE == 1 ? cur_nt : min(np, p.k);
+#pragma unroll
+                for (int j = 0; j < kAccCols; ++j)
+                    if (j < rows) atomicAdd(out + (int64_t)j * p.ldc, sum[j]);
             } else if (writer) {
                 if (MODE != 1) {
                     float* out = p.yhat + (int64_t)id * p.k * p.ldc;

@@ -105,7 +105,8 @@ __device__ __forceinline__ void pack_cols(uint8_t* tile, int kp, int es, int i0,
 // them).  It gathers the leaf's rows of X itself, writes X|_t̂ and x̂_t as the split
 // tiles the tensor-core phases read, and x̂_t in FP32 for the pairs.  On the way the
 // launch clears what later ones start from: the ready flags of the hybrid coupling
-// launch, and ŷ of the clusters without couplings.
+// launch, ŷ of the clusters without couplings or with a split list, and the leaf
+// results if some are split.
 struct LeafUp {
     const int4* rec;  // per leaf: cluster, first position, points, first column of its X tile
     const int32_t* perm;
@@ -121,6 +122,7 @@ struct LeafUp {
     const int32_t* zid;
     int nzid;
     float* yhat;
+    float* z;  // the leaf results to clear, or null
 };
 
 // acc[r][c] += Σ_kk a[kk·lda + 4ty + r]·b[kk·ldb + 4tx + c]; rows and columns past
@@ -205,6 +207,9 @@ __global__ void __launch_bounds__(CN == 4 ? 256 : 128) k_leaf_up(const LeafUp p)
         const int64_t blk = (int64_t)k * m / 4;
         for (int64_t e = i0; e < p.nzid * blk; e += n)
             reinterpret_cast<float4*>(p.yhat)[p.zid[e / blk] * blk + e % blk] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (p.z)
+            for (int e = threadIdx.x; e < nt * m / 4; e += T)
+                reinterpret_cast<float4*>(p.z + (int64_t)off * m)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
@@ -586,7 +591,7 @@ int build_pairs(h2_matrix* A, cudaStream_t st) {
 // multiple of 4), with `below` only of the clusters at or below the cut.
 int launch_forward(h2_matrix* A, const double* X, int64_t ldx, int mreal, int m, float* xhat, uint8_t* xcm,
                    uint8_t* Xcm, int R, int es, bool below, int* zflag, int nflag, const int32_t* zid, int nzid,
-                   float* yhat, bool overlap, cudaStream_t st) {
+                   float* yhat, float* z, bool overlap, cudaStream_t st) {
     int rc = pairs_prepare();
     if (rc) return rc;
     const int NL = (int)A->leaves.size();
@@ -610,6 +615,7 @@ int launch_forward(h2_matrix* A, const double* X, int64_t ldx, int mreal, int m,
     p.zid = zid;
     p.nzid = nzid;
     p.yhat = yhat;
+    p.z = z;
     const bool full = A->k == 64;
     auto leaves = [&](void (*kernel)(const LeafUp), int threads) {
         return launch_chained(overlap, kernel, NL, threads, 0, st, p);
