@@ -325,11 +325,13 @@ int h2_batch_matmul(h2_batch* b, double alpha, const double* const* X, const int
         return 0;
     }
     H2_CUDA_TRY(cudaStreamWaitEvent(b->origin, b->ev_in, 0));
-    // the graph holds the workspaces' addresses: a product outside the batch may have grown them
+    // the graph holds the addresses of the workspaces and the lists of transfer pairs: a
+    // product outside the batch may have grown the first, the autotuner rebuilt the second
     for (int i : sys) {
         int rc = product_prepare(b->mats[i], m[i], dtype, b->origin);
         if (rc) return rc;
-        key.insert(key.end(), {(int64_t)(uintptr_t)b->mats[i]->ws.base, (int64_t)(uintptr_t)b->mats[i]->sync_cnt});
+        key.insert(key.end(), {(int64_t)(uintptr_t)b->mats[i]->ws.base, (int64_t)(uintptr_t)b->mats[i]->sync_cnt,
+                               b->mats[i]->pairs_gen});
     }
     if (!b->mm_exec || key != b->mm_key) {
         if (b->mm_exec) { cudaGraphExecDestroy(b->mm_exec); b->mm_exec = nullptr; }

@@ -411,6 +411,7 @@ struct h2_matrix {
     h2::PairPass up_pairs, down_pairs;  // transfer passes of the tensor-core products (q = 2..4)
     int4* d_leaf_rec = nullptr;         // [n_leaves] (cluster, first position, points, first X tile column)
     bool pairs_built = false;
+    int64_t pairs_gen = 0;  // counts the builds of the lists of pairs
     int32_t* d_adm_rowptr = nullptr; // [nc+1] by row cluster
     int32_t* d_adm_col = nullptr;    // [n_adm]
     int32_t* d_adm_row = nullptr;    // [n_adm]

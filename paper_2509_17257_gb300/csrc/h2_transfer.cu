@@ -471,6 +471,7 @@ int upload_pass(h2_matrix* A, PairPass& ps, std::vector<PairItem>& items, const 
 // Lists of both passes for the cut targets A->up_target and A->down_target
 // (replacing earlier ones once the stream has finished with them); sets A->up_cut.
 int build_pairs(h2_matrix* A, cudaStream_t st) {
+    ++A->pairs_gen;
     A->up_cut = 0;
     if (A->q < 2 || A->q > 4) return 0;
     const Tree& T = A->T;

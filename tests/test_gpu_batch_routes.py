@@ -37,3 +37,35 @@ def test_batch_routes_equal_single_fp64_products(no_pairs, monkeypatch):
             # a few FP32 roundings, as for the single products of the other batches' tests
             assert rel_fro(y.cpu().numpy(), r.cpu().numpy()) <= 3e-6
     B.close()
+
+
+def test_cached_graph_follows_workspaces_and_lists():
+    """A batch's graph is replayed for the same buffers: not after a wider product outside the batch has grown a
+    workspace, nor after the autotuner has rebuilt a matrix's lists."""
+    torch = require_cuda()
+    import paper_2509_17257_gb300.build as bld
+    bld.build()
+    import paper_2509_17257_gb300 as P
+    n, m = 3001, 5
+    mats = [P.H2Matrix(ellipsoid_points(n, (1.0, 0.7, 0.5), s), q=3, leaf_size=64, eta=2.0, sigma=1e-2,
+                       precisions=("f32",)) for s in (1, 2)]
+    B = P.H2Batch(mats)
+    X = [torch.from_numpy(gaussian_rhs(n, m, 60 + i)).cuda() for i in range(2)]
+    Y = [torch.zeros_like(x) for x in X]
+
+    def check():
+        for y in Y:
+            y.zero_()
+        B.matmul(X, Y, dtype="f32")
+        for A, x, y in zip(mats, X, Y):
+            ref = torch.zeros_like(x)
+            A.matmul(x, ref, dtype="f64")
+            assert rel_fro(y.cpu().numpy(), ref.cpu().numpy()) <= 3e-6
+
+    check()
+    wide = torch.from_numpy(gaussian_rhs(n, 64, 7)).cuda()
+    mats[0].matmul(wide, torch.zeros_like(wide), dtype="f32")
+    check()
+    P.h2_autotune_ex(mats[1].handle, m, "f32")
+    check()
+    B.close()
