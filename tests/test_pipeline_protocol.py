@@ -2,7 +2,8 @@
 checked on the CPU by a model with random interleavings.
 
 The model has the kernel's agents:
-  - the producer: one copy per term into a ring of `nst` stages;
+  - the producers (one, or two that share the stages): one copy per term into a ring
+    of `nst` stages;
   - four splitter warps: [B; B_lo] into one of `kASlots` TMEM A slots, with
     the look-ahead that tests the next term's stage and slot barriers;
   - two MMA issuers, taking the terms by parity;
@@ -59,12 +60,13 @@ class Hazard(AssertionError):
 
 
 def run_pipeline(T, nst=6, nacc=4, nslots=4, seed=0, mutate=None, max_steps=200000, splitter_warps=True,
-                 items=None):
+                 items=None, producers=None):
     """Simulate one CTA on T terms; raises Hazard or returns normally.  Without
     splitter warps (the BF16 kernel) the issuers wait on the copies directly.
     With `items` (term counts of the CTA's items; the BF16 kernel's protocol)
     one issuer accumulates all terms of an item into one accumulator and the
-    epilogue reads each accumulator once per item."""
+    epilogue reads each accumulator once per item.  producers: None for one, "stages" for
+    two that own the even and the odd stages, "terms" for two that take the terms by parity."""
     if items is not None:
         T = sum(items)
         splitter_warps = False
@@ -93,9 +95,17 @@ def run_pipeline(T, nst=6, nacc=4, nslots=4, seed=0, mutate=None, max_steps=2000
         return ("wait", bar, parity)
 
     # ---------------- producer ----------------
-    def producer():
+    def producer(me=0):
         stage, phase = 0, 0
+
+        def owner(t):
+            return 0 if producers is None else ((t % nst) & 1 if producers == "stages" else t & 1)
         for t in range(T):
+            if owner(t) != me:
+                stage += 1
+                if stage == nst:
+                    stage, phase = 0, phase ^ 1
+                continue
             p = phase if mutate == "producer_parity" else phase ^ 1
             yield W(empty[stage], p)
             if stage_readers[stage] or (stage_term[stage] is not None and not consumed.get(stage_term[stage])):
@@ -112,6 +122,8 @@ def run_pipeline(T, nst=6, nacc=4, nslots=4, seed=0, mutate=None, max_steps=2000
             stage += 1
             if stage == nst:
                 stage, phase = 0, phase ^ 1
+        if owner(T) != me:
+            return
         yield W(empty[stage], phase ^ 1)
         stage_term[stage], stage_landed[stage] = END, True
         full[stage].arrive()
@@ -237,10 +249,11 @@ def run_pipeline(T, nst=6, nacc=4, nslots=4, seed=0, mutate=None, max_steps=2000
             acc_unread[acc] -= 1
             acce[acc].arrive()
 
+    feed = [producer()] if producers is None else [producer(0), producer(1)]
     if items is not None:
-        agents = [producer(), issuer_items()] + [epilogue_items(e) for e in range(4)]
+        agents = feed + [issuer_items()] + [epilogue_items(e) for e in range(4)]
     else:
-        agents = ([producer()] + ([splitter(w) for w in range(4)] if splitter_warps else []) + [issuer(0), issuer(1)]
+        agents = (feed + ([splitter(w) for w in range(4)] if splitter_warps else []) + [issuer(0), issuer(1)]
                   + [epilogue(e) for e in range(4)])
     state = [None] * len(agents)   # the pending request of each agent
     done = [False] * len(agents)
@@ -349,3 +362,27 @@ def test_bf16_item_protocol_planted_mistakes_are_caught(mutate):
             break
     assert caught, mutate
 
+
+# Two producers share the ring: by stages, any stage count from two on is safe, with the
+# accumulators and A slots of both instances.
+@pytest.mark.parametrize("nst", [2, 3, 4, 5, 6, 9])
+@pytest.mark.parametrize("nacc,nslots", [(4, 4), (2, 2), (4, 2)])
+def test_two_producers_by_stages(nst, nacc, nslots):
+    for T in (1, 2, 7, 40):
+        for seed in range(8):
+            run_pipeline(T, nst=nst, nacc=nacc, nslots=nslots, seed=seed, producers="stages")
+    for shape in ITEM_SHAPES:
+        run_pipeline(0, nst=nst, nacc=4, seed=nst, items=shape, producers="stages")
+
+
+# By terms, an odd stage count hands every stage to the other producer at every use, and as
+# the issuers may finish terms out of order, a phase two uses old passes for the one awaited.
+def test_two_producers_by_terms_are_unsafe_with_odd_stages():
+    caught = False
+    for seed in range(400):
+        try:
+            run_pipeline(40, nst=3, nacc=2, nslots=2, seed=seed, producers="terms")
+        except Hazard:
+            caught = True
+            break
+    assert caught
