@@ -1,6 +1,6 @@
 // Shared-memory mbarriers and bulk copies (cp.async.bulk, completed through an
-// mbarrier's transaction count), used by the tensor-core kernels and the
-// staged transfer passes.  Every wait is bounded by kSpinLimit polls; the
+// mbarrier's transaction count), used by the tensor-core kernels; programmatic
+// dependent launch.  Every wait is bounded by kSpinLimit polls; the
 // caller turns a timeout into an error flag.
 #pragma once
 

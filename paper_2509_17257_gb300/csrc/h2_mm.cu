@@ -10,9 +10,9 @@
 //                                                  one owner per row cluster, Alg. "list_addeval")
 //   down(l)     ŷ_{t'} += E_{t'} ŷ_t                levels 1 .. deepest
 //   leaf_bwd    Y|_t̂ += α (V_t ŷ_t + Σ_{b=(t,s)∈L-} G_b Xp|_ŝ + σ Xp|_t̂)   scattered through perm
-// Every output tile has exactly one owning CTA, so no atomics are needed: the
-// race the paper resolves by sequential sums (Sec. 3, after Alg.
-// "forward/backward") is resolved here by ownership.
+// Every output tile has exactly one owning CTA (or, in short work lists, two that
+// each add a half to a cleared tile): the race the paper resolves by sequential
+// sums (Sec. 3, after Alg. "forward/backward") is resolved here by ownership.
 #include <cuda_runtime.h>
 
 #include <algorithm>
