@@ -291,8 +291,10 @@ int split_items(h2_matrix* A, const std::vector<TcItem>& items, size_t max_items
     if (items.size() > max_items || (e && e[0] == '0')) return 0;
     int64_t total = 0;
     for (const TcItem& it : items) total += cost(it);
-    std::vector<TcItem> out;
-    std::vector<int32_t> z = zero;
+    std::vector<TcItem>& out = H->host_items;  // kept: the copies below may read them later
+    std::vector<int32_t>& z = H->host_zero;
+    out.clear();
+    z = zero;
     for (TcItem it : items) {
         const int32_t mid = it.e0 + (it.e1 - it.e0) / 2, e1 = it.e1;
         if (it.e1 - it.e0 < 4 || 2 * kTcDeal * cost(it) <= total) {
@@ -311,7 +313,6 @@ int split_items(h2_matrix* A, const std::vector<TcItem>& items, size_t max_items
     balance_order(out, [&](const TcItem& a) { return cost(a) / ((a.np & kItemHalf) ? 2 : 1); }, kTcDeal);
     int rc = upload(A, &H->items, out, st);
     if (!rc) rc = upload(A, &H->zero, z, st);
-    if (!rc) H2_CUDA_TRY(cudaStreamSynchronize(st));  // out and z go out of scope
     H->n = (int)out.size();
     H->nzero = (int)z.size();
     H->any = !rc;

@@ -187,6 +187,8 @@ struct TcHalves {
     int n = 0;
     int32_t* zero = nullptr;
     int nzero = 0;
+    std::vector<TcItem> host_items;
+    std::vector<int32_t> host_zero;
 };
 
 // BF16 tensor-core copy of the matrix data and the schedules of its kernels.

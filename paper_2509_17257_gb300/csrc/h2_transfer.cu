@@ -462,7 +462,6 @@ int upload_pass(h2_matrix* A, PairPass& ps, std::vector<PairItem>& items, const 
         k_pair_factors<<<1216, 256, 0, st>>>(ps.pair, (int64_t)pair.size(), A->d_nodes, A->q, up ? 1 : 0, ps.fac);
         H2_LAUNCH_CHECK();
     }
-    H2_CUDA_TRY(cudaStreamSynchronize(st));  // the host lists go out of scope
     return 0;
 }
 
@@ -482,9 +481,17 @@ int build_pairs(h2_matrix* A, cudaStream_t st) {
     // tree of depth 66 stays below a quarter of this.)
     const size_t most = (size_t)nc * 32 + 4096;
     A->pairs_built = false;
-    H2_CUDA_TRY(cudaStreamSynchronize(st));
+    if (A->up_pairs.items || A->down_pairs.items) H2_CUDA_TRY(cudaStreamSynchronize(st));
     int rc = pairs_prepare();
     if (rc) return rc;
+    std::vector<int4> rec;
+    std::vector<PairItem> up_items, down_items;
+    std::vector<int2> up_list, down_list;
+    // the copies from these vectors have finished before they go out of scope
+    struct Drain {
+        cudaStream_t st;
+        ~Drain() { cudaStreamSynchronize(st); }
+    } drain{st};
     std::vector<int64_t> end(nc);  // pre-order: the subtree of c is [c, end[c])
     for (int64_t c = nc - 1; c >= 0; --c) end[c] = T.is_leaf((int32_t)c) ? c + 1 : end[T.son1[c]];
     auto add_stage = [](PairPass& ps, const std::vector<PairItem>& items, int32_t from) {
@@ -499,7 +506,7 @@ int build_pairs(h2_matrix* A, cudaStream_t st) {
     };
     if (!A->d_leaf_rec) {
         // the leaves by falling size; X tiles as in the leaf phase (columns rounded up to 16)
-        std::vector<int4> rec(NL);
+        rec.resize(NL);
         int32_t x0 = 0;
         for (int64_t lp = 0; lp < NL; ++lp) {
             const int32_t c = A->leaves[lp];
@@ -509,15 +516,14 @@ int build_pairs(h2_matrix* A, cudaStream_t st) {
         std::stable_sort(rec.begin(), rec.end(), [](const int4& a, const int4& b) { return a.z > b.z; });
         if ((rc = device_alloc(A, (void**)&A->d_leaf_rec, NL * sizeof(int4)))) return rc;
         H2_CUDA_TRY(cudaMemcpyAsync(A->d_leaf_rec, rec.data(), NL * sizeof(int4), cudaMemcpyHostToDevice, st));
-        H2_CUDA_TRY(cudaStreamSynchronize(st));
     }
     {
         // upward: inner clusters of the levels [cut, above) from the clusters at level
         // `above` and the leaves before it, cut after cut
         PairPass& ps = A->up_pairs;
         ps.stages.clear();
-        std::vector<PairItem> items;
-        std::vector<int2> pair;
+        std::vector<PairItem>& items = up_items;
+        std::vector<int2>& pair = up_list;
         int above = T.depth + 1, cut = cut_level(T, NL, A->up_target, kUpTasks);
         A->up_cut = cut;
         while (above > 0) {
@@ -553,8 +559,8 @@ int build_pairs(h2_matrix* A, cudaStream_t st) {
         // starts at the cut above (whose ŷ is final by then)
         PairPass& ps = A->down_pairs;
         ps.stages.clear();
-        std::vector<PairItem> items;
-        std::vector<int2> pair;
+        std::vector<PairItem>& items = down_items;
+        std::vector<int2>& pair = down_list;
         const int cut = cut_level(T, NL, A->down_target, kDownTasks);
         std::vector<int> cuts;
         if (cut > 10) cuts.push_back((cut + 1) / 2);
