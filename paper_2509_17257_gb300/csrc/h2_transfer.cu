@@ -19,7 +19,7 @@
 //
 // Against subtree passes (one CTA per subtree, three dependent steps a level), in
 // µs: n = 65536, q = 4, m = 32: gather and upward pass below the cut 68 → 48,
-// downward 57 → 37; m = 16 with the whole climb: 86 → 55 and 44 → 29; n = 262144,
+// downward 57 → 37 (30 now); m = 16 with the whole climb: 86 → 55 and 44 → 29; n = 262144,
 // m = 16: 164 → 104 and 99 → 80; n = 8192, m = 32 with the climb: 55 → 32, 22 → 19.
 // The roundings of a path are now one product's: FP32 error at n = 262144, m = 16
 // 3.1e-6 → 1.2e-6.
@@ -106,7 +106,11 @@ __device__ __forceinline__ void pack_cols(uint8_t* tile, int kp, int es, int i0,
 // tiles the tensor-core phases read, and x̂_t in FP32 for the pairs.  On the way the
 // launch clears what later ones start from: the ready flags of the hybrid coupling
 // launch, ŷ of the clusters without couplings or with a split list, and the leaf
-// results if some are split.
+// results if some are split.  Bound by its loads' latency (record, then indices and V,
+// then rows of X) and by 1535 leaves being 1.1 waves of nine CTAs an SM: V comes into
+// shared memory asynchronously beside the rows of X, whose indices are read before the
+// wait for the launch before.  n = 65536, m = 32 (µs): through registers, one after the
+// other 28.9 → 27.1, conversions to FP32 off the FP64 pipe 25.4.
 struct LeafUp {
     const int4* rec;  // per leaf: cluster, first position, points, first column of its X tile
     const int32_t* perm;
@@ -252,7 +256,9 @@ __global__ void __launch_bounds__(CN == 4 ? 256 : 128) k_leaf_up(const LeafUp p)
 // A group of P lanes takes every (groups)-th pair of the list, and adds its results
 // in a block of shared memory of its own.  A pair's factors come in by the group's
 // lanes together.  LOGP > 0: m = P = 2^LOGP, so that rows are at constant offsets
-// (as many instructions went into addresses as into multiply-adds).
+// (as many instructions went into addresses as into multiply-adds).  The first
+// factors come in ahead of the wait for the launch before, the own block while slower
+// groups finish: n = 65536, m = 32: up 19.8 → 18.2, down 12.3 + 24.7 → 9.8 + 20.5 µs.
 struct Pairs {
     const PairItem* items;
     const int2* pair;  // (descendant, ancestor)
