@@ -49,6 +49,15 @@ int batch_capture(h2_batch* b, cudaStream_t origin, const std::vector<int>& sys,
 
 namespace {
 
+// What a captured product of A holds besides the caller's blocks: the addresses of its
+// workspace and of the transfer passes' bookkeeping, which a product outside the batch
+// may have grown (each in its own allocation; the second's layout goes by its column
+// tiles), and the lists of transfer pairs, which the autotuner may have rebuilt.  Part of
+// the key of every cached graph.
+void key_of_buffers(const h2_matrix* A, std::vector<int64_t>& key) {
+    key.insert(key.end(), {(int64_t)(uintptr_t)A->ws.base, (int64_t)(uintptr_t)A->sync_cnt, A->sync_tiles, A->pairs_gen});
+}
+
 struct MmCtx {
     h2_batch* b;
     double alpha;
@@ -217,8 +226,8 @@ int batch_flow_matmul(h2_batch* b, double alpha, const double* const* X, const i
     key.push_back(abits);
     for (int j = 0; j < ns; ++j) {
         const int i = sys[j];
-        key.insert(key.end(), {i, (int64_t)(uintptr_t)X[i], ldx[i], (int64_t)(uintptr_t)Y[i], ldy[i], m[i],
-                               (int64_t)(uintptr_t)fb[j].Xp});
+        key.insert(key.end(), {i, (int64_t)(uintptr_t)X[i], ldx[i], (int64_t)(uintptr_t)Y[i], ldy[i], m[i]});
+        key_of_buffers(b->mats[i], key);
     }
     if (!b->flow_exec || key != b->flow_key) {
         if (b->flow_exec) { cudaGraphExecDestroy(b->flow_exec); b->flow_exec = nullptr; }
@@ -325,13 +334,10 @@ int h2_batch_matmul(h2_batch* b, double alpha, const double* const* X, const int
         return 0;
     }
     H2_CUDA_TRY(cudaStreamWaitEvent(b->origin, b->ev_in, 0));
-    // the graph holds the addresses of the workspaces and the lists of transfer pairs: a
-    // product outside the batch may have grown the first, the autotuner rebuilt the second
     for (int i : sys) {
         int rc = product_prepare(b->mats[i], m[i], dtype, b->origin);
         if (rc) return rc;
-        key.insert(key.end(), {(int64_t)(uintptr_t)b->mats[i]->ws.base, (int64_t)(uintptr_t)b->mats[i]->sync_cnt,
-                               b->mats[i]->pairs_gen});
+        key_of_buffers(b->mats[i], key);
     }
     if (!b->mm_exec || key != b->mm_key) {
         if (b->mm_exec) { cudaGraphExecDestroy(b->mm_exec); b->mm_exec = nullptr; }

@@ -69,3 +69,33 @@ def test_cached_graph_follows_workspaces_and_lists():
     P.h2_autotune_ex(mats[1].handle, m, "f32")
     check()
     B.close()
+
+
+def test_cached_multi_system_graph_follows_the_bookkeeping(monkeypatch):
+    """The multi-system route's graph holds the addresses of the ready flags too: a product of more than 64 columns
+    outside the batch lays the bookkeeping out anew, while the workspace is large enough already and stays."""
+    torch = require_cuda()
+    import paper_2509_17257_gb300.build as bld
+    bld.build()
+    import paper_2509_17257_gb300 as P
+    monkeypatch.setenv("H2_KRON", "0")
+    n, m = 3001, 64
+    mats = [P.H2Matrix(ellipsoid_points(n, (1.0, 0.7, 0.5), s), q=3, leaf_size=64, eta=2.0, sigma=1e-2,
+                       precisions=("f32",)) for s in (1, 2)]
+    B = P.H2Batch(mats)
+    X = [torch.from_numpy(gaussian_rhs(n, m, 80 + i)).cuda() for i in range(2)]
+    Y = [torch.zeros_like(x) for x in X]
+    ref = [torch.zeros_like(x) for x in X]
+    for A, x, r in zip(mats, X, ref):
+        A.matmul(x, r, dtype="f64")
+    for wide in (0, 65, 200):
+        if wide:
+            w = torch.from_numpy(gaussian_rhs(n, wide, 7)).cuda()
+            mats[0].matmul(w, torch.zeros_like(w), dtype="f32")
+        for y in Y:
+            y.zero_()
+        B.matmul(X, Y, dtype="f32")
+        torch.cuda.synchronize()
+        for y, r in zip(Y, ref):
+            assert rel_fro(y.cpu().numpy(), r.cpu().numpy()) <= 3e-6
+    B.close()
