@@ -52,10 +52,13 @@ namespace {
 // What a captured product of A holds besides the caller's blocks: the addresses of its
 // workspace and of the transfer passes' bookkeeping, which a product outside the batch
 // may have grown (each in its own allocation; the second's layout goes by its column
-// tiles), and the lists of transfer pairs, which the autotuner may have rebuilt.  Part of
-// the key of every cached graph.
-void key_of_buffers(const h2_matrix* A, std::vector<int64_t>& key) {
-    key.insert(key.end(), {(int64_t)(uintptr_t)A->ws.base, (int64_t)(uintptr_t)A->sync_cnt, A->sync_tiles, A->pairs_gen});
+// tiles), the lists of transfer pairs, which the autotuner may have rebuilt, and the
+// shift, which h2_shift_set may have changed.  Part of the key of every cached graph.
+void key_of_matrix(const h2_matrix* A, std::vector<int64_t>& key) {
+    int64_t sbits;
+    memcpy(&sbits, &A->sigma, sizeof(sbits));
+    key.insert(key.end(), {(int64_t)(uintptr_t)A->ws.base, (int64_t)(uintptr_t)A->sync_cnt, A->sync_tiles, A->pairs_gen,
+                           sbits});
 }
 
 struct MmCtx {
@@ -227,7 +230,7 @@ int batch_flow_matmul(h2_batch* b, double alpha, const double* const* X, const i
     for (int j = 0; j < ns; ++j) {
         const int i = sys[j];
         key.insert(key.end(), {i, (int64_t)(uintptr_t)X[i], ldx[i], (int64_t)(uintptr_t)Y[i], ldy[i], m[i]});
-        key_of_buffers(b->mats[i], key);
+        key_of_matrix(b->mats[i], key);
     }
     if (!b->flow_exec || key != b->flow_key) {
         if (b->flow_exec) { cudaGraphExecDestroy(b->flow_exec); b->flow_exec = nullptr; }
@@ -337,7 +340,7 @@ int h2_batch_matmul(h2_batch* b, double alpha, const double* const* X, const int
     for (int i : sys) {
         int rc = product_prepare(b->mats[i], m[i], dtype, b->origin);
         if (rc) return rc;
-        key_of_buffers(b->mats[i], key);
+        key_of_matrix(b->mats[i], key);
     }
     if (!b->mm_exec || key != b->mm_key) {
         if (b->mm_exec) { cudaGraphExecDestroy(b->mm_exec); b->mm_exec = nullptr; }

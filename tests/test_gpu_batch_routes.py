@@ -99,3 +99,30 @@ def test_cached_multi_system_graph_follows_the_bookkeeping(monkeypatch):
         for y, r in zip(Y, ref):
             assert rel_fro(y.cpu().numpy(), r.cpu().numpy()) <= 3e-6
     B.close()
+
+
+@pytest.mark.parametrize("kron,dtype", [("1", "f32"), ("0", "f32"), ("1", "f64")], ids=["branches", "multi", "f64"])
+def test_cached_graph_follows_the_shift(kron, dtype, monkeypatch):
+    """A changed shift counts at the next batched product, also for the same blocks."""
+    torch = require_cuda()
+    import paper_2509_17257_gb300.build as bld
+    bld.build()
+    import paper_2509_17257_gb300 as P
+    monkeypatch.setenv("H2_KRON", kron)
+    n, m = 1200, 6
+    mats = [P.H2Matrix(ellipsoid_points(n, (1.0, 0.7, 0.5), s), q=3, leaf_size=64, eta=2.0, sigma=1e-2,
+                       precisions=("f32",)) for s in (1, 2)]
+    B = P.H2Batch(mats)
+    X = [torch.from_numpy(gaussian_rhs(n, m, 90 + i)).cuda() for i in range(2)]
+    Y = [torch.zeros_like(x) for x in X]
+    for sigma in (1e-2, 1e3):
+        P.h2_shift_set(mats[1].handle, sigma)
+        for y in Y:
+            y.zero_()
+        B.matmul(X, Y, dtype=dtype)
+        for A, x, y in zip(mats, X, Y):
+            ref = torch.zeros_like(x)
+            A.matmul(x, ref, dtype="f64")
+            torch.cuda.synchronize()
+            assert rel_fro(y.cpu().numpy(), ref.cpu().numpy()) <= 3e-6
+    B.close()
