@@ -1207,6 +1207,14 @@ int refuse_complex(const h2_matrix* A, const char* what) {
     return 0;
 }
 
+// Whether a product of m columns runs on the tensor cores (run_chain_tc, which sizes its
+// workspace by chunks of 64 columns) or on the CUDA cores (run_chain: all columns at once).
+bool on_tensor_cores(const h2_matrix* A, int64_t m, int32_t dtype) {
+    if (dtype == H2_BF16 || dtype == H2_F32_MF) return true;
+    return dtype == H2_F32 && A->tc.has_tf32 && !A->force_simt &&
+           A->tune[0][column_class((int)std::min<int64_t>(m, 64))].path != kPathSimt;
+}
+
 int matmul_device(h2_matrix* A, double alpha, const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m,
                   int32_t dtype, cudaStream_t st, bool transposed, bool overwrite, const double* alpha_im) {
     if (!alpha_im) {
@@ -1225,7 +1233,8 @@ int matmul_device(h2_matrix* A, double alpha, const double* X, int64_t ldx, doub
     const size_t bC = align_up((size_t)A->nc * A->k * m * elt);
     int rc = check_device_error(A);
     if (rc) return rc;
-    rc = dtype == H2_BF16 ? 0 : ensure_workspace(A, bXp + 2 * bC, st);
+    const bool tc = on_tensor_cores(A, m, dtype);
+    rc = tc ? 0 : ensure_workspace(A, bXp + 2 * bC, st);
     if (rc) return rc;
     SyncBufs sb;
     if ((rc = ensure_sync(A, sync_tiles_for(m), st, &sb))) return rc;
@@ -1239,14 +1248,12 @@ int matmul_device(h2_matrix* A, double alpha, const double* X, int64_t ldx, doub
         if (!A->f32.built) { set_error("FP32 copy not built (add 1<<H2_F32 to params->precisions)"); return H2_E_UNSUPPORTED; }
         if (alpha_im) {
             // the complex product: split-TF32 tensor cores where their tiles were built
-            if (A->tc.has_tf32 && !A->force_simt)
+            if (tc)
                 return dispatch_tc(A, 1, alpha, X, ldx, Y, ldy, m, st, overwrite, sb, false, alpha_im);
             return dispatch_cn<float>(A, A->f32, alpha, X, ldx, Y, ldy, (int)m, st, false, overwrite, (float*)base,
                                       (float*)(base + bXp), (float*)(base + bXp + bC), sb, alpha_im);
         }
-        const Tune& tn = A->tune[0][column_class((int)std::min<int64_t>(m, 64))];
-        if (A->tc.has_tf32 && !A->force_simt && tn.path != kPathSimt)
-            return dispatch_tc(A, 1, alpha, X, ldx, Y, ldy, m, st, overwrite, sb, transposed);
+        if (tc) return dispatch_tc(A, 1, alpha, X, ldx, Y, ldy, m, st, overwrite, sb, transposed);
         return dispatch_cn<float>(A, A->f32, alpha, X, ldx, Y, ldy, (int)m, st, transposed, overwrite,
                                   (float*)base, (float*)(base + bXp), (float*)(base + bXp + bC), sb);
     }
@@ -1276,9 +1283,7 @@ int product_prepare(h2_matrix* A, int64_t m, int32_t dtype, cudaStream_t st) {
     const int64_t n = A->n, nc = A->nc;
     const int k = A->k;
     size_t need = 0;
-    const bool tc = (dtype == H2_BF16) || ((dtype == H2_F32 || dtype == H2_F32_MF) && A->tc.has_tf32 && !A->force_simt &&
-                                           A->tune[0][column_class((int)std::min<int64_t>(m, 64))].path != kPathSimt);
-    if (tc) {
+    if (on_tensor_cores(A, m, dtype)) {
         const TcData& D = A->tc;
         const int es = dtype == H2_BF16 ? 2 : 4;
         const int mc = (int)std::min<int64_t>(64, m);

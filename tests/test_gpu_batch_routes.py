@@ -101,6 +101,28 @@ def test_cached_multi_system_graph_follows_the_bookkeeping(monkeypatch):
     B.close()
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "f64"])
+def test_first_batched_product_of_many_columns(dtype):
+    """Everything a captured product needs is allocated before the capture, at several chunks of 64 columns too."""
+    torch = require_cuda()
+    import paper_2509_17257_gb300.build as bld
+    bld.build()
+    import paper_2509_17257_gb300 as P
+    n, m = 900, 300
+    mats = [P.H2Matrix(ellipsoid_points(n, (1.0, 0.7, 0.5), s), q=4, leaf_size=64, eta=2.0, sigma=1e-2,
+                       precisions=("f32", "bf16")) for s in (1, 2)]
+    B = P.H2Batch(mats)
+    X = [torch.from_numpy(gaussian_rhs(n, m, 95 + i)).cuda() for i in range(2)]
+    Y = [torch.zeros_like(x) for x in X]
+    B.matmul(X, Y, dtype=dtype)
+    for A, x, y in zip(mats, X, Y):
+        ref = torch.zeros_like(x)
+        A.matmul(x, ref, dtype="f64")
+        torch.cuda.synchronize()
+        assert rel_fro(y.cpu().numpy(), ref.cpu().numpy()) <= {"f32": 3e-6, "bf16": 3e-3, "f64": 1e-13}[dtype]
+    B.close()
+
+
 @pytest.mark.parametrize("kron,dtype", [("1", "f32"), ("0", "f32"), ("1", "f64")], ids=["branches", "multi", "f64"])
 def test_cached_graph_follows_the_shift(kron, dtype, monkeypatch):
     """A changed shift counts at the next batched product, also for the same blocks."""
