@@ -84,7 +84,10 @@ __device__ __forceinline__ void bulk_g2s_hint(void* dst, const void* src, uint32
 // calls chain_release(), after which the successor's CTAs may be scheduled (they take
 // what this grid leaves free), and chain_wait(), after which everything that earlier
 // kernels wrote is visible; only work on data that no kernel writes stands before it.
-// Every kernel waits, so completion passes down the chain.
+// Every kernel waits, so completion passes down the chain.  Such a kernel is alive while
+// its predecessors write, so what they write (and the caller's blocks, which may be the
+// output of the product before) is not read-only to it: __ldg and __restrict__, which
+// promise that and let loads pass the wait, are for matrix data and index lists alone.
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -231,8 +231,7 @@ __device__ __forceinline__ int row_lanes(int m) {
 
 // ---- gather: Xp[i, :] = X[perm[i], :] in the compute type ----
 template <typename T>
-__global__ void k_gather(const double* __restrict__ X, int64_t ldx, const int32_t* __restrict__ perm, int64_t n,
-                         int m, T* __restrict__ Xp) {
+__global__ void k_gather(const double* X, int64_t ldx, const int32_t* __restrict__ perm, int64_t n, int m, T* Xp) {
     chain_release();
     chain_wait();
     const int P = row_lanes(m), R = 32 / P;
@@ -256,9 +255,9 @@ __device__ __forceinline__ double widen(float x) {
 }
 
 // ---- scatter of the tensor-core leaf result: Y[perm[i], :] (+)= α (Z[i, :] + σ X[perm[i], :]) ----
-__global__ void k_scatter_y(const float* __restrict__ Z, int ldz, const int32_t* __restrict__ perm, int64_t n, int m,
-                            const double* __restrict__ X, int64_t ldx, double* __restrict__ Y, int64_t ldy,
-                            double alpha, double sigma, int overwrite) {
+__global__ void k_scatter_y(const float* Z, int ldz, const int32_t* __restrict__ perm, int64_t n, int m,
+                            const double* X, int64_t ldx, double* Y, int64_t ldy, double alpha, double sigma,
+                            int overwrite) {
     chain_release();
     chain_wait();
     const int P = row_lanes(m), R = 32 / P;
@@ -286,9 +285,9 @@ int launch_scatter_y(const float* Z, int ldz, const int32_t* perm, int64_t n, in
 
 // ---- the same over C: interleaved (real, imaginary) columns, m2 = 2·m_c, and
 // Y[perm[i], :] (+)= α (Z[i, :] + σ X[perm[i], :]) with α = alpha_re + i·alpha_im ----
-__global__ void k_scatter_yc(const float* __restrict__ Z, int ldz, const int32_t* __restrict__ perm, int64_t n,
-                             int m2, const double* __restrict__ X, int64_t ldx, double* __restrict__ Y, int64_t ldy,
-                             double alpha_re, double alpha_im, double sigma, int overwrite) {
+__global__ void k_scatter_yc(const float* Z, int ldz, const int32_t* __restrict__ perm, int64_t n, int m2,
+                             const double* X, int64_t ldx, double* Y, int64_t ldy, double alpha_re, double alpha_im,
+                             double sigma, int overwrite) {
     chain_release();
     chain_wait();
     const int mc = m2 >> 1;

@@ -31,10 +31,11 @@ constexpr int kT = 128;       // threads of the transfer passes' CTAs
 constexpr int kColTile = 32;  // columns of one contraction CTA at most
 
 // acc0 += A[r0, 0:K]·B[0:K, c], acc1 likewise for r1, with the row of A at a0/a1
-// (stride sa between contraction indices) and the column of B at b (stride ldb).
+// (stride sa between contraction indices) and the column of B at b (stride ldb).  A is
+// matrix data, which no kernel of the chain writes; B comes from earlier kernels.
 template <bool UNIT>
 __device__ __forceinline__ void dot2(double& acc0, double& acc1, const double* __restrict__ a0,
-                                     const double* __restrict__ a1, int64_t sa, const double* __restrict__ b,
+                                     const double* __restrict__ a1, int64_t sa, const double* b,
                                      int64_t ldb, int K) {
     constexpr int U = 8;
     double x[U], u[U], v[U];
@@ -42,7 +43,7 @@ __device__ __forceinline__ void dot2(double& acc0, double& acc1, const double* _
 #pragma unroll
         for (int i = 0; i < U; ++i) {
             if (i < n) {
-                x[i] = __ldg(b + i * ldb);
+                x[i] = b[i * ldb];
                 u[i] = __ldg(a0 + (UNIT ? i : i * sa));
                 v[i] = __ldg(a1 + (UNIT ? i : i * sa));
             } else {
@@ -118,8 +119,7 @@ __global__ void __launch_bounds__(32 * kSplitWarps64) k_coupling64(int chunks, c
                                                    const int32_t* __restrict__ rowptr,
                                                    const int32_t* __restrict__ other,
                                                    const int32_t* __restrict__ blk, const double* __restrict__ S,
-                                                   const double* __restrict__ xhat, double* __restrict__ yhat, int k,
-                                                   int m) {
+                                                   const double* xhat, double* yhat, int k, int m) {
     chain_release();
     chain_wait();
     const int pos = blockIdx.x / chunks;
@@ -149,10 +149,9 @@ template <bool TRANS>
 __global__ void __launch_bounds__(32 * kSplitWarps64) k_leaf64(
     int chunks, const int32_t* __restrict__ order, const int32_t* __restrict__ leaves, const int32_t* __restrict__ cl_off,
     const int32_t* __restrict__ cl_size, const int32_t* __restrict__ perm, const double* __restrict__ V,
-    const double* __restrict__ yhat, const int32_t* __restrict__ nptr, const int32_t* __restrict__ nother,
+    const double* yhat, const int32_t* __restrict__ nptr, const int32_t* __restrict__ nother,
     const int32_t* __restrict__ nblk, const int64_t* __restrict__ near_off, const double* __restrict__ G,
-    const double* __restrict__ Xp, double* __restrict__ Y, int64_t ldy, double alpha, double sigma, int k, int m,
-    int overwrite) {
+    const double* Xp, double* Y, int64_t ldy, double alpha, double sigma, int k, int m, int overwrite) {
     chain_release();
     chain_wait();
     const int pos = blockIdx.x / chunks;
@@ -192,9 +191,8 @@ __global__ void __launch_bounds__(32 * kSplitWarps64) k_leaf64(
 __global__ void __launch_bounds__(32) k_leaf_fwd64(int chunks, const int32_t* __restrict__ leaves,
                                                    const int32_t* __restrict__ cl_off,
                                                    const int32_t* __restrict__ cl_size,
-                                                   const double* __restrict__ V, const double* __restrict__ Xp,
-                                                   double* __restrict__ xhat, int k, int m, int* __restrict__ flag,
-                                                   int64_t nflag, unsigned* __restrict__ claim, int nclaim) {
+                                                   const double* __restrict__ V, const double* Xp, double* xhat, int k,
+                                                   int m, int* flag, int64_t nflag, unsigned* claim, int nclaim) {
     chain_release();
     chain_wait();
     // the downward pass starts from cleared flags and claim tickets
@@ -283,8 +281,8 @@ template <int CS>
 __global__ void __launch_bounds__(kT) k_up64(const int32_t* __restrict__ leaves, int NL,
                                              const int32_t* __restrict__ parent, const int32_t* __restrict__ son0,
                                              const int32_t* __restrict__ son1, const double* __restrict__ E,
-                                             const double* __restrict__ kron, double* xhat,
-                                             unsigned* __restrict__ cnt, int k, int m) {
+                                             const double* __restrict__ kron, double* xhat, unsigned* cnt, int k,
+                                             int m) {
     chain_release();
     chain_wait();
     __shared__ double xs[2 * 64 * CS], ys[2 * 64 * CS], F[96];
@@ -388,8 +386,8 @@ template <int CS>
 __global__ void __launch_bounds__(kT) k_down64(const int32_t* __restrict__ order, int n_items, int slices,
                                                const int32_t* __restrict__ parent, const double* __restrict__ E,
                                                const double* __restrict__ kron, double* yhat,
-                                               unsigned* __restrict__ claim, unsigned* flag, int* __restrict__ err,
-                                               int k, int m, long long spin_limit) {
+                                               unsigned* claim, unsigned* flag, int* err, int k, int m,
+                                               long long spin_limit) {
     chain_release();
     chain_wait();
     __shared__ double xs[64 * CS], ys[4 * 64 * CS], F[48];
