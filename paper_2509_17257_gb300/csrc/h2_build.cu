@@ -274,9 +274,8 @@ void balance_order(std::vector<TcItem>& v, Cost cost, int G) {
 }
 
 // Cuts the long items of a short list in two, so that their terms run on two CTAs:
-// each half adds its result to the cleared output, and a sum of two does not depend on
-// their order.  (The additions take place in memory, where FP32 subnormals count as
-// zero.)  Items of at least 4 terms and more than half of a CTA's share of the work, in
+// each half adds its result to the cleared output (add_half), and a sum of two does not
+// depend on their order.  Items of at least 4 terms and more than half of a CTA's share of the work, in
 // lists of at most max_items: where CTAs are left over, a launch takes as long as its
 // longest item; where they are not, the cuts only add results to store.  µs whole →
 // halves, q = 4: n = 2048, m = 1: 68 → 57 and q = 3: 55 → 46; n = 4096, m = 32: 82 → 70;

@@ -175,6 +175,7 @@ struct TcGemmParams {
     // by log2(e) / length: S_b[ν, μ] = 2^(-|node_{t,ν} - node_{s,μ}|) for ν, μ < k
     const float4* nodes;
     int KP;
+    int mreal;  // modes 0 to 2: columns before the padding to mc
     // modes 0 and 1 of the complex product: terms marked kTermImag apply i·act
     int cplx;
 };

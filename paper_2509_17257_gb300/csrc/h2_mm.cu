@@ -1065,6 +1065,7 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
         cp.bmat = bmat;
         cp.R = R;
         cp.mc = ml;
+        cp.mreal = mc;
         cp.yhat = yhat;
         cp.k = k;
         cp.ldc = ml;
@@ -1103,6 +1104,7 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
         lp.bmat = bmat;
         lp.R = R;
         lp.mc = ml;
+        lp.mreal = mc;
         lp.leaves = A->d_leaves;
         lp.cl_off = A->d_cl_off;
         lp.cl_size = A->d_cl_size;

@@ -158,6 +158,53 @@ __device__ __forceinline__ void stage_copy_elect(uint32_t meta, int m0, int m1, 
         "l"(pol_a), "r"(dst_b), "l"(src_b), "r"(bytes_b), "l"(pol_b)
         : "memory");
 }
+// One of two halves of an item's result onto its cleared output: entries i < count at
+// out[i·stride], of which those from `real` on are zero (the columns' padding; ROW: out and
+// count are multiples of 4 floats, stride is 1).  An addition in memory counts FP32
+// subnormals, its result too, as zero (a product whose results are of 1e-38 was off by 14 %
+// instead of 6e-4), so it is for values from 2^-100 on: two of them, or one and a smaller
+// normal one, differ by a multiple of 2^-124 or more, and a subnormal is less than half of
+// the distance from one of them to its neighbours.  A thread with smaller values exchanges:
+// the half that finds zero leaves its value, the other one stores the sum of both.  So the
+// sum is the rounded one in any order of the halves.  µs, additions of 32 or 64 values one
+// by one → this (rows by vectors; BF16, two lanes a column): FP32 n = 6000, q = 4, m = 1:
+// 58.7 → 59.7, m = 32: 79.6 → 76.2, m = 64: 101.1 → 96.3; BF16 m = 1: 47.0 → 48.0, m = 32:
+// 59.0 → 60.5; n = 4096, m = 32: 50.3 → 48.6.  All by exchange, a round trip for every 16
+// values: BF16, n = 4096, m = 32: 63.
+template <bool ROW, int N>
+__device__ __forceinline__ void add_half(float* out, int64_t stride, const float (&v)[N], int count, int real) {
+    constexpr uint32_t kAdd = 27u << 23;  // 2^-100
+    uint32_t lo = ~0u, hi = 0u;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const uint32_t b = i < real ? __float_as_uint(v[i]) & 0x7FFFFFFFu : kAdd;
+        lo = min(lo, b);
+        if (i < real) hi = max(hi, b);
+    }
+    if (hi == 0u) return;
+    if (lo >= kAdd) {
+        if constexpr (ROW) {
+#pragma unroll
+            for (int i = 0; i < N; i += 4)
+                if (i < count)
+                    asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(out + i), "f"(v[i]),
+                                 "f"(v[i + 1]), "f"(v[i + 2]), "f"(v[i + 3])
+                                 : "memory");
+        } else {
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+                if (i < count) atomicAdd(out + i * stride, v[i]);
+        }
+        return;
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        if (i >= real || v[i] == 0.f) continue;
+        float* o = out + i * stride;
+        const float other = atomicExch(o, v[i]);
+        if (other != 0.f) asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" ::"l"(o), "f"(other + v[i]) : "memory");
+    }
+}
 // Named barrier over `count` threads that also ORs a predicate across them.
 __device__ __forceinline__ bool bar_red_or(int id, int count, bool pred) {
     uint32_t r;
@@ -832,12 +879,7 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
                     if (n < cur_nt) out = SYSF(cur, zp) + ((int64_t)cur_off + n) * ldci;
                 }
                 if (!LIST && (cur.np & kItemHalf)) {
-                    // one of two halves, onto zero
-                    if (out) {
-#pragma unroll
-                        for (int i = 0; i < kSums; ++i)
-                            if (i < mci) atomicAdd(out + i, sum[i]);
-                    }
+                    if (out) add_half<true>(out, 1, sum, mci, p.mreal);
                 } else if (out) {
                     if (vec4) {
 #pragma unroll
@@ -898,7 +940,31 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
                     failed = true;
                 }
             }
-            if (!failed) {
+            // one of two halves of an item: the two lanes of a row pair take 32 rows of the
+            // output each, which halves a thread's additions
+            const bool half = !LIST && (cur.np & kItemHalf);
+            if (!failed && half) {
+                const int acc = (it - 1) % kAccBufs;
+                tc_fence_after();
+                const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * acc_cols);
+                uint32_t r0[32], r1[32];
+                tmem_ld32_async(ta, r0);
+                tmem_ld32_async(ta + 32, r1);
+                tmem_wait_ld();
+                const bool odd = lane & 1;
+                float v[32];
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    const uint32_t other = __shfl_xor_sync(0xffffffffu, odd ? r0[j] : r1[j], 1);
+                    v[j] = __uint_as_float(odd ? r1[j] : r0[j]) + __uint_as_float(other);
+                }
+                const int j0 = odd ? 32 : 0, rows = (MODE == 1 ? cur_nt : min(np, p.k)) - j0;
+                float* out = MODE == 1 ? p.zp + (int64_t)cur_off * p.ldc + i : p.yhat + (int64_t)id * p.k * p.ldc + i;
+                if (row >= 0 && i < p.mc) add_half<false>(out + (int64_t)j0 * p.ldc, p.ldc, v, rows, rows);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&acce_bar[acc]);
+            } else if (!failed) {
                 const int acc = (it - 1) % kAccBufs;
                 tc_fence_after();
                 // both halves of the accumulator in flight, one wait; the row pair
@@ -967,14 +1033,7 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
                 if (lane == 0) atomicExch(p.err, 6);
                 abort_flag = 1;
                 break;
-            } else if (writer && !LIST && (cur.np & kItemHalf)) {
-                // one of two halves, onto zero
-                float* out = MODE == 1 ? p.zp + (int64_t)cur_off * p.ldc + i : p.yhat + (int64_t)id * p.k * p.ldc + i;
-                const int rows = MODE == 1 ? cur_nt : min(np, p.k);
-#pragma unroll
-                for (int j = 0; j < kAccCols; ++j)
-                    if (j < rows) atomicAdd(out + (int64_t)j * p.ldc, sum[j]);
-            } else if (writer) {
+            } else if (writer && !half) {
                 if (MODE != 1) {
                     float* out = p.yhat + (int64_t)id * p.k * p.ldc;
 #pragma unroll
