@@ -425,7 +425,6 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
     __shared__ __align__(16) int4 s_term[2][kTermBatch];  // the producers' current terms
     __shared__ int abort_shared;
     volatile int& abort_flag = abort_shared;
-    chain_release();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int R = p.R;
     const int M = R <= 64 ? 64 : 128;
@@ -473,8 +472,10 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
-    // the barriers, TMEM and the item count (of static lists) are set up while the
-    // launch before still runs
+    // This CTA has its TMEM before a later launch can start (that one's CTAs may come to
+    // this SM, take TMEM in their turn and wait for this grid).  The barriers, TMEM and
+    // the item count (of static lists) are set up while the launch before still runs.
+    chain_release();
     chain_wait();
 
     if (warp == 0 || warp == tc_producer2<KIND>()) {

@@ -1,6 +1,6 @@
-"""Kernels that start under their predecessor's tail (those that call chain_wait) are alive while that one still writes.
-Only what no kernel of a product writes may be promised to be read-only there: read from the sources, every
-__restrict__ parameter and every __ldg of these kernels names matrix data or an index list."""
+"""Dependent launches, read from the sources.  Kernels that call chain_wait start under their predecessor's tail and are
+alive while that one still writes.  Only what no kernel of a product writes may be promised to be read-only there:
+every __restrict__ parameter and every __ldg of these kernels names matrix data or an index list."""
 import glob
 import os
 import re
@@ -59,3 +59,11 @@ def test_contractions_promise_their_matrix_operand_only():
     text = src[at:block_end(src, at)]
     assert set(re.findall(r"__restrict__\s+(\w+)", text)) == {"a0", "a1"}
     assert set(re.findall(r"__ldg\((\w+)", text)) == {"a0", "a1"}
+
+
+def test_tensor_memory_is_taken_before_the_successor_may_start():
+    """A successor's CTA that took TMEM of an SM first, and then waited for this grid, would leave both waiting: every
+    CTA has its TMEM (allocated, and seen by the whole CTA past a barrier) when it lets the next launch start."""
+    _, body = KERNELS["k_tc_gemm"]
+    alloc = body.index("tcgen05.alloc")
+    assert alloc < body.index("__syncthreads()", alloc) < body.index("chain_release()") < body.index("chain_wait()")
