@@ -402,8 +402,9 @@ int h2_batch_block_cg(h2_batch* batch, const double* const* B, const int64_t* ld
  *      cores with the CUDA-core transfer passes stopping at the upward cut,
  *      whose clusters above the cut become transfer items of the coupling
  *      launch (path 5; FP32 and BF16);
- *   2. on the best path, the pipeline stage count of the tensor-core kernels
- *      (4 and 5 against as many as fit);
+ *   2. on the best path, fewer pipeline stages of the tensor-core kernels than
+ *      fit: 4 and 5 where more than 5 do (BF16: 6 or 9), else one fewer (FP32:
+ *      3 or 4 fit);
  *   3. on paths 1 and 5, the cut targets of the CUDA-core transfer passes (half and
  *      twice the default, upward first).
  * The fastest variant is kept for later products of this precision whose

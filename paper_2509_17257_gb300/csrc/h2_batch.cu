@@ -435,9 +435,14 @@ int h2_autotune_ex(h2_matrix* A, int64_t m, int32_t dtype, void* stream, h2_tune
     }
     if (dtype == H2_F32 ? A->tc.hybrid : A->tc.hybrid_bf16) trial(Tune{kPathTcHybrid, 0}, keep_up, keep_down);
     if (dtype == H2_F32) trial(Tune{kPathSimt, 0}, keep_up, keep_down);
-    // 2. the stage count of the tensor-core kernels on the best path
-    if (!rc && best_t.path != kPathSimt)
-        for (int sc : {4, 5}) trial(Tune{best_t.path, (int8_t)sc}, best_up, best_down);
+    // 2. fewer stages of the tensor-core kernels than fit, on the best path: 4 and 5 where
+    // more than 5 do (BF16: 6 or 9), else one fewer (FP32: 3 or 4 fit)
+    if (!rc && best_t.path != kPathSimt) {
+        const int fit = tc_stages(mc, dtype == H2_BF16 ? 0 : 1);
+        const int8_t path = best_t.path;
+        for (int sc : {fit > 5 ? 4 : fit - 1, fit > 5 ? 5 : 0})
+            if (sc >= 2) trial(Tune{path, (int8_t)sc}, best_up, best_down);
+    }
     // 3. the cuts of the CUDA-core transfer passes, upward then downward
     const bool subtree = A->pairs_built && A->use_kron;
     if (!rc && (best_t.path == kPathTcOwn || best_t.path == kPathTcHybrid) && subtree) {

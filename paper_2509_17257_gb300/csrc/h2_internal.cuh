@@ -632,6 +632,9 @@ int tc_prepare();
 // transfer-pass bookkeeping, kernel attributes), so that the product itself
 // allocates nothing (e.g. while it is captured into a CUDA graph).
 int product_prepare(h2_matrix* A, int64_t m, int32_t dtype, cudaStream_t st);
+// Pipeline stages that fit for a chunk of mc columns (all modes but the matrix-free
+// coupling); launch_tc_gemm takes fewer with 2 <= stages below that.
+int tc_stages(int mc, int kind);
 int launch_tc_gemm(int mode, int kind, TcGemmParams p, cudaStream_t st, int stages = 0, bool overlap = false);
 // Rebuild the CUDA-core transfer passes' lists of pairs for other cut targets.
 int set_transfer_targets(h2_matrix* A, int up_target, int down_target, cudaStream_t st);

@@ -1285,6 +1285,11 @@ int tc_prepare() {
     return 0;
 }
 
+int tc_stages(int mc, int kind) {
+    const int R = round16(2 * mc);
+    return tc_geometry(R, 0, kind, R <= 64).nstages;
+}
+
 int launch_tc_gemm(int mode, int kind, TcGemmParams p, cudaStream_t st, int stages, bool overlap) {
     const bool narrow = p.R <= 64;
     TcGeometry g = tc_geometry(p.R, mode, kind, narrow);

@@ -61,3 +61,16 @@ def test_tuning_rejects_bad_arguments(case):
     with pytest.raises(P.H2Error) as e:
         P.h2_autotune_ex(G.handle, 8, "f64")
     assert e.value.code == P.H2_E_BADARG
+
+
+@pytest.mark.parametrize("dtype,m,fit", [("f32", 6, 4), ("f32", 24, 3), ("f32", 50, 4), ("bf16", 24, 6), ("bf16", 50, 9)])
+def test_every_stage_count_tried_is_another_launch(case, dtype, m, fit):
+    """Stage counts are tried below the number that fits (shared memory over a stage's bytes); a count from that number
+    on is the untuned launch again."""
+    P, H, G = case
+    r = P.h2_autotune_ex(G.handle, m, dtype)
+    # the untuned paths come first, then the stage trials, then the cuts' (on the best variant so far)
+    untuned = [c for c in r["candidates"] if c["stages"] == 0]
+    tried = [c["stages"] for c in r["candidates"] if c["stages"]]
+    assert untuned and (tried or r["path"] == 4)
+    assert all(2 <= t < fit for t in tried)
