@@ -163,10 +163,12 @@ __global__ void k_coupling_entries(const int32_t* __restrict__ adm_row, const in
     }
 }
 
-// FP32 tensor nodes for the matrix-free coupling: nodes4[c·KP + ν] = scale·ξ_{c,ν}
-// (x, y, z, 0) for ν < k, zero for k <= ν < KP; with scale = log2(e) / length the
-// kernel is 2^(-|difference|) (kept finite: at 1e38 lengths its values are 0 or 1).
-__global__ void k_nodes4(const double* __restrict__ nodes, int64_t nc, int q, int KP, double scale,
+// FP32 tensor nodes for the matrix-free coupling: nodes4[c·KP + ν] = scale·(ξ_{c,ν} -
+// origin) (x, y, z, 0) for ν < k, zero for k <= ν < KP; with scale = log2(e) / length the
+// kernel is 2^(-|difference|) (kept finite: at 1e38 lengths its values are 0 or 1).  The
+// origin is the centre of the points' box: only differences count, and FP32 rounds
+// relative to the distance from it (a unit cube 1000 away from zero: error 7e-5 → 8e-7).
+__global__ void k_nodes4(const double* __restrict__ nodes, int64_t nc, int q, int KP, double scale, double3 origin,
                          float4* __restrict__ nodes4) {
     const int k = q * q * q;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nc * KP; e += (int64_t)gridDim.x * blockDim.x) {
@@ -176,7 +178,8 @@ __global__ void k_nodes4(const double* __restrict__ nodes, int64_t nc, int q, in
         if (nu < k) {
             double x[3];
             tensor_node(nodes + (size_t)c * 3 * q, q, nu, x);
-            for (int d = 0; d < 3; ++d) x[d] = fmin(fmax(scale * x[d], -3e38), 3e38);
+            const double o[3] = {origin.x, origin.y, origin.z};
+            for (int d = 0; d < 3; ++d) x[d] = fmin(fmax(scale * (x[d] - o[d]), -3e38), 3e38);
             v = make_float4((float)x[0], (float)x[1], (float)x[2], 0.f);
         }
         nodes4[e] = v;
@@ -1224,7 +1227,9 @@ int build_tc(h2_matrix* A, bool bf16, bool tf32, cudaStream_t st) {
     if (tf32 && !A->cplx) {
         if ((rc = device_alloc(A, (void**)&D.nodes4, (size_t)nc * KP * sizeof(float4)))) return rc;
         const unsigned g = (unsigned)std::min<int64_t>((nc * KP + 255) / 256, 152 * 16);
-        k_nodes4<<<g, 256, 0, st>>>(A->d_nodes, nc, A->q, KP, 1.4426950408889634 / A->length, D.nodes4);
+        const double* b = A->T.box.data();  // the root's
+        const double3 origin = make_double3(0.5 * (b[0] + b[3]), 0.5 * (b[1] + b[4]), 0.5 * (b[2] + b[5]));
+        k_nodes4<<<g, 256, 0, st>>>(A->d_nodes, nc, A->q, KP, 1.4426950408889634 / A->length, origin, D.nodes4);
         H2_LAUNCH_CHECK();
     }
 

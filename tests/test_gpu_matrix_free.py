@@ -86,3 +86,14 @@ def test_matrix_free_refuses_replaced_couplings(P):
     P.h2_coupling_set(G.handle, S)
     with pytest.raises(P.H2Error):
         G.matmul(X, Y, dtype="f32mf")
+
+
+@pytest.mark.parametrize("shift", [(0.0, 0.0, 0.0), (900.0, 0.0, 0.0), (-1000.0, 3e4, 700.0)])
+def test_matrix_free_does_not_depend_on_where_the_points_lie(P, shift):
+    """Only differences of nodes count: away from the origin the error is that of the same points around it."""
+    n, m = 3000, 5
+    pts = ellipsoid_points(n, (1.0, 0.8, 0.6), 4) + np.array(shift)
+    G = P.H2Matrix(pts, q=3, leaf_size=64, eta=2.0, sigma=1e-2, length=0.5, precisions=("f32",))
+    X = gaussian_rhs(n, m, 3)
+    Y0 = np.zeros((n, m))
+    assert rel_fro(_apply(G, X, Y0, 1.0, "f32mf"), _apply(G, X, Y0, 1.0, "f64")) <= TOL_STORED
