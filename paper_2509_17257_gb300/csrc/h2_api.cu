@@ -318,7 +318,7 @@ int h2_info(const h2_matrix* A, h2_info_t* info) {
     // tensor-core chain with the transfer passes as lists of pairs: leaves, a launch per stage of
     // both passes, coupling, leaf phase, scatter into Y.  Without: gather, upward pass, coupling,
     // downward pass, leaf phase, scatter, three packing launches, + zeroing of clusters without couplings
-    const bool pairs = A->pairs_built && A->use_kron;
+    const bool pairs = A->pairs_built;
     const bool hybrid = pairs && A->tc.hybrid && A->tc.h_default;
     info->launches_tc = 0;
     if (A->tc.built && pairs)

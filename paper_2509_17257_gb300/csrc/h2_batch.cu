@@ -207,7 +207,7 @@ bool flow_batch_ok(h2_batch* b, const std::vector<int>& sys, const int64_t* m, i
     for (int i : sys) {
         const h2_matrix* A = b->mats[i];
         multi = multi && flow_batchable(b->mats[i], m[i]) && A->use_flow != 0;
-        pairs = pairs && A->pairs_built && A->use_kron && A->use_flow != 1;
+        pairs = pairs && A->pairs_built && A->use_flow != 1;
     }
     return multi && !pairs;
 }
@@ -444,7 +444,7 @@ int h2_autotune_ex(h2_matrix* A, int64_t m, int32_t dtype, void* stream, h2_tune
             if (sc >= 2) trial(Tune{path, (int8_t)sc}, best_up, best_down);
     }
     // 3. the cuts of the CUDA-core transfer passes, upward then downward
-    const bool subtree = A->pairs_built && A->use_kron;
+    const bool subtree = A->pairs_built;
     if (!rc && (best_t.path == kPathTcOwn || best_t.path == kPathTcHybrid) && subtree) {
         const int up0 = best_up;
         for (int u : {kUpTasks / 2, kUpTasks * 2}) trial(best_t, u, best_down);

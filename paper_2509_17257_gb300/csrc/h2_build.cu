@@ -1000,6 +1000,7 @@ int hybrid_lists(h2_matrix* A, cudaStream_t st) {
     D.hybrid = false;
     D.hybrid_bf16 = false;
     D.h_default = false;
+    if (!A->pairs_built) return 0;  // the upward pass below the cut is theirs
     // FP32 lists: the Eᵀ tiles of the tensor-core transfer passes; BF16 lists: the
     // split BF16 Eᵀ tiles
     const bool f32 = D.flow && D.et_off_host.size() == (size_t)nc;

@@ -626,7 +626,6 @@ int launch_leaf64(h2_matrix* A, const double* V, const double* G, const double* 
                   int64_t ldy, double alpha, int m, bool trans, bool overwrite, bool overlap, cudaStream_t st);
 
 // tcgen05 BF16 kernels (h2_tc.cu)
-int tc_smem_bytes();
 int tc_prepare();
 // Allocate everything a product of m columns in dtype needs (workspace,
 // transfer-pass bookkeeping, kernel attributes), so that the product itself

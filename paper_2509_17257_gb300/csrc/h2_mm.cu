@@ -873,7 +873,7 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
         const int stg = tn.stages;
         // the transfer passes as lists of pairs (q = 2, 3, 4), with the columns padded to
         // a multiple of 4
-        const bool fast = A->pairs_built && A->use_kron;
+        const bool fast = A->pairs_built;
         bool want_flow = !fast;
         if (tn.path == kPathTcOwn || tn.path == kPathTcHybrid) want_flow = false;
         if (tn.path == kPathTcFlow || tn.path == kPathTcFused) want_flow = true;

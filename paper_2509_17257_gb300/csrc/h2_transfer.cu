@@ -64,9 +64,10 @@ __global__ void k_pair_factors(const int2* __restrict__ pair, int64_t np, const 
 
 // Rows 2i, 2i + 1 (high and low parts of column i) of a split tile of kp
 // contraction columns, for columns i0 <= i < i1: entry κ of column i is
-// x[κ·ld + i - i0] for κ < rows and i - i0 < valid, zero elsewhere.  The layout and
-// the split are put_act4's; a thread has one column, so its rows' place is fixed
-// and the entries advance by whole core matrices.
+// x[κ·ld + i - i0] for κ < rows and i - i0 < valid, zero elsewhere.  es = 4 (TF32): v and
+// v - tf32(v), the MMA reading the top 19 bits of the first; es = 2 (BF16): bf16(v) and
+// bf16(v - bf16(v)).  A thread has one column, so its rows' place (cm_off) is fixed and
+// the entries advance by whole core matrices.
 __device__ __forceinline__ void pack_cols(uint8_t* tile, int kp, int es, int i0, int i1, const float* x, int ld,
                                           int rows, int valid) {
     const int ni = i1 - i0, per = blockDim.x / ni, g0 = threadIdx.x / ni, i = threadIdx.x - g0 * ni;
@@ -478,7 +479,7 @@ int upload_pass(h2_matrix* A, PairPass& ps, std::vector<PairItem>& items, const 
 int build_pairs(h2_matrix* A, cudaStream_t st) {
     ++A->pairs_gen;
     A->up_cut = 0;
-    if (A->q < 2 || A->q > 4) return 0;
+    if (A->q < 2 || A->q > 4 || !A->use_kron) return 0;
     const Tree& T = A->T;
     const int64_t nc = A->nc, NL = (int64_t)A->leaves.size();
     // A tree that peels off a leaf a level has paths as long as it has leaves, and
