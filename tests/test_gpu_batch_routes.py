@@ -148,3 +148,28 @@ def test_cached_graph_follows_the_shift(kron, dtype, monkeypatch):
             torch.cuda.synchronize()
             assert rel_fro(y.cpu().numpy(), ref.cpu().numpy()) <= 3e-6
     B.close()
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
+def test_branches_equal_single_products_of_whole_items_bit_for_bit(dtype, monkeypatch):
+    """A captured branch runs whole items and no hybrid upward pass; with both switched off a single product runs the
+    same lists, so the bits agree.  (By default a single FP32 product may sum in another order.)"""
+    torch = require_cuda()
+    import paper_2509_17257_gb300.build as bld
+    bld.build()
+    import paper_2509_17257_gb300 as P
+    monkeypatch.setenv("H2_TC_HALVES", "0")
+    monkeypatch.setenv("H2_TC_HYBRID", "0")
+    mats = [P.H2Matrix(ellipsoid_points(n, (1.0, 0.7, 0.5), 40 + i), q=q, leaf_size=64, eta=2.0, sigma=1e-2,
+                       precisions=("f32", "bf16")) for i, (n, q, _) in enumerate(SIZES)]
+    B = P.H2Batch(mats)
+    X = [torch.from_numpy(gaussian_rhs(n, m, 10 + i)).cuda() for i, (n, _, m) in enumerate(SIZES)]
+    Y = [torch.from_numpy(gaussian_rhs(n, m, 50 + i)).cuda() for i, (n, _, m) in enumerate(SIZES)]
+    ref = [y.clone() for y in Y]
+    for A, x, y in zip(mats, X, ref):
+        A.matmul(x, y, alpha=0.5, dtype=dtype)
+    B.matmul(X, Y, alpha=0.5, dtype=dtype)
+    torch.cuda.synchronize()
+    for y, r in zip(Y, ref):
+        assert torch.equal(y, r)
+    B.close()
