@@ -120,7 +120,7 @@ typedef struct h2_info_t {
                              most 64 columns: with q = 2, 3, 4 the transfer passes are lists
                              of pairs, otherwise three packing launches are counted        */
     int32_t kernel;       /* h2_kernel of the build                                     */
-    int32_t hybrid;       /* 1: the FP32 and BF16 tensor-core products take, by default,
+    int32_t hybrid;       /* 1: the FP32 tensor-core product takes, by default,
                              the hybrid upward pass (the lists of pairs stop at the first
                              cut, the clusters above it are transfer items of the coupling
                              launch)                                                      */
@@ -134,7 +134,8 @@ typedef struct h2_info_t {
  *     H2_TC_TRANSFER=0|1     FP32 transfer passes on the CUDA cores / the tensor cores
  *     H2_TC_HYBRID=0|1       the hybrid upward pass off / on
  *     H2_KRON=0              transfer passes on the dense transfer matrices
- *     H2_HYBRID_ROUND_TERMS  coupling terms per CTA between two heights of the hybrid
+ *     H2_TC_HALVES=0         short work lists without cutting their long items in halves
+ *     H2_HYBRID_ROUND_TERMS  coupling terms per SM between two heights of the hybrid
  *                            pass's transfer items (1..64, default 16)
  *   read by h2_batch_create for that batch:
  *     H2_BATCH_MULTI=0       batched FP32 products as per-system graph branches

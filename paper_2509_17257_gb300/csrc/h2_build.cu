@@ -970,10 +970,10 @@ int flow_lists(h2_matrix* A, const FlowTiles& ft, const std::vector<int64_t>& s_
 // sons, a coupling item for its source cluster.  Keys order the list so that
 // every wait points to a strictly smaller key (each CTA takes its items in list
 // order, so the item with the smallest unfinished key can always proceed):
-//   transfer item at height h above the cut (h = 1 for fathers of task roots): 2h - 1;
+//   transfer item at height h above the cut (h = 1 for fathers of clusters at the cut): 2h - 1;
 //   coupling item reading only clusters at or below the cut: key 2r for the
 //     rounds r < H between two heights, the smallest items first and about
-//     kHybridRoundTerms terms per CTA per round (the time a transfer item takes
+//     kHybridRoundTerms terms per SM per round (the time a transfer item takes
 //     to become readable), the rest key 2H;
 //   coupling item reading a cluster above the cut: key 2H too if its highest
 //     source is at height H - 3 or below, else 2H + 1.
@@ -983,7 +983,7 @@ int flow_lists(h2_matrix* A, const FlowTiles& ft, const std::vector<int64_t>& s_
 // last.
 constexpr int kHybridRoundTerms = 16;  // H2_HYBRID_ROUND_TERMS overrides it (1..64)
 // The product takes the hybrid upward pass by default when the coupling work
-// that reads no cluster above the cut gives every CTA at least this many terms
+// that reads no cluster above the cut gives every SM at least this many terms
 // per height above the cut: then the chain of transfer items (a few
 // microseconds per height) runs under that work instead of after it.  FP32, q = 4,
 // m = 32, without → with (µs): 8 terms per height (n = 20011) 120 → 123, 10 (24000)
@@ -1057,7 +1057,7 @@ int hybrid_lists(h2_matrix* A, cudaStream_t st) {
             if (hs > 0) late.push_back(Free{j1 - j0, it, hs});
             else free_items.push_back(Free{j1 - j0, it, 0});
         }
-        // smallest first into the rounds, each round up to kHybridRoundTerms terms per CTA
+        // smallest first into the rounds, each round up to kHybridRoundTerms terms per SM
         std::stable_sort(free_items.begin(), free_items.end(),
                          [](const Free& a, const Free& b) { return a.cost < b.cost; });
         const int64_t budget = (int64_t)round_terms * kTcGrid;

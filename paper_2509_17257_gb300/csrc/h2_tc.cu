@@ -1091,9 +1091,11 @@ __global__ void __launch_bounds__(tc_threads<KIND>(), NARROW ? 2 : 1) k_tc_gemm(
                 // swap halves through shared memory.  The source nodes come with the stage
                 // and are read by the whole warp at once (one broadcast per node); the
                 // row's own node stays in a register over the item.  The nodes are scaled,
-                // so a value is a hardware square root and a hardware 2^x (relative error
-                // below 1e-6): 8 instructions and 16 cycles of the SFU per warp.  n = 65536,
-                // q = 4, m = 32: 786 µs with node loads from global memory, shuffles and one
+                // so a value is a hardware square root and a hardware 2^x: 8 instructions and
+                // 16 cycles of the SFU per warp.  Their relative errors, 2^-23 and 2^-22 at
+                // most, make a relative error of r ln 2 · 2^-23 + 2^-22 of the value 2^-r, which
+                // grows with r; r 2^-r is 0.53 at most, so the absolute error stays below 3e-7
+                // (besides the FP32 rounding of the nodes).  n = 65536, q = 4, m = 32: 786 µs with node loads from global memory, shuffles and one
                 // CTA per SM, 670 with the nodes in the stage, 402 with two CTAs, about 190
                 // with scaled nodes, a square root and 16-byte exchanges.
                 if (ok && !end) {

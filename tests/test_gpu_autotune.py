@@ -1,7 +1,7 @@
 """The product autotuner (h2_autotune_ex): it times the product paths (tensor
 cores with the CUDA-core or the tensor-core transfer passes, the latter alone
 or sharing the coupling and leaf launches, and the CUDA cores), then stage
-counts, then the cut targets of the subtree passes, and keeps the fastest.
+counts, then the cut targets of the lists of pairs, and keeps the fastest.
 Every candidate it leaves behind must still compute the same product: the
 tuned products are checked against the FP64 oracle, for FP32 and BF16, and
 for column counts in different classes."""
@@ -40,7 +40,7 @@ def test_tuned_products_stay_correct(case, dtype, m):
     assert (chosen["path"], chosen["stages"], chosen["up_target"], chosen["down_target"]) == \
         (r["path"], r["stages"], r["up_target"], r["down_target"])
     if dtype == "bf16":
-        # the BF16 product: the subtree passes, with or without the hybrid upward pass
+        # the BF16 product: the lists of pairs, with or without the hybrid upward pass
         assert 1 in {c["path"] for c in r["candidates"]} <= {1, 5}
     else:
         assert {1, 4} <= {c["path"] for c in r["candidates"]}

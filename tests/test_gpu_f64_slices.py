@@ -1,5 +1,6 @@
 """The FP64 phases (h2_mm64.cu) at the edges of their cuts: output pairs (odd k and odd leaf
-sizes), chunks of 128 pairs, column tiles of 32, slices of 1, 2 and 4 columns, 64-column tiles."""
+sizes), chunks of 32 pairs (ceil(rows / 2) times the columns, at most 32, of a tile), column
+tiles of 32, slices of 1, 2 and 4 columns, 64-column tiles."""
 import numpy as np
 import pytest
 
@@ -39,4 +40,25 @@ def test_f64_product_at_the_cuts(q, leaf, m):
             Yd.copy_(torch.from_numpy(Y0))
             product(Xd, Yd, alpha=0.5, dtype="f64")
             assert np.array_equal(first, Yd.cpu().numpy())
+    A.close()
+
+
+# leaves of one size each (a power of two of them): 31, 32 and 33 pairs of a leaf's rows and
+# columns, and twice as many; k = 27 has 14 row pairs: 28 pairs with 2 columns, 42 with 3
+@pytest.mark.parametrize("size,m", [(62, 1), (63, 1), (64, 1), (6, 11), (62, 2), (64, 2), (22, 3), (21, 3)])
+def test_f64_product_at_the_chunks(size, m):
+    torch = require_cuda()
+    import paper_2509_17257_gb300 as P
+
+    n = 16 * size
+    pts = ellipsoid_points(n, (0.6, 1.1, 1.9), 3)
+    H = O.H2Matrix(pts, q=3, leaf_size=size, eta=2.0, sigma=1e-2)
+    A = P.H2Matrix(pts, q=3, leaf_size=size, eta=2.0, sigma=1e-2, precisions=())
+    assert P.h2_info(A.handle)["n_leaves"] == 16
+    X, Y0 = gaussian_rhs(n, m, 5), gaussian_rhs(n, m, 6)
+    want = O.h2mm(H, 0.5, X, Y0)
+    for product in (A.matmul, A.matmul_transposed):  # the kernel is symmetric
+        Yd = torch.from_numpy(Y0).cuda()
+        product(torch.from_numpy(X).cuda(), Yd, alpha=0.5, dtype="f64")
+        assert rel_fro(Yd.cpu().numpy(), want) <= TOL
     A.close()

@@ -83,7 +83,7 @@ def test_transposed_of_a_nonsymmetric_matrix(P, dtype):
     """After the couplings are replaced by non-symmetric ones (S_(s,t) no longer
     S_(t,s)ᵀ), Aᵀ differs from A; the tensor-core product with Aᵀ (S_bᵀ tiles,
     column-cluster lists) must follow, including the tiles rebuilt by
-    h2_coupling_set.  A q = 4 tree so the subtree-owning transfer passes run."""
+    h2_coupling_set.  A q = 4 tree so the transfer passes are lists of pairs."""
     torch = require_cuda()
     pts = sphere_points(3000, 11)
     H, G = _pair(P, pts, q=4)
@@ -133,7 +133,7 @@ def test_pinned_host_buffers_in_place(P, dtype):
     """Pinned host X and Y (device-mapped) are read and updated where they are;
     the result equals the product on device copies, columns outside the views
     untouched.  A q = 4 tree, so the FP32 and BF16 products take the
-    subtree-owning transfer passes."""
+    transfer passes as lists of pairs."""
     torch = require_cuda()
     n = 3000
     pts = sphere_points(n, 8)

@@ -1,11 +1,10 @@
-"""The hybrid upward pass of the FP32 and BF16 tensor-core products: the CUDA-core
-subtree pass stops at its cut, and the clusters above the cut (x̂_t =
+"""The hybrid upward pass of the FP32 and BF16 tensor-core products: the lists of
+pairs stop at their first cut, and the clusters above the cut (x̂_t =
 E_s0ᵀ x̂_s0 + E_s1ᵀ x̂_s1, Alg. "forward/backward") are transfer items of the
 coupling launch, waiting for their sons' ready flags, with the coupling items
 that read them waiting in turn.  Checked against the FP64 oracle and the
-same product without it (H2_TC_HYBRID=0), for shapes where the subtree passes
-apply (k a multiple of 8: q = 2 and 4; columns a multiple of 4 per 64-column
-chunk), one, two and three chunks, leaves on several levels, cut targets
+same product without it (H2_TC_HYBRID=0), for q = 2 and 4, column counts that
+are multiples of 4, one, two and three 64-column chunks, leaves on several levels, cut targets
 moved by the tuner, and repeated products (bit for bit).  The BF16 product's
 transfer items take E_sᵀ as a BF16 tile and its BF16 remainder, so they add
 next to nothing to the BF16 coupling's error: against the oracle within the

@@ -1,6 +1,6 @@
-"""Host logic of the subtree-owning transfer passes (no GPU): the schedules
-that h2_build hands to the upward and downward pass kernels, replayed in
-numpy exactly as the kernels walk them, against a plain level-by-level pass
+"""The subtree schedules of the two transfer passes (h2_tree_schedule, no GPU):
+tasks that each own the subtree of a cut cluster, replayed in numpy as a caller
+that walks the tree would, against a plain level-by-level pass
 (Sec. 3, Alg. "fast_addeval": x̂_t = Σ E_{t'}ᵀ x̂_{t'} upwards, ŷ_{t'} += E_{t'} ŷ_t
 downwards), with random transfer matrices.
 
