@@ -43,18 +43,20 @@ def test_f64_product_at_the_cuts(q, leaf, m):
     A.close()
 
 
-# leaves of one size each (a power of two of them): 31, 32 and 33 pairs of a leaf's rows and
-# columns, and twice as many; k = 27 has 14 row pairs: 28 pairs with 2 columns, 42 with 3
+# groups of `size` points at the corners of a cube, a leaf each: 31, 32 and 33 pairs of a leaf's
+# row pairs and columns, and twice 31 and 32; k = 27 has 14 row pairs: 28 pairs with 2 columns,
+# 42 with 3
 @pytest.mark.parametrize("size,m", [(62, 1), (63, 1), (64, 1), (6, 11), (62, 2), (64, 2), (22, 3), (21, 3)])
 def test_f64_product_at_the_chunks(size, m):
     torch = require_cuda()
     import paper_2509_17257_gb300 as P
 
-    n = 16 * size
-    pts = ellipsoid_points(n, (0.6, 1.1, 1.9), 3)
+    corners = np.array([[i & 1, i >> 1 & 1, i >> 2] for i in range(8)], dtype=np.float64)
+    pts = np.repeat(corners, size, axis=0) + 0.1 * ellipsoid_points(8 * size, (0.6, 1.1, 1.9), 3)
+    n = len(pts)
     H = O.H2Matrix(pts, q=3, leaf_size=size, eta=2.0, sigma=1e-2)
     A = P.H2Matrix(pts, q=3, leaf_size=size, eta=2.0, sigma=1e-2, precisions=())
-    assert P.h2_info(A.handle)["n_leaves"] == 16
+    assert P.h2_info(A.handle)["n_leaves"] == 8  # of exactly `size` points then
     X, Y0 = gaussian_rhs(n, m, 5), gaussian_rhs(n, m, 6)
     want = O.h2mm(H, 0.5, X, Y0)
     for product in (A.matmul, A.matmul_transposed):  # the kernel is symmetric
