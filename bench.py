@@ -115,14 +115,16 @@ def product_bytes(n, k, m, nc, n_adm, nnz_near, elt, elt_x=8, elt_acc=4):
 def phase_bytes(n, k, m, nc, n_leaves, n_adm, nnz_near, elt, n_above=0):
     """Algorithmic bytes of each phase of the tensor-core FP32/BF16 product, as timed by
     h2_timing (coefficients, gathered X and leaf results in FP32; the caller's X, Y in FP64).
-    n_above: clusters above the upward cut computed in the coupling launch (hybrid)."""
+    n_above: clusters above the upward cut computed in the coupling launch (hybrid).  The
+    transfer passes read E_c as its three q×q Kronecker factors (FP32), not as k×k."""
     a = 4  # coefficient / gathered-block element size
+    e = a * 3 * round(k ** (1 / 3)) ** 2
     return {
-        "gather": 8 * n * m + a * n * m,
-        "leaf_fwd": (elt * (n * k + (nc - 1 - 2 * n_above) * k * k) + a * n * m
-                     + a * (nc - n_above) * k * m),  # upward pass fused in
+        # the leaves' launch gathers X and packs it; the upward pass is counted with it
+        "leaf_fwd": (a * n * k + e * (nc - 1 - 2 * n_above) + 8 * n * m + elt * 2 * n * m
+                     + a * (nc - n_above) * k * m),
         "coupling": elt * (n_adm + 2 * n_above) * k * k + 2 * a * nc * k * m + a * n_above * k * m,
-        "down": elt * (nc - 1) * k * k + 2 * a * nc * k * m,
+        "down": e * (nc - 1) + 2 * a * nc * k * m,
         "leaf_bwd_near": (elt * (n * k + nnz_near) + a * n_leaves * k * m + 2 * a * n * m
                           + a * n * m + 8 * n * m + 2 * 8 * n * m),  # leaf kernel, then the scatter into Y
     }

@@ -444,8 +444,8 @@ int h2_autotune_ex(h2_matrix* A, int64_t m, int32_t dtype, void* stream, h2_tune
             if (sc >= 2) trial(Tune{path, (int8_t)sc}, best_up, best_down);
     }
     // 3. the cuts of the CUDA-core transfer passes, upward then downward
-    const bool subtree = A->pairs_built;
-    if (!rc && (best_t.path == kPathTcOwn || best_t.path == kPathTcHybrid) && subtree) {
+    const bool pairs = A->pairs_built;
+    if (!rc && (best_t.path == kPathTcOwn || best_t.path == kPathTcHybrid) && pairs) {
         const int up0 = best_up;
         for (int u : {kUpTasks / 2, kUpTasks * 2}) trial(best_t, u, best_down);
         (void)up0;

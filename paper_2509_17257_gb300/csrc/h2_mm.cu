@@ -917,7 +917,9 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
         if (fast && !flow) {
             // one chain of launches: gather and leaves, then the upward pass (the leaves'
             // launch also clears the hybrid launch's ready flags, ŷ of the clusters without
-            // couplings or with a split list, and the leaf results if some are split)
+            // couplings or with a split list, and the leaf results if some are split, and
+            // the lists of pairs write the split tiles of X (leaves), x̂ and leaf ŷ)
+            marks.mark();
             if ((rc = launch_forward(A, X + c0, ldx, mc, ml, xhat, xcm, Xcm, R, es, hybrid, sbc.fflag,
                                      hybrid ? (int)nc : 0, zid, nzid, yhat, l_halves ? Xp : nullptr, overlap, st)))
                 return rc;
@@ -926,12 +928,10 @@ int run_chain_tc(h2_matrix* A, int kind, double alpha, const double* X, int64_t 
             const unsigned g = (unsigned)std::min<int64_t>((total + 255) / 256, 152 * 32);
             k_gather<float><<<g, 256, 0, st>>>(X + c0, ldx, A->d_perm, n, mc, Xp);
             H2_LAUNCH_CHECK();
+            if ((rc = launch_pack_act(Xp, mc, NL, nullptr, D.leaf_base, D.leaf_kdim, 0, D.xkoff, 0, mc, R, Xcm, es, st)))
+                return rc;
+            marks.mark();
         }
-        // (the lists of pairs also write the split tiles of X (leaves), x̂ and leaf ŷ)
-        if ((!fast || flow) &&
-            (rc = launch_pack_act(Xp, mc, NL, nullptr, D.leaf_base, D.leaf_kdim, 0, D.xkoff, 0, mc, R, Xcm, es, st)))
-            return rc;
-        marks.mark();
         if (flow) {
             // Both transfer passes on the tensor cores.  With A (and the stored
             // couplings) the upward pass shares one launch with the coupling phase
